@@ -120,6 +120,12 @@ void cdet_tune_options_set(int fsc_from_n, int cdet_ctas_per_sm);
 // Launches the fused minors / connected-sum kernel. Returns a cudaError_t.
 int launch_fpm_cdet(const CdetArgs &a, cudaStream_t s);
 
+// Small orders, a few lanes per matrix (cdet_lanes.cu): log2 of the lanes each
+// matrix gets at this order and batch, or -1 where the one-CTA-per-matrix
+// kernel is the faster one; results are the same bits either way.
+int cdet_lanes_log2(int n, int64_t batch, int mode);
+int launch_cdet_lanes(const CdetArgs &a, int lg, cudaStream_t s);
+
 // All principal minors for orders 9..16 (minors only), one warp per matrix;
 // matrices with a small pivot are redone by the fused kernel (fpm_warp.cu).
 constexpr int kWarpMinorsFromN = 9;

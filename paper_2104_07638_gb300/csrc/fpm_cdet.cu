@@ -531,7 +531,7 @@ __device__ __forceinline__ void cdet_item(const CdetArgs &p, int n, const double
     }
     __syncthreads();
     if (p.mode == kModeWeights) {
-        for (int t = tid; t < N; t += blockDim.x) MA[t] = __ldg(ain + t);
+        for (int t = tid; t < N; t += blockDim.x) MA[t] = t ? __ldg(ain + t) : 1.0;  // a[0] is not read
         __syncthreads();
     } else if (given) {
         // the weights from the given minors (one matrix: det^2, or det)
@@ -842,6 +842,10 @@ int ensure_tables() {
 }
 
 int launch_fpm_cdet(const CdetArgs &a, cudaStream_t s) {
+    if (!a.redo_list && !a.pre && !a.anorm_in) {
+        const int lg = cdet_lanes_log2(a.n, a.batch, a.mode);
+        if (lg >= 0) return launch_cdet_lanes(a, lg, s);
+    }
     int err = ensure_tables();
     if (err) return err;
     CdetKernelParams P;

@@ -1,0 +1,75 @@
+"""The size of a batch decides which kernel and how many lanes, warps or CTAs a
+matrix gets, never its result: every row of a large batch equals, bit for bit,
+the same matrix in a call on a few, across the sizes where the routes change;
+sampled rows against the CPU oracle (tolerance 1e-10 times the sum of the
+absolute values of the terms)."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_2104_07638_gb300 import inputs as I
+
+pytestmark = pytest.mark.gpu
+TOL = 1e-10
+
+
+@pytest.fixture(scope="module")
+def apm():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2104_07638_gb300 import apm as m
+    m.lib()
+    m.tune_set(None)
+    m.tune_options_set(0, 0, 0)
+    return m
+
+
+def mixed(n, batch, seed):
+    """Gaussian and Hubbard matrices; among the first ones zero diagonals (a
+    correction at every pivot), equal vertices, the zero matrix, non-finite entries."""
+    rng = np.random.default_rng(seed)
+    A = rng.standard_normal((batch, n, n))
+    A[::2] = I.hubbard_batch(batch, n, seed=seed)[::2]
+    A[1][np.diag_indices(n)] = 0.0
+    A[3] = 0.0
+    A[5, 0, n - 1] = np.inf
+    A[7, n - 1, 0] = np.nan
+    if n > 2:
+        A[2][:, 1] = A[2][:, n - 1]
+        A[2][1] = A[2][n - 1]
+    return A
+
+
+def rows_equal(big, small, idx):
+    for x, y in zip(big, small):
+        x, y = x[idx].cpu().numpy(), y.cpu().numpy()
+        assert np.array_equal(x, y, equal_nan=True)
+
+
+# both sides of every change of route of the lane-group kernel (orders 1..8)
+LANES = [(1, 40), (2, 3000), (3, 40000), (4, 299), (4, 301), (4, 8000), (4, 30001), (5, 457), (5, 3001), (5, 29200),
+         (6, 551), (6, 2000), (6, 8000), (6, 14600), (6, 29190), (7, 951), (7, 3700), (7, 20001), (8, 2001), (8, 4001),
+         (8, 9000)]
+
+
+@pytest.mark.parametrize("n,batch", LANES)
+def test_small_orders(apm, n, batch):
+    A = mixed(n, batch, 8100 + n)
+    B = I.hubbard_batch(batch, n, seed=8200 + n)
+    d, e = torch.as_tensor(A).cuda(), torch.as_tensor(B).cuda()
+    few = torch.as_tensor([0, 1, 2, 3, 5, 7, batch // 2, batch - 2, batch - 1]).cuda()
+    for f in (lambda x, y: apm.cdet_connected(x, return_minors=True, return_status=True),
+              lambda x, y: apm.cdet_connected(x, y, return_minors=True, return_status=True),
+              lambda x, y: apm.cdet_connected(x, single_det=True, return_status=True, piv_threshold=0.5),
+              lambda x, y: apm.all_minors(x, return_status=True)):
+        rows_equal(f(d, e), f(d[few], e[few]), few)
+    w = torch.as_tensor(np.random.default_rng(n).standard_normal((batch, 1 << n))).cuda()
+    w[3, 0] = float("nan")                      # a[0] is not read
+    rows_equal((apm.cdet_from_weights(w),), (apm.cdet_from_weights(w[few]),), few)
+    c, m = apm.cdet_connected(d, return_minors=True)
+    pick = [0, 1, 2, batch - 1]
+    mref, ms = oracle.minors_lu(A[pick]), oracle.minors_scale(A[pick])
+    assert np.all(np.abs(m.cpu().numpy()[pick] - mref) <= TOL * np.maximum(ms, 1e-300))
+    cref, cs = oracle.cdet_recursion(mref * mref), oracle.cdet_scale(ms * ms)
+    assert np.all(np.abs(c.cpu().numpy()[pick] - cref) <= TOL * np.maximum(cs, 1e-300))
