@@ -961,7 +961,12 @@ int launch_cdet_varlen(const CdetArgs &a, const int64_t *a_off, const int *n_arr
     err = launch_order(n_arr, a.batch, n_max, order, ctr, s, fsc_from);
     if (err) return err;
     // the minors of the items of orders >= wfrom, one launch per order from its
-    // first index and count in the sorted list, one warp per matrix
+    // first index and count in the sorted list, the flags zeroed before them
+    // (a small batch's matrices are several warps each, which only set them)
+    if (wfrom) {
+        err = static_cast<int>(cudaMemsetAsync(wflag, 0, static_cast<size_t>(a.batch), s));
+        if (err) return err;
+    }
     for (int m = n_max; wfrom && m >= wfrom && !err; --m)
         err = launch_fpm_warp_route(a.A_up, m, a.batch, a.minors_out ? a.minors_out : a.c_out, a.piv_thr, wflag,
                                     a.status, slots, order, a_off, c_off, ctr + 2 + 2 * m, ctr + 3 + 2 * m, s);

@@ -25,6 +25,13 @@
 // Node i of the lane level carries element e's decision in bit e - L, so lane i
 // writes the minors of the sets (i << L) | X, X within 0 .. L-1, contiguously.
 //
+// Few matrices: a warp is not one matrix then but a run of consecutive leaves
+// of its depth-first part (2^kc runs per matrix, each rebuilding its path from
+// the matrix), and the tail gets shorter (T = 9..12), so that 40 matrices of
+// order 16 are 640 warps of one 12-element tail instead of 40 warps of 16, and
+// one matrix of order 12 is 8 warps of 9-element tails. The tree and its
+// operations do not depend on where the tail begins, so neither changes a bit.
+//
 // Pivot correction (Section II): this kernel shifts nothing. A matrix that
 // meets a pivot with |p| <= thr ||A||max is flagged, and the fused kernel,
 // launched after it on the flagged matrices only, computes them again with
@@ -69,9 +76,10 @@ struct alignas(16) FwWarpSmem {
 };
 static_assert(sizeof(FwWarpSmem) % 16 == 0, "per-warp blocks stay 16-byte aligned");
 
-// stack entries (doubles) for order n: the kept-pivot matrices of depths 1..D-1 (D = n - 12)
-__host__ __device__ constexpr size_t fw_stack_entries(int n) {
-    const int D = n > kFwTail ? n - kFwTail : 0;
+// stack entries (doubles) for order n and a tail of T elements: the kept-pivot
+// matrices of depths 1..D-1 (D = n - T)
+__host__ __device__ constexpr size_t fw_stack_entries(int n, int T) {
+    const int D = n > T ? n - T : 0;
     size_t t = 0;
     for (int d = 1; d < D; ++d) t += static_cast<size_t>(n - d) * (n - d);
     return t;
@@ -211,13 +219,15 @@ __device__ __forceinline__ void fw_tail(double *out, FwWarpSmem &w, int lane, do
     fw_tail_levels<T, 0>(w.bufE, w.bufO, out, w, lane, thrA, fl);
 }
 
-// One matrix of order n (9..16), whole warp: its 2^n minors, each times pre,
-// into out. Returns 1 when a pivot is below thrA or zero (the fused kernel
+// Depth-first leaves t0 <= t < t1 of one matrix of order n (9..16), whole warp
+// (all 2^(n-T) of them, or one run): their minors, each times pre, into out
+// (the matrix's row). Returns 1 when a pivot is below thrA or zero (the fused kernel
 // redoes the matrix) or the input is not finite (the fused kernel then sets the
 // status and NaN).
 template <int T>
 __device__ __forceinline__ int fw_matrix(const double *A, int n, double *out, double thr, double pre,
-                                         const double *anorm, double *stack, FwWarpSmem &w, int lane) {
+                                         const double *anorm, int64_t t0, int64_t t1, double *stack,
+                                         FwWarpSmem &w, int lane) {
     const int D = n - T;
     int fl = 0, nonfin = 0;
     // ||A||max and the finiteness test on the bit patterns of |x| (integer
@@ -243,9 +253,10 @@ __device__ __forceinline__ int fw_matrix(const double *A, int n, double *out, do
         w.pdet[0] = pre;
     }
     __syncwarp();
-    for (int64_t t = 0; t < (int64_t(1) << D); ++t) {
-        // first depth whose decision changed from t-1 to t (element n-1 <-> top bit)
-        const int d0 = t == 0 ? 0 : D - __ffsll(t);
+    for (int64_t t = t0; t < t1; ++t) {
+        // first depth whose decision changed from t-1 to t (element n-1 <-> top
+        // bit); a run's first leaf builds its whole path
+        const int d0 = t == t0 ? 0 : D - __ffsll(t);
         for (int d = d0; d < D; ++d) {
             const int keep = static_cast<int>((t >> (D - 1 - d)) & 1);
             const double *P = w.vp[d];
@@ -297,35 +308,38 @@ __device__ __forceinline__ int fw_matrix(const double *A, int n, double *out, do
     return __any_sync(0xffffffffu, fl);
 }
 
-// Every matrix; b is appended to redo_list (*redo_count entries, zeroed
-// before) where the fused kernel must compute it again. pre
+// Every matrix, 2^kc runs of leaves each; b is appended once to redo_list
+// (*redo_count entries, zeroed before; mark[b] too where kc > 0) where the
+// fused kernel must compute it again, which then writes its status. pre
 // (or NULL for 1): a factor per matrix on all its minors; anorm (or NULL): the
 // scale of the threshold, anorm[b >> anorm_shift], in place of the matrix's own
-// ||A||max (the leaves of a larger matrix take its norm). T = min(n, 12), one
-// instantiation each, so that the register allocation of the largest lane
-// subtree does not burden the others. Shared memory (90 KB per CTA) admits two
-// CTAs per SM, so each thread may use up to 255 registers.
+// ||A||max (the leaves of a larger matrix take its norm). One instantiation per
+// T, so that the register allocation of the largest lane subtree does not
+// burden the others. Shared memory (90 KB per CTA) admits two CTAs per SM, so
+// each thread may use up to 255 registers.
 template <int T>
 __global__ void __launch_bounds__(kFwWarps * 32, 2) fpm_warp_kernel(const double *__restrict__ A, int n,
                                                                   int64_t batch, double *minors, double thr,
                                                                   const double *__restrict__ pre,
                                                                   uint32_t *redo_list, unsigned *redo_count,
-                                                                  uint32_t *status, double *stack_base,
-                                                                  size_t stack_per_warp,
+                                                                  unsigned *mark, uint32_t *status,
+                                                                  double *stack_base, size_t stack_per_warp,
                                                                   const double *__restrict__ anorm,
-                                                                  int anorm_shift) {
+                                                                  int anorm_shift, int kc) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     FwWarpSmem &w = reinterpret_cast<FwWarpSmem *>(smem_raw)[wid];
     const int64_t gw = static_cast<int64_t>(blockIdx.x) * kFwWarps + wid;
     const int64_t nw = static_cast<int64_t>(gridDim.x) * kFwWarps;
     double *stack = stack_base ? stack_base + gw * stack_per_warp : nullptr;
-    const int64_t nn = static_cast<int64_t>(n) * n, N = int64_t(1) << n;
-    for (int64_t b = gw; b < batch; b += nw) {
+    const int64_t nn = static_cast<int64_t>(n) * n, N = int64_t(1) << n, run = int64_t(1) << (n - T - kc);
+    for (int64_t it = gw; it < (batch << kc); it += nw) {
+        const int64_t b = it >> kc, t0 = (it - (b << kc)) * run;
         const int r = fw_matrix<T>(A + b * nn, n, minors + b * N, thr, pre ? pre[b] : 1.0,
-                                   anorm ? anorm + (b >> anorm_shift) : nullptr, stack, w, lane);
+                                   anorm ? anorm + (b >> anorm_shift) : nullptr, t0, t0 + run, stack, w, lane);
         if (lane == 0) {
-            if (r) redo_list[atomicAdd(redo_count, 1u)] = static_cast<uint32_t>(b);
+            if (r && (kc == 0 || atomicExch(mark + b, 1u) == 0u))
+                redo_list[atomicAdd(redo_count, 1u)] = static_cast<uint32_t>(b);
             if (status && !r) status[b] = 0u;
         }
     }
@@ -335,52 +349,67 @@ __global__ void __launch_bounds__(kFwWarps * 32, 2) fpm_warp_kernel(const double
 // them back unless a matrix is flagged): matrix b's minors go to
 // out + b * 2^n, or, with an item list (order != NULL), the items
 // order[*first + i], i < *count, of an uneven batch, matrix A + a_off[b] and
-// minors out + o_off[b]. flag[b] = 1 where the fused kernel must compute the
-// matrix itself (a pivot at or below the threshold, a non-finite entry), else 0
-// with status[b] = 0. Orders above 12 only (tail of 12 elements).
+// minors out + o_off[b]; 2^kc runs of leaves per matrix. flag[b] = 1 where the
+// fused kernel must compute the matrix itself (a pivot at or below the
+// threshold, a non-finite entry) and write its status, else 0 with
+// status[b] = 0; with kc > 0 the flags are zero before. Orders above 12 only.
+template <int T>
 __global__ void __launch_bounds__(kFwWarps * 32, 2) fpm_warp_route_kernel(
     const double *__restrict__ A, int n, int64_t batch, double *out, double thr, uint8_t *flag,
     uint32_t *status, double *stack_base, size_t stack_per_warp, const int *__restrict__ order,
     const int64_t *__restrict__ a_off, const int64_t *__restrict__ o_off, const unsigned *first,
-    const unsigned *count) {
+    const unsigned *count, int kc) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     FwWarpSmem &w = reinterpret_cast<FwWarpSmem *>(smem_raw)[wid];
     const int64_t gw = static_cast<int64_t>(blockIdx.x) * kFwWarps + wid;
     const int64_t nw = static_cast<int64_t>(gridDim.x) * kFwWarps;
     double *stack = stack_base ? stack_base + gw * stack_per_warp : nullptr;
-    const int64_t nn = static_cast<int64_t>(n) * n, N = int64_t(1) << n;
+    const int64_t nn = static_cast<int64_t>(n) * n, N = int64_t(1) << n, run = int64_t(1) << (n - T - kc);
     const int64_t items = order ? static_cast<int64_t>(*count) : batch;
     const int64_t i0 = order ? static_cast<int64_t>(*first) : 0;
-    for (int64_t i = gw; i < items; i += nw) {
+    for (int64_t it = gw; it < (items << kc); it += nw) {
+        const int64_t i = it >> kc, t0 = (it - (i << kc)) * run;
         const int64_t b = order ? order[i0 + i] : i;
         const double *Ab = order ? A + a_off[b] : A + b * nn;
         double *ob = order ? out + o_off[b] : out + b * N;
-        const int r = fw_matrix<kFwTail>(Ab, n, ob, thr, 1.0, nullptr, stack, w, lane);
+        const int r = fw_matrix<T>(Ab, n, ob, thr, 1.0, nullptr, t0, t0 + run, stack, w, lane);
         if (lane == 0) {
-            flag[b] = static_cast<uint8_t>(r);
+            if (kc == 0 || r) flag[b] = static_cast<uint8_t>(r);
             if (status && !r) status[b] = 0u;
         }
     }
 }
 
 using FwKernel = void (*)(const double *, int, int64_t, double *, double, const double *, uint32_t *, unsigned *,
-                         uint32_t *, double *, size_t, const double *, int);
-static FwKernel fw_kernel_for(int n) {
-    switch (n < kFwTail ? n : kFwTail) {
+                         unsigned *, uint32_t *, double *, size_t, const double *, int, int);
+static FwKernel fw_kernel_for(int T) {
+    switch (T) {
         case 9: return fpm_warp_kernel<9>;
         case 10: return fpm_warp_kernel<10>;
         case 11: return fpm_warp_kernel<11>;
         default: return fpm_warp_kernel<12>;
     }
 }
+using FwRouteKernel = void (*)(const double *, int, int64_t, double *, double, uint8_t *, uint32_t *, double *,
+                              size_t, const int *, const int64_t *, const int64_t *, const unsigned *,
+                              const unsigned *, int);
+static FwRouteKernel fw_route_kernel_for(int T) {
+    switch (T) {
+        case 9: return fpm_warp_route_kernel<9>;
+        case 10: return fpm_warp_route_kernel<10>;
+        case 11: return fpm_warp_route_kernel<11>;
+        default: return fpm_warp_route_kernel<12>;
+    }
+}
 
-static int fpm_warp_grid(int n, int64_t batch, int *err) {
+// The warps the chip holds (CTAs of kFwWarps) of one of the kernels above.
+template <class K>
+static int fw_resident(K kern, int *err) {
     int dev = 0, sms = 0, per_sm = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const size_t smem = kFwWarps * sizeof(FwWarpSmem);
-    const FwKernel kern = fw_kernel_for(n);
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
     if (e == cudaSuccess)
@@ -390,25 +419,45 @@ static int fpm_warp_grid(int n, int64_t batch, int *err) {
         return 0;
     }
     *err = 0;
-    const int64_t need = (batch + kFwWarps - 1) / kFwWarps;
-    int64_t g = static_cast<int64_t>(sms) * per_sm;
-    if (need < g) g = need;
-    return static_cast<int>(g < 1 ? 1 : g);
+    return sms * per_sm * kFwWarps;
 }
 
-// Workspace: per resident warp the depth-first stack, the redo list (a
-// counter, then up to one entry per matrix), and for n > 12 the fused kernel's
-// global scratch (its redo launch).
+// Tail size and runs per matrix (log2) for a batch: the longest tail whose
+// leaves, one warp each, give every SM kFwFill warps (else the shortest), and
+// as few runs as leave no warp waiting for another's last matrix (4 rounds of
+// the 8 resident warps per SM; a run's path costs 3 % of a 12-element leaf).
+constexpr int kFwFill = 4, kFwRounds = 4;
+struct FwShape {
+    int T, kc;
+};
+static FwShape fw_shape(int n, int64_t batch) {
+    const int64_t want = int64_t(152) * kFwFill, most = int64_t(152) * 2 * kFwWarps * kFwRounds;
+    FwShape s = {n < kFwTail ? n : kFwTail, 0};
+    while (s.T > 9 && (batch << (n - s.T)) < want) --s.T;
+    while (s.kc < n - s.T && (batch << s.kc) < most) ++s.kc;
+    return s;
+}
+// Warps that a batch of up to `batch` matrices can occupy, whatever its shape
+// (does not shrink as the batch grows, so scratch for a batch serves a smaller one).
+static int64_t fw_most_warps(int n, int64_t batch, int64_t resident) {
+    const int64_t cap = batch >= resident ? resident : batch << (n - 9);
+    const int64_t w = cap < resident ? cap : resident;
+    return (w + kFwWarps - 1) / kFwWarps * kFwWarps;
+}
+
+// Workspace: per resident warp the depth-first stack (sized for the shortest
+// tail), the redo list (a counter, a mark per matrix, then up to one entry per
+// matrix), and for n > 12 the fused kernel's global scratch (its redo launch).
 struct FwPlan {
     size_t stack, list, fused, total;
 };
-static int fw_plan(int n, int64_t batch, FwPlan *p, int *grid) {
+static int fw_plan(int n, int64_t batch, FwPlan *p, int *resident) {
     int err = 0;
-    *grid = fpm_warp_grid(n, batch, &err);
+    *resident = fw_resident(fw_kernel_for(kFwTail), &err);
     if (err) return err;
     auto al = [](size_t x) { return (x + 255) & ~static_cast<size_t>(255); };
-    p->stack = al(static_cast<size_t>(*grid) * kFwWarps * fw_stack_entries(n) * sizeof(double));
-    p->list = 256 + al(static_cast<size_t>(batch) * sizeof(uint32_t));
+    p->stack = al(static_cast<size_t>(fw_most_warps(n, batch, *resident)) * fw_stack_entries(n, 9) * sizeof(double));
+    p->list = 256 + 2 * al(static_cast<size_t>(batch) * sizeof(uint32_t));
     p->fused = 0;
     if (n > cdet_smem_max_n(false)) {
         const int g = cdet_grid(n, batch, false, false, &err);
@@ -423,8 +472,8 @@ size_t fpm_warp_workspace_bytes(int n, int64_t batch, int *err) {
     *err = 0;
     if (batch == 0) return 0;
     FwPlan p;
-    int grid = 0;
-    *err = fw_plan(n, batch, &p, &grid);
+    int resident = 0;
+    *err = fw_plan(n, batch, &p, &resident);
     return *err ? 0 : p.total;
 }
 
@@ -432,20 +481,34 @@ int launch_fpm_warp(const double *A, int n, int64_t batch, double *minors, doubl
                     uint32_t *status, void *workspace, cudaStream_t s, const double *pre,
                     const double *anorm_in, int anorm_shift) {
     FwPlan plan;
-    int grid = 0;
-    int err = fw_plan(n, batch, &plan, &grid);
+    int resident = 0;
+    int err = fw_plan(n, batch, &plan, &resident);
     if (err) return err;
+    const FwShape sh = fw_shape(n, batch);
+    const FwKernel kern = fw_kernel_for(sh.T);
+    if (sh.T != kFwTail) {
+        // a shorter tail needs no fewer resident warps: the stacks are sized for
+        // the longest tail's, and its grid stays within them
+        int err2 = 0;
+        const int r = fw_resident(kern, &err2);
+        if (err2) return err2;
+        if (r < resident) resident = r;
+    }
+    const int64_t items = batch << sh.kc, need = (items + kFwWarps - 1) / kFwWarps;
+    const int grid = static_cast<int>(need * kFwWarps < resident ? need : resident / kFwWarps);
     const size_t smem = kFwWarps * sizeof(FwWarpSmem);
-    const size_t per = fw_stack_entries(n);
+    const size_t per = fw_stack_entries(n, sh.T);
     char *ws = static_cast<char *>(workspace);
     double *stack = per ? reinterpret_cast<double *>(ws) : nullptr;
     unsigned *count = reinterpret_cast<unsigned *>(ws + plan.stack);
-    uint32_t *list = reinterpret_cast<uint32_t *>(ws + plan.stack + 256);
+    unsigned *mark = reinterpret_cast<unsigned *>(ws + plan.stack + 256);
+    uint32_t *list = reinterpret_cast<uint32_t *>(ws + plan.stack + 256 + (plan.list - 256) / 2);
     double *fused = plan.fused ? reinterpret_cast<double *>(ws + plan.stack + plan.list) : nullptr;
-    err = static_cast<int>(cudaMemsetAsync(count, 0, sizeof(unsigned), s));
+    err = static_cast<int>(cudaMemsetAsync(
+        count, 0, sh.kc ? 256 + static_cast<size_t>(batch) * sizeof(unsigned) : sizeof(unsigned), s));
     if (err) return err;
-    fw_kernel_for(n)<<<grid, kFwWarps * 32, smem, s>>>(A, n, batch, minors, thr, pre, list, count, status, stack,
-                                                        per, anorm_in, anorm_shift);
+    kern<<<grid, kFwWarps * 32, smem, s>>>(A, n, batch, minors, thr, pre, list, count, mark, status, stack, per,
+                                           anorm_in, anorm_shift, sh.kc);
     err = static_cast<int>(cudaGetLastError());
     if (err) return err;
     // the flagged matrices again, by the fused kernel with the pivot correction
@@ -468,33 +531,12 @@ int launch_fpm_warp(const double *A, int n, int64_t batch, double *minors, doubl
     return launch_fpm_cdet(a, s);
 }
 
-static int fw_route_grid(int64_t batch, int *err) {
-    int dev = 0, sms = 0, per_sm = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const size_t smem = kFwWarps * sizeof(FwWarpSmem);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(fpm_warp_route_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 static_cast<int>(smem));
-    if (e == cudaSuccess)
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fpm_warp_route_kernel, kFwWarps * 32, smem);
-    if (e != cudaSuccess || per_sm < 1) {
-        *err = e != cudaSuccess ? static_cast<int>(e) : static_cast<int>(cudaErrorInvalidConfiguration);
-        return 0;
-    }
-    *err = 0;
-    const int64_t need = (batch + kFwWarps - 1) / kFwWarps;
-    int64_t g = static_cast<int64_t>(sms) * per_sm;
-    if (need < g) g = need;
-    return static_cast<int>(g < 1 ? 1 : g);
-}
-
 size_t fpm_warp_route_stack_bytes(int n, int64_t batch, int *err) {
     *err = 0;
     if (batch == 0 || n <= kFwTail) return 0;
-    const int grid = fw_route_grid(batch, err);
+    const int resident = fw_resident(fw_route_kernel_for(kFwTail), err);
     if (*err) return 0;
-    return static_cast<size_t>(grid) * kFwWarps * fw_stack_entries(n) * sizeof(double);
+    return static_cast<size_t>(fw_most_warps(n, batch, resident)) * fw_stack_entries(n, 9) * sizeof(double);
 }
 
 int launch_fpm_warp_route(const double *A, int n, int64_t batch, double *out, double thr, uint8_t *flag,
@@ -502,10 +544,26 @@ int launch_fpm_warp_route(const double *A, int n, int64_t batch, double *out, do
                           const int64_t *o_off, const unsigned *first, const unsigned *count, cudaStream_t s) {
     if (n <= kFwTail || n > kFwMaxN) return static_cast<int>(cudaErrorInvalidValue);
     int err = 0;
-    const int grid = fw_route_grid(batch, &err);
+    // an uneven batch's orders have an unknown share of it each: runs of one
+    // leaf there (they cost a path each, about 3 % of the leaf)
+    FwShape sh = order ? FwShape{kFwTail, batch <= 8192 ? n - kFwTail : 0} : fw_shape(n, batch);
+    const FwRouteKernel kern = fw_route_kernel_for(sh.T);
+    int resident = fw_resident(fw_route_kernel_for(kFwTail), &err);
     if (err) return err;
-    fpm_warp_route_kernel<<<grid, kFwWarps * 32, kFwWarps * sizeof(FwWarpSmem), s>>>(
-        A, n, batch, out, thr, flag, status, stack, fw_stack_entries(n), order, a_off, o_off, first, count);
+    if (sh.T != kFwTail) {
+        const int r = fw_resident(kern, &err);
+        if (err) return err;
+        if (r < resident) resident = r;
+    }
+    if (sh.kc && !order) {
+        err = static_cast<int>(cudaMemsetAsync(flag, 0, static_cast<size_t>(batch), s));
+        if (err) return err;
+    }
+    const int64_t need = ((batch << sh.kc) + kFwWarps - 1) / kFwWarps;
+    const int grid = static_cast<int>(need * kFwWarps < resident ? need : resident / kFwWarps);
+    kern<<<grid, kFwWarps * 32, kFwWarps * sizeof(FwWarpSmem), s>>>(A, n, batch, out, thr, flag, status, stack,
+                                                                    fw_stack_entries(n, sh.T), order, a_off, o_off,
+                                                                    first, count, sh.kc);
     return static_cast<int>(cudaGetLastError());
 }
 

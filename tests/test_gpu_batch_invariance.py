@@ -73,3 +73,18 @@ def test_small_orders(apm, n, batch):
     assert np.all(np.abs(m.cpu().numpy()[pick] - mref) <= TOL * np.maximum(ms, 1e-300))
     cref, cs = oracle.cdet_recursion(mref * mref), oracle.cdet_scale(ms * ms)
     assert np.all(np.abs(c.cpu().numpy()[pick] - cref) <= TOL * np.maximum(cs, 1e-300))
+
+
+# the warp-per-run minors kernel: tails of 9..12 elements, one run or several per matrix
+@pytest.mark.parametrize("n,batch", [(9, 700), (10, 305), (11, 160), (11, 700), (12, 80), (12, 160), (12, 5000),
+                                     (13, 39), (13, 5000), (14, 155), (15, 77), (16, 45)])
+def test_minors_runs(apm, n, batch):
+    d = torch.as_tensor(mixed(n, batch, 8300 + n)).cuda()
+    few = torch.as_tensor([0, 1, 2, 3, 5, 7, batch // 2, batch - 2, batch - 1]).cuda()
+    big, st = apm.all_minors(d, return_status=True)
+    one = [apm.all_minors(d[i:i + 1].clone(), return_status=True) for i in few.tolist()]
+    rows_equal((big, st), (torch.cat([m for m, _ in one]), torch.cat([s for _, s in one])), few)
+    rows_equal((big, st), apm.all_minors(d[few], return_status=True), few)
+    if n > 12:      # the connected sums' minors take the same route
+        rows_equal((big[few], st[few]), apm.cdet_connected(d[few], return_minors=True, return_status=True)[1:],
+                   list(range(9)))
