@@ -413,22 +413,26 @@ static int lanes_launch(const LanesParams &P, cudaStream_t s) {
 static int lanes_most(int n) { return n < 4 ? 2 : n == 4 ? 3 : 4; }
 
 // Lanes per matrix (log2) at order n and this batch, or -1 for the
-// one-CTA-per-matrix kernel. Both sides measured on a GB300, us per call with
-// the host side of about 11 us in it (CTA kernel | this one, cdet mode):
-//   n = 4: 801 | 29 at 65536, 11 | 11 at 300      n = 5: 999 | 72, 11 | 13 at 300
-//   n = 6: 1220 | 148 at 65536, 31 | 21 at 1000, 13 | 19 at 300
-//   n = 7: 1581 | 355 at 65536, 37 | 35 at 1000   n = 8: 2210 | 918 at 65536,
-//   109 | 88 at 3000, 50 | 65 at 1000 (weights alone 60 | 70 at 3000, 142 | 109
-//   at 8000; minors alone 58 | 54 at 3000).
-// One round of resident CTAs (3 per SM) is the faster while it lasts, the lane
-// groups from `from` matrices on. As few lanes per matrix as fill the chip (6
-// warps per SM) waste the fewest; below `least` lanes a warp's arrays leave too
-// few warps per SM (n = 8, 65536: 918 us with 8 lanes, 1046 with 4, 1442 with 2).
+// one-CTA-per-matrix kernel (of 64 or 128 threads here). Both sides measured on
+// a GB300, us per call with the host side of about 11 us in it (CTA | this):
+//   minors and sums: n = 5: 1200 matrices 14 | 15, 2000 19 | 17, 65536 410 | 72
+//     n = 6: 1200 15 | 21, 2000 22 | 23, 3000 30 | 25, 65536 498 | 148
+//     n = 7: 4096 51 | 62, 6000 74 | 64, 65536 706 | 355
+//     n = 8: 4096 74 | 97, 16384 267 | 278, 65536 1048 | 918
+//   minors: n = 6: 3500 25 | 18, 65536 375 | 68;  n = 7: 8000 60 | 35, 65536 433 | 140
+//     n = 8: 8000 70 | 83, 12000 98 | 88, 65536 514 | 323
+//   sums from weights: n = 6: 4096 17 | 21, 9000 25 | 23, 65536 146 | 78
+//     n = 7: 16384 74 | 72, 65536 282 | 205;  n = 8: 65536 537 | 595
+// (256-thread CTAs took 1220, 1581 and 2210 us on 65536 of order 6, 7 and 8.)
+// As few lanes per matrix as fill the chip (6 warps per SM) waste the fewest;
+// below `least` lanes a warp's arrays leave too few warps per SM (n = 8, 65536:
+// 918 us with 8 lanes, 1046 with 4, 1442 with 2).
 int cdet_lanes_log2(int n, int64_t batch, int mode) {
     if (n > kLanesMaxN) return -1;
-    static const int from[3][kLanesMaxN + 1] = {{0, 0, 0, 0, 300, 456, 700, 1300, 2800},   // minors
-                                                {0, 0, 0, 0, 300, 456, 550, 950, 2000},    // minors and sums
-                                                {0, 0, 0, 0, 300, 456, 700, 1500, 4000}};  // sums
+    static const int from[3][kLanesMaxN + 1] = {
+        {0, 0, 0, 0, 456, 2500, 2500, 5000, 10000},       // minors
+        {0, 0, 0, 0, 456, 1500, 2200, 5500, 20000},       // minors and sums
+        {0, 0, 0, 0, 456, 4000, 8000, 16000, 1 << 30}};   // sums from weights
     if (batch < from[mode][n]) return -1;
     const int least = mode == kModeMinors ? (n > 6 ? n - 6 : 0) : (n > 5 ? n - 5 : n == 5 ? 1 : 0);
     int lg = least;

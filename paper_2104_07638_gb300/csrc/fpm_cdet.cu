@@ -783,6 +783,28 @@ void cdet_tune_set(const unsigned long long *table) {
     for (int n = 0; n <= 16; ++n) g_tuned[n] = table ? table[n] : 0ull;
 }
 
+// Threads of a CTA (one matrix) at order n <= 12. A small order's phases have
+// too little to do for 256 threads, and every barrier of its tree and its layers
+// stops the whole CTA: more, smaller CTAs on an SM (its registers hold 768
+// threads of this kernel in any case) fill each other's waits. Wide CTAs are the
+// faster only while one round of them holds the batch. Measured, us per call
+// (256 | 128 | 64 threads; host side of 11 us included):
+//   n = 8:  300 matrices 19 | 19 | 21, 1200 51 | 39 | 26, 65536 2224 | 1173 | 1048
+//   n = 9:  300 24 | 25 | 33, 777 47 | 37 | 41, 1200 68 | 61 | 47, 16384 755 | 555 | 543
+//   n = 10: 456 46 | 49 | 62, 777 86 | 76 | 82, 1200 125 | 119 | 99, 2000 197 | 170 | 179,
+//           16384 1447 | 1258 | 1255
+//   n = 11: 456 103 | 111 | 146, 2000 459 | 443 | 525, 16384 3497 | 3303 | 3436
+//   n = 12: 456 256 | 270 | 353, 16384 8864 | 9299 | 12462
+static int cdet_threads(int n, int64_t batch) {
+    if (n > 11) return kCdetThreads;
+    const int64_t round = 3 * 152;  // resident CTAs of 256 threads
+    if (n <= 8) return batch <= 2 * round ? 128 : 64;
+    if (batch <= round) return kCdetThreads;
+    if (n == 9) return batch <= 2 * round ? 128 : 64;
+    if (n == 10) return batch > 2 * round && batch <= 11 * 152 ? 64 : 128;
+    return 128;
+}
+
 int cdet_grid(int n, int64_t batch, bool two_mats, bool smem_arrays, int *err) {
     int dev = 0, sms = 0, per_sm = 0;
     cudaError_t e = cudaGetDevice(&dev);
@@ -794,7 +816,7 @@ int cdet_grid(int n, int64_t batch, bool two_mats, bool smem_arrays, int *err) {
                                      static_cast<int>(smem));
             if (e == cudaSuccess)
                 e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fpm_cdet_kernel<true>,
-                                                                  kCdetThreads, smem);
+                                                                  cdet_threads(n, batch), smem);
         } else {
             e = cudaFuncSetAttribute(fpm_cdet_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      static_cast<int>(smem));
@@ -866,7 +888,7 @@ int launch_fpm_cdet(const CdetArgs &a, cudaStream_t s) {
         if (err) return err;
     }
     if (smem_arrays)
-        fpm_cdet_kernel<true><<<grid, kCdetThreads, smem, s>>>(P);
+        fpm_cdet_kernel<true><<<grid, cdet_threads(a.n, a.batch), smem, s>>>(P);
     else
         fpm_cdet_kernel<false><<<grid, kCdetThreads, smem, s>>>(P);
     err = static_cast<int>(cudaGetLastError());
@@ -880,25 +902,34 @@ int launch_fpm_cdet(const CdetArgs &a, cudaStream_t s) {
 // ---------------------------------------------------------------------------
 
 constexpr int kVarlenSmemMaxN = 12;
+// Threads of a CTA and the order its shared arrays hold, from the largest order
+// present: as for a fixed order, a batch of small orders only takes small CTAs,
+// and the arrays of its largest order rather than of order 12 (4096 walkers of
+// orders 4..9: 201 -> 156 us).
+static int varlen_threads(int n_max) { return n_max <= 9 ? 64 : n_max <= 11 ? 128 : kCdetThreads; }
+static int varlen_smem_n(int n_max) { return n_max < kVarlenSmemMaxN ? n_max : kVarlenSmemMaxN; }
 
 static size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
 
-int cdet_varlen_grid(bool two_mats, int *err) {
+static int cdet_varlen_grid(int n_max, bool two_mats, int *err) {
     int dev = 0, sms = 0, per_sm = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const size_t smem = cdet_smem_bytes(kVarlenSmemMaxN, two_mats, true);
+    const size_t smem = cdet_smem_bytes(varlen_smem_n(n_max), two_mats, true);
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(fpm_cdet_varlen_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 static_cast<int>(smem));
+                                 static_cast<int>(cdet_smem_bytes(kVarlenSmemMaxN, true, true)));
     if (e == cudaSuccess)
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fpm_cdet_varlen_kernel, kCdetThreads, smem);
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fpm_cdet_varlen_kernel, varlen_threads(n_max),
+                                                          smem);
     if (e != cudaSuccess || per_sm < 1) {
         *err = e != cudaSuccess ? static_cast<int>(e) : static_cast<int>(cudaErrorInvalidConfiguration);
         return 0;
     }
     *err = 0;
-    if (g_varlen_ctas > 0 && g_varlen_ctas < per_sm) per_sm = g_varlen_ctas;
+    // the tuned limit counts CTAs of kCdetThreads threads
+    const int most = g_varlen_ctas * (kCdetThreads / varlen_threads(n_max));
+    if (most > 0 && most < per_sm) per_sm = most;
     return sms * per_sm;
 }
 
@@ -915,7 +946,7 @@ static int warp_route_from(int n_max, bool two_mats) {
 size_t cdet_varlen_workspace(int n_max, int64_t batch, bool two_mats, int *err) {
     size_t bytes = 256 + align256(static_cast<size_t>(batch) * sizeof(int));
     if (n_max > kVarlenSmemMaxN) {
-        const int grid = cdet_varlen_grid(two_mats, err);
+        const int grid = cdet_varlen_grid(n_max, two_mats, err);
         if (*err) return 0;
         size_t slots = static_cast<size_t>(grid) * slot_doubles(n_max) * sizeof(double);
         if (n_max >= g_fsc_from_n) {  // the same region then holds the ranked arrays
@@ -947,7 +978,7 @@ int launch_cdet_varlen(const CdetArgs &a, const int64_t *a_off, const int *n_arr
     int err = ensure_tables();
     if (err) return err;
     const bool two = a.two_mats != 0;
-    const int grid = cdet_varlen_grid(two, &err);
+    const int grid = cdet_varlen_grid(n_max, two, &err);
     if (err) return err;
     unsigned char *ws = static_cast<unsigned char *>(workspace);
     unsigned *ctr = reinterpret_cast<unsigned *>(ws);
@@ -987,7 +1018,8 @@ int launch_cdet_varlen(const CdetArgs &a, const int64_t *a_off, const int *n_arr
     const bool fsc = a.mode == kModeCdet && n_max >= fsc_from;
     V.a.fsc_from_n = fsc ? fsc_from : 0;
     const int64_t g = a.batch < grid ? a.batch : grid;
-    fpm_cdet_varlen_kernel<<<static_cast<int>(g), kCdetThreads, cdet_smem_bytes(kVarlenSmemMaxN, two, true), s>>>(V);
+    fpm_cdet_varlen_kernel<<<static_cast<int>(g), varlen_threads(n_max),
+                             cdet_smem_bytes(varlen_smem_n(n_max), two, true), s>>>(V);
     err = static_cast<int>(cudaGetLastError());
     if (err || !fsc) return err;
     // the items of the orders >= fsc_from (the longest-first prefix), one launch

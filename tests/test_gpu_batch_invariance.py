@@ -47,10 +47,10 @@ def rows_equal(big, small, idx):
         assert np.array_equal(x, y, equal_nan=True)
 
 
-# both sides of every change of route of the lane-group kernel (orders 1..8)
-LANES = [(1, 40), (2, 3000), (3, 40000), (4, 299), (4, 301), (4, 8000), (4, 30001), (5, 457), (5, 3001), (5, 29200),
-         (6, 551), (6, 2000), (6, 8000), (6, 14600), (6, 29190), (7, 951), (7, 3700), (7, 20001), (8, 2001), (8, 4001),
-         (8, 9000)]
+# both sides of every change of route and of CTA width at orders 1..11
+LANES = [(1, 40), (2, 3000), (3, 40000), (4, 455), (4, 457), (4, 8000), (4, 30001), (5, 913), (5, 1501), (5, 3001),
+         (5, 29200), (6, 2201), (6, 8001), (6, 14600), (6, 29190), (7, 4999), (7, 5501), (7, 20001), (8, 913),
+         (8, 10001), (8, 20001), (9, 457), (9, 913), (10, 500), (10, 1000), (10, 1673), (11, 460)]
 
 
 @pytest.mark.parametrize("n,batch", LANES)
