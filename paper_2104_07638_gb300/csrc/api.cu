@@ -43,9 +43,8 @@ apm_status_t cdet_common(apm::CdetArgs &a, void *workspace, size_t workspace_byt
     const bool smem_arrays = a.n <= apm::cdet_smem_max_n(two);
     if (!smem_arrays) {
         int err = 0;
-        const int grid = apm::cdet_grid(a.n, a.batch, two, false, &err);
+        size_t need = apm::cdet_scratch_bytes(a.n, a.batch, two, &err);
         if (err) return cuda_fail(err);
-        size_t need = static_cast<size_t>(grid) * apm::cdet_slot_doubles(a.n) * sizeof(double);
         if (a.mode == apm::kModeCdet && a.n >= apm::cdet_fsc_from_n()) {
             const size_t f = apm::fsc_workspace_bytes(a.n, a.batch, &err);
             if (err) return cuda_fail(err);
@@ -546,9 +545,8 @@ apm_status_t apm_workspace_size(int op, int n_max, int64_t batch, int two_mats, 
             const bool two = op == APM_OP_CDET && two_mats;
             if (n_max <= apm::cdet_smem_max_n(two) || batch == 0) return APM_OK;
             int err = 0;
-            const int grid = apm::cdet_grid(n_max, batch, two, false, &err);
+            *bytes = apm::cdet_scratch_bytes(n_max, batch, two, &err);
             if (err) return cuda_fail(err);
-            *bytes = static_cast<size_t>(grid) * apm::cdet_slot_doubles(n_max) * sizeof(double);
             if (op == APM_OP_CDET && n_max >= apm::cdet_fsc_from_n()) {  // then the ranked arrays
                 const size_t f = apm::fsc_workspace_bytes(n_max, batch, &err);
                 if (err) return cuda_fail(err);
@@ -580,9 +578,8 @@ apm_status_t apm_workspace_size(int op, int n_max, int64_t batch, int two_mats, 
             size_t need = apm::xnor_workspace_bytes(n_max, batch, &err);
             if (err) return cuda_fail(err);
             if (op == APM_OP_NAMBU_CDET && n_max > apm::cdet_smem_max_n(false)) {
-                const int grid = apm::cdet_grid(n_max, batch, false, false, &err);
+                const size_t rec = apm::cdet_scratch_bytes(n_max, batch, false, &err);
                 if (err) return cuda_fail(err);
-                const size_t rec = static_cast<size_t>(grid) * apm::cdet_slot_doubles(n_max) * sizeof(double);
                 if (rec > need) need = rec;
             }
             *bytes = need;
@@ -597,9 +594,8 @@ apm_status_t apm_workspace_size(int op, int n_max, int64_t batch, int two_mats, 
             size_t need = apm::nand_workspace_bytes(n_max, batch, &err);
             if (err) return cuda_fail(err);
             if (op == APM_OP_TWO_TYPE_CDET && n_max > apm::cdet_smem_max_n(false)) {
-                const int grid = apm::cdet_grid(n_max, batch, false, false, &err);
+                const size_t rec = apm::cdet_scratch_bytes(n_max, batch, false, &err);
                 if (err) return cuda_fail(err);
-                const size_t rec = static_cast<size_t>(grid) * apm::cdet_slot_doubles(n_max) * sizeof(double);
                 if (rec > need) need = rec;
             }
             *bytes = need;

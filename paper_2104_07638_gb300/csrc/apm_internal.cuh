@@ -61,6 +61,10 @@ size_t cdet_smem_bytes(int n, bool two_mats, bool smem_arrays);
 // Grid size used for a fixed-order launch (also sizes the workspace).
 int cdet_grid(int n, int64_t batch, bool two_mats, bool smem_arrays, int *err);
 
+// Bytes of global scratch of a fixed-order connected-sum launch above order 12:
+// the CTAs' slots, and rows for the terms of few matrices' blocks.
+size_t cdet_scratch_bytes(int n, int64_t batch, bool two_mats, int *err);
+
 // Doubles of global scratch one CTA uses when the arrays do not fit on chip.
 size_t cdet_slot_doubles(int n);
 
@@ -102,6 +106,10 @@ struct CdetArgs {
     // wflag[b] != 0 (b: the item's batch index)
     uint8_t *wflag;
     int warp_from_n;
+    // fixed-order launch above order 12, one CTA per matrix (batch <= grid): stop
+    // at the weights, left in the CTA's slot of gscratch, and skip the matrices
+    // whose minors the warp-per-matrix kernel has left
+    int weights_only;
 };
 
 // Orders whose connected sums apm_cdet_connected and its uneven-batch form take

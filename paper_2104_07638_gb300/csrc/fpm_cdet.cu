@@ -576,6 +576,7 @@ __device__ __forceinline__ void cdet_item(const CdetArgs &p, int n, const double
         }
         __syncthreads();
     }
+    if (p.weights_only) return;
     if (in_smem) {
         cdet_layers(MA, MA, MC, n, gsel);
         if (tid == 0) bulk_store(co, MC, N * 8u);
@@ -608,6 +609,7 @@ __global__ void __launch_bounds__(kCdetThreads, 3) fpm_cdet_kernel(const CdetKer
     double *MU = MC + NC;
     const int64_t mat = static_cast<int64_t>(n) * n;
     auto item = [&](int64_t b) {
+        if (p.weights_only && p.wflag && !p.wflag[b]) return;
         cdet_item(p, n, p.A_up ? p.A_up + b * mat : nullptr, p.A_dn ? p.A_dn + b * mat : nullptr,
                   p.a_in ? p.a_in + b * N : nullptr,
                   p.minors_out ? p.minors_out + b * (p.two_mats ? 2 * N : N) : nullptr,
@@ -623,6 +625,236 @@ __global__ void __launch_bounds__(kCdetThreads, 3) fpm_cdet_kernel(const CdetKer
         for (int64_t b = blockIdx.x; b < p.batch; b += gridDim.x) item(b);
     }
     if (threadIdx.x == 0) bulk_wait_all();
+}
+
+// ---------------------------------------------------------------------------
+// Orders 13..15, few matrices: the blocked recursion of cdet_blocked with a
+// matrix's blocks on many CTAs
+// ---------------------------------------------------------------------------
+// One CTA per matrix leaves 24 matrices on 24 of 152 SMs, 1.5 ms each at order
+// 14. The blocks S_H of one popcount depend only on those of smaller popcounts,
+// so the recursion runs level by level over the whole batch, two launches per
+// level: the off-diagonal contributions of every block (its masks S_L dealt out
+// to `parts` CTAs, each walking all T_H), left in the block's own place in the
+// output row, then the diagonal recursion of every block. Each mask's terms are
+// added in the order of cdet_blocked: the results are the same bits.
+
+// Weights of the matrices the warp-per-matrix kernel has not flagged, from
+// their minors (rows of 2^n doubles) into the slots' first 2^n doubles.
+__global__ void __launch_bounds__(256) cdet_square_kernel(const double *__restrict__ minors,
+                                                          const uint8_t *__restrict__ flag, double *slots,
+                                                          size_t slot, int n, int64_t batch, int single) {
+    const int64_t pairs = int64_t(1) << (n - 1);
+    const int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x, b = i >> (n - 1);
+    if (b >= batch || flag[b]) return;
+    const int64_t t = 2 * (i & (pairs - 1));
+    double2 m = *reinterpret_cast<const double2 *>(minors + (b << n) + t);
+    if (!single) m = make_double2(m.x * m.x, m.y * m.y);
+    *reinterpret_cast<double2 *>(slots + b * slot + t) = m;
+}
+
+// sum over UH within H, in descending order, of c[j u UL u UH] a[S' less UL and
+// UH], four terms a step, their operands loaded a step ahead: with few warps on
+// an SM the chain of FMAs is what a set costs, not the loads before each.
+__device__ __forceinline__ double cdet_walk(const double *c, const double *a, int j, int Sp, int UL, int H) {
+    const int e0 = H & (-H), H1 = H ^ e0, e1 = H1 & (-H1), H2 = H1 ^ e1;
+    double acc = 0.0;
+    if (H1 == 0) {  // one or two terms
+        if (H) acc = fma(c[j | UL | H], a[Sp ^ (UL | H)], acc);
+        return fma(c[j | UL], a[Sp ^ UL], acc);
+    }
+    int X = H2, cu = j | UL | H2, au = Sp ^ (UL | H2);
+    double c3 = c[cu | e1 | e0], a3 = a[au ^ (e1 | e0)], c2 = c[cu | e1], a2 = a[au ^ e1];
+    double c1 = c[cu | e0], a1 = a[au ^ e0], c0 = c[cu], a0 = a[au];
+    while (X) {
+        X = (X - 1) & H2;
+        cu = j | UL | X;
+        au = Sp ^ (UL | X);
+        const double d3 = c[cu | e1 | e0], b3 = a[au ^ (e1 | e0)], d2 = c[cu | e1], b2 = a[au ^ e1];
+        const double d1 = c[cu | e0], b1 = a[au ^ e0], d0 = c[cu], b0 = a[au];
+        acc = fma(c0, a0, fma(c1, a1, fma(c2, a2, fma(c3, a3, acc))));
+        c3 = d3, a3 = b3, c2 = d2, a2 = b2, c1 = d1, a1 = b1, c0 = d0, a0 = b0;
+    }
+    return fma(c0, a0, fma(c1, a1, fma(c2, a2, fma(c3, a3, acc))));
+}
+
+// first index of popcount class k in g_popmasks, from the constant bank
+__device__ __forceinline__ int cdet_popoff(int k) {
+    int o = 0;
+    for (int i = 0; i < k; ++i) o += c_binom[16][i];
+    return o;
+}
+// the masks of kBlkB elements by (popcount, value) into pop, one independent
+// load per mask
+__device__ __forceinline__ void cdet_block_masks(uint16_t *pop) {
+    for (int t = threadIdx.x; t < (1 << kBlkB); t += blockDim.x) {
+        int rest = t, src = t, k = 0;
+        for (; k < kBlkB && rest >= c_binom[kBlkB][k]; ++k) {
+            rest -= c_binom[kBlkB][k];
+            src += c_binom[16][k] - c_binom[kBlkB][k];
+        }
+        pop[t] = g_popmasks[src];
+    }
+}
+
+// one group step of a layer: lane's set S, its lanes' shares UL, the rest H
+struct CdetSet {
+    int S, j, Sp, UL, H, gl;
+};
+__device__ __forceinline__ CdetSet cdet_set(int S, int r, int lane) {
+    CdetSet q;
+    q.S = S;
+    q.j = S & (-S);
+    q.Sp = S ^ q.j;
+    q.gl = lane & ((1 << r) - 1);
+    q.UL = 0;
+    q.H = q.Sp;
+    for (int i = 0; i < r; ++i) {
+        const int bt = q.H & (-q.H);
+        q.H ^= bt;
+        if ((q.gl >> i) & 1) q.UL |= bt;
+    }
+    return q;
+}
+
+// Off-diagonal contributions of the blocks with |S_H| = k. Task = (matrix,
+// block, part); the warps of a block's parts take the set groups of all layers
+// in turn, and the next T_H's operand blocks arrive while the current ones are
+// used; the sums go to the block's place in the rows of c. With `rows` (few
+// matrices) a task is one T_H alone instead, (matrix, block, T_H, part), and its
+// terms go to a row of their own, which the diagonal launch adds in T_H's order.
+__global__ void __launch_bounds__(kCdetThreads, 3) cdet_split_conv_kernel(const double *__restrict__ a, size_t astride,
+                                                                       double *c, int n, int64_t batch, int k,
+                                                                       int lparts, double *rows,
+                                                                       unsigned long long gsel) {
+    constexpr int b = kBlkB, NB = 1 << kBlkB;
+    __shared__ __align__(16) double cb[2][NB], ab[2][NB], acc[NB];
+    __shared__ uint16_t pop[NB];
+    const int tid = threadIdx.x, T = blockDim.x, lane = tid & 31;
+    const int h = n - b, nblk = c_binom[h][k], pk = cdet_popoff(k);
+    const int parts = 1 << lparts, W = (T >> 5) << lparts;
+    cdet_block_masks(pop);
+    const int nth = rows ? (1 << k) - 1 : 1;
+    for (int64_t task = blockIdx.x; task < (batch * nblk * nth) << lparts; task += gridDim.x) {
+        const int part = static_cast<int>(task & (parts - 1));
+        const int64_t row = task >> lparts, mb = row / nth, mat = mb / nblk;
+        const int SH = g_popmasks[pk + static_cast<int>(mb - mat * nblk)], jH = SH & (-SH);
+        const double *am = a + mat * astride;
+        double *cm = c + (mat << n);
+        const int wg = part * (T >> 5) + (tid >> 5);
+        // f(first lane's set) for the sets of this warp, in every layer
+        auto sets = [&](auto &&f) {
+            int done = 0, off = 1;
+            for (int kk = 1; kk <= b; ++kk) {
+                const int cnt = c_binom[b][kk];
+                const int r = static_cast<int>((gsel >> (3 * kk)) & 7ull), spw = 32 >> r;
+                const int steps = (cnt + spw - 1) >> (5 - r);
+                int s0 = wg - done % W;
+                if (s0 < 0) s0 += W;
+                for (int s = s0; s < steps; s += W) {
+                    const int G = s * spw + (lane >> r);
+                    f(pop[off + (G < cnt ? G : cnt - 1)], r, G < cnt);
+                }
+                done += steps;
+                off += cnt;
+            }
+        };
+        auto fetch = [&](int TH, int q) {
+            const double *cT = cm + (static_cast<size_t>(TH) << b), *aR = am + (static_cast<size_t>(SH ^ TH) << b);
+            for (int t = tid; t < NB / 2; t += T) {
+                cp_async16(cb[q] + 2 * t, cT + 2 * t);
+                cp_async16(ab[q] + 2 * t, aR + 2 * t);
+            }
+        };
+        int T0 = (SH - 1) & SH;
+        if (rows)
+            for (int i = static_cast<int>(row - mb * nth); i > 0; --i) T0 = (T0 - 1) & SH;
+        fetch(T0, 0);
+        for (int t = tid; t < NB; t += T) acc[t] = 0.0;
+        int q = 0;
+        for (int TH = T0;; TH = (TH - 1) & SH, q ^= 1) {
+            cp_async_wait_all();
+            __syncthreads();
+            if (TH && !rows) fetch((TH - 1) & SH, q ^ 1);
+            sets([&](int S, int r, bool act) {
+                const CdetSet g = cdet_set(S, r, lane);
+                double sum = cdet_walk(cb[q], ab[q], g.j, g.Sp, g.UL, g.H);
+                for (int o = (1 << r) >> 1; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+                if (act && g.gl == 0) acc[S] += sum;
+            });
+            if (rows) break;
+            if (tid == 0 && part == 0 && (TH & jH)) acc[0] = fma(cb[q][0], ab[q][0], acc[0]);
+            if (TH == 0) break;
+        }
+        __syncthreads();
+        double *out = rows ? rows + (row << b) : cm + (static_cast<size_t>(SH) << b);
+        sets([&](int S, int r, bool act) {
+            if (act && (lane & ((1 << r) - 1)) == 0) out[S] = acc[S];
+        });
+        if (tid == 0 && part == 0) out[0] = acc[0];
+        __syncthreads();
+    }
+}
+
+// The diagonal recursion of the blocks with |S_H| = k, one CTA each; rows: the
+// T_H's terms, one row each, or NULL where the block's place in c holds their sum.
+__global__ void __launch_bounds__(kCdetThreads, 3) cdet_split_diag_kernel(const double *__restrict__ a, size_t astride,
+                                                                       double *c, int n, int64_t batch, int k,
+                                                                       const double *__restrict__ rows,
+                                                                       unsigned long long gsel) {
+    constexpr int b = kBlkB, NB = 1 << kBlkB;
+    __shared__ __align__(16) double cs[NB], as[NB], a0[NB];
+    __shared__ uint16_t pop[NB];
+    const int tid = threadIdx.x, T = blockDim.x, lane = tid & 31, warp = tid >> 5, nw = T >> 5;
+    const int nblk = c_binom[n - b][k], pk = cdet_popoff(k);
+    cdet_block_masks(pop);
+    for (int64_t task = blockIdx.x; task < batch * nblk; task += gridDim.x) {
+        const int64_t mat = task / nblk;
+        const int SH = g_popmasks[pk + static_cast<int>(task - mat * nblk)];
+        const double *am = a + mat * astride;
+        double *out = c + (mat << n) + (static_cast<size_t>(SH) << b);
+        for (int t = tid; t < NB; t += T) {
+            a0[t] = t ? am[t] : 1.0;
+            double sum = 0.0;
+            if (SH && !rows) {
+                sum = out[t];
+            } else if (SH && t) {
+                const double *pr = rows + ((task * ((1 << k) - 1)) << b) + t;
+                for (int i = 0; i < (1 << k) - 1; i += 8) {  // the loads of eight rows in flight
+                    double v[8];
+#pragma unroll
+                    for (int e = 0; e < 8; ++e)
+                        if (i + e < (1 << k) - 1) v[e] = pr[static_cast<size_t>(i + e) << b];
+#pragma unroll
+                    for (int e = 0; e < 8; ++e)
+                        if (i + e < (1 << k) - 1) sum += v[e];
+                }
+            } else if (SH) {
+                const double *cm = c + (mat << n);
+                for (int TH = (SH - 1) & SH; TH; TH = (TH - 1) & SH)
+                    if (TH & SH & -SH)
+                        sum = fma(cm[static_cast<size_t>(TH) << b], am[static_cast<size_t>(SH ^ TH) << b], sum);
+            }
+            const double v = am[(static_cast<size_t>(SH) << b) + t] - sum;
+            as[t] = v;
+            cs[t] = (t & (t - 1)) ? 0.0 : v;  // sets of one element are their own sums
+        }
+        __syncthreads();
+        for (int kk = 2, off = 1 + b; kk <= b; off += c_binom[b][kk], ++kk) {
+            const int cnt = c_binom[b][kk];
+            const int r = static_cast<int>((gsel >> (3 * kk)) & 7ull), spw = 32 >> r;
+            for (int base = warp * spw; base < cnt; base += nw * spw) {
+                const int G = base + (lane >> r);
+                const CdetSet g = cdet_set(pop[off + (G < cnt ? G : cnt - 1)], r, lane);
+                double acc = cdet_walk(cs, a0, g.j, g.Sp, g.UL, g.H);
+                for (int o = (1 << r) >> 1; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+                if (G < cnt && g.gl == 0) cs[g.S] = as[g.S] - acc;
+            }
+            __syncthreads();
+        }
+        for (int t = tid; t < NB; t += T) out[t] = (t == 0) ? (SH ? as[0] : 0.0) : cs[t];
+        __syncthreads();
+    }
 }
 
 // Uneven batch: items taken longest-first from `order` through a global
@@ -835,6 +1067,23 @@ int cdet_grid(int n, int64_t batch, bool two_mats, bool smem_arrays, int *err) {
     return static_cast<int>(g < 1 ? 1 : g);
 }
 
+// Rows (of 2^kBlkB doubles) that the levels' terms may take, at most 64 MB; does
+// not shrink as the batch grows.
+constexpr int64_t kSplitMaxRows = 8192;
+static int64_t cdet_split_rows(int n, int64_t batch) {
+    const int h = n - kBlkB;
+    if (h < 3 || h > 6) return 0;
+    const int most = h == 3 ? 9 : h == 4 ? 28 : h == 5 ? 75 : 225;  // max over k of C(h, k) (2^k - 1)
+    return batch < kSplitMaxRows / most ? batch * most : kSplitMaxRows;
+}
+
+size_t cdet_scratch_bytes(int n, int64_t batch, bool two_mats, int *err) {
+    const int grid = cdet_grid(n, batch, two_mats, false, err);
+    if (*err) return 0;
+    return (static_cast<size_t>(grid) * slot_doubles(n) +
+            (static_cast<size_t>(cdet_split_rows(n, batch)) << kBlkB)) * sizeof(double);
+}
+
 int ensure_tables() {
     static int done_mask = 0;  // bit per device id < 32
     int dev = 0;
@@ -863,6 +1112,38 @@ int ensure_tables() {
     return 0;
 }
 
+// The recursion above order 12 with every matrix's blocks on many CTAs: a (rows
+// astride doubles apart) -> c; rows: cdet_split_rows rows of scratch.
+static int launch_cdet_split(const double *a, size_t astride, double *c, int n, int64_t batch, double *rows,
+                             unsigned long long gsel_b, cudaStream_t s) {
+    const int h = n - kBlkB;
+    const int64_t round = 3 * 152;  // resident CTAs of either kernel
+    for (int k = 0, nblk = 1; k <= h; nblk = nblk * (h - k) / (k + 1), ++k) {
+        const int64_t tasks = batch * nblk, pairs = tasks * ((1 << k) - 1);
+        double *rk = pairs <= cdet_split_rows(n, batch) ? rows : nullptr;
+        if (k) {
+            int lparts = 0;
+            const int64_t each = rk ? pairs : tasks;
+            while (lparts < (rk ? 2 : 3) && (each << lparts) < (rk ? 152 : 2 * round)) ++lparts;
+            const int64_t g = each << lparts;
+            cdet_split_conv_kernel<<<static_cast<int>(g < 8 * round ? g : 8 * round), kCdetThreads, 0, s>>>(
+                a, astride, c, n, batch, k, lparts, rk, gsel_b);
+        }
+        cdet_split_diag_kernel<<<static_cast<int>(tasks < 8 * round ? tasks : 8 * round), kCdetThreads, 0, s>>>(
+            a, astride, c, n, batch, k, rk, gsel_b);
+    }
+    return static_cast<int>(cudaGetLastError());
+}
+
+// Whether a launch (or the last, partial round of one) of this many matrices
+// above order 12 goes level by level over many CTAs rather than with one CTA
+// per matrix, whose time hardly depends on how many of a round's 456 there are.
+// Measured, us per call (one CTA per matrix | level by level):
+//   n = 13: 1 matrix 500 | 152, 24 501 | 184, 152 512 | 373, 300 607 | 640
+//   n = 14: 1 1428 | 198, 24 1435 | 288, 152 1456 | 929, 300 1727 | 1629, 456 2336 | 2410
+//   n = 15: 1 4195 | 249, 24 4215 | 580, 152 4267 | 2615, 456 6757 | 6756
+static bool cdet_split_pays(int n, int64_t batch) { return batch <= (n == 13 ? 260 : n == 14 ? 350 : 456); }
+
 int launch_fpm_cdet(const CdetArgs &a, cudaStream_t s) {
     if (!a.redo_list && !a.pre && !a.anorm_in) {
         const int lg = cdet_lanes_log2(a.n, a.batch, a.mode);
@@ -886,6 +1167,40 @@ int launch_fpm_cdet(const CdetArgs &a, cudaStream_t s) {
         err = launch_fpm_warp_route(a.A_up, a.n, a.batch, a.minors_out ? a.minors_out : a.c_out, a.piv_thr,
                                     a.wflag, a.status, a.gscratch, nullptr, nullptr, nullptr, nullptr, nullptr, s);
         if (err) return err;
+    }
+    // (weights that the sums overwrite in place have to be copied to the slots)
+    const bool in_place = a.mode == kModeWeights && a.a_in < a.c_out + (a.batch << a.n) &&
+                          a.c_out < a.a_in + (a.batch << a.n);
+    if (!smem_arrays && !fsc && a.mode != kModeMinors && !in_place) {
+        // full rounds of one CTA per matrix, then the rest
+        const int full = cdet_grid(a.n, INT64_MAX, a.two_mats != 0, false, &err);
+        if (err) return err;
+        const int64_t part = a.batch % full, rest = cdet_split_pays(a.n, part) ? part : 0, b0 = a.batch - rest;
+        if (b0) {
+            P.a.batch = b0;
+            fpm_cdet_kernel<false><<<grid, kCdetThreads, smem, s>>>(P);
+            err = static_cast<int>(cudaGetLastError());
+        }
+        if (err || !rest) return err;
+        const size_t slot = slot_doubles(a.n), row = size_t(1) << a.n, mats = a.two_mats ? 2 : 1;
+        double *rows = a.gscratch + grid * slot, *c = a.c_out + b0 * row;
+        if (a.mode == kModeWeights) return launch_cdet_split(a.a_in + b0 * row, row, c, a.n, rest, rows, P.gsel_b, s);
+        P.a.batch = rest;
+        P.a.weights_only = 1;
+        P.a.A_up += b0 * a.n * a.n;
+        if (a.A_dn) P.a.A_dn += b0 * a.n * a.n;
+        P.a.c_out = c;
+        if (a.minors_out) P.a.minors_out += b0 * row * mats;
+        if (a.status) P.a.status += b0;
+        if (a.wflag) {
+            P.a.wflag += b0;
+            cdet_square_kernel<<<static_cast<int>(((rest << (a.n - 1)) + 255) / 256), 256, 0, s>>>(
+                a.minors_out ? P.a.minors_out : c, P.a.wflag, a.gscratch, slot, a.n, rest, a.single_det);
+        }
+        fpm_cdet_kernel<false><<<static_cast<int>(rest), kCdetThreads, smem, s>>>(P);
+        err = static_cast<int>(cudaGetLastError());
+        if (err) return err;
+        return launch_cdet_split(a.gscratch, slot, c, a.n, rest, rows, P.gsel_b, s);
     }
     if (smem_arrays)
         fpm_cdet_kernel<true><<<grid, cdet_threads(a.n, a.batch), smem, s>>>(P);

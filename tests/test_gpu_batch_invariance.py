@@ -88,3 +88,33 @@ def test_minors_runs(apm, n, batch):
     if n > 12:      # the connected sums' minors take the same route
         rows_equal((big[few], st[few]), apm.cdet_connected(d[few], return_minors=True, return_status=True)[1:],
                    list(range(9)))
+
+
+# above order 12: one CTA per matrix, or the blocks of a matrix on many CTAs with
+# the terms in rows of their own (few matrices) or summed in place, and the last
+# partial round of a larger batch
+@pytest.mark.parametrize("n,batch", [(13, 261), (13, 470), (14, 351), (14, 300), (15, 120), (15, 11)])
+def test_blocked_orders(apm, n, batch):
+    d = torch.as_tensor(mixed(n, batch, 8400 + n)).cuda()
+    e = torch.as_tensor(I.hubbard_batch(batch, n, seed=8500 + n)).cuda()
+    few = torch.as_tensor([0, 1, 2, 5, batch // 2, batch - 1]).cuda()
+    for f in (lambda x, y: apm.cdet_connected(x, return_minors=True, return_status=True),
+              lambda x, y: apm.cdet_connected(x, single_det=True, return_status=True),
+              lambda x, y: apm.cdet_connected(x, y, return_minors=True, return_status=True)):
+        rows_equal(f(d, e), f(d[few], e[few]), few)
+
+
+@pytest.mark.parametrize("n,batch", [(13, 300), (14, 360), (16, 40)])
+def test_blocked_orders_from_weights(apm, n, batch):
+    w = torch.as_tensor(np.random.default_rng(n).standard_normal((batch, 1 << n))).cuda()
+    few = torch.as_tensor([0, 3, batch // 2, batch - 1]).cuda()
+    w[3, 0] = float("nan")                      # a[0] is not read
+    c = apm.cdet_from_weights(w)
+    rows_equal((c,), (apm.cdet_from_weights(w[few]),), few)
+    # in place, as the one-CTA-per-matrix route takes it
+    z = w[few].clone()
+    nb = apm.workspace_size(apm.OP_CDET_FROM_WEIGHTS, n, 4)
+    ws = torch.empty(nb, dtype=torch.uint8, device="cuda")
+    apm._check(apm.lib().apm_cdet_from_weights(apm._ptr(z), n, 4, apm._ptr(z), apm._ptr(ws), nb, apm._stream(z)),
+               "apm_cdet_from_weights")
+    rows_equal((c,), (z,), few)
