@@ -14,7 +14,8 @@
 // The logarithm comes from k Z_k = sum_{j=1..k} j L_j Z_{k-j}: with M_k = k L_k,
 //     M_k = k Z_k - sum_{m=1..k-1} Z_m M_{k-m}.
 //
-// One CTA (256 threads) per matrix, persistent over the batch; the ranked
+// One CTA (256 threads) per matrix, persistent over the batch (the last round of
+// fewer rows than CTAs: a CTA per tile and a launch per pass); the ranked
 // arrays R[k][X] (k = 1..n) are transformed in tiles of 512 masks in shared
 // memory. n <= 9 is one tile (init, zeta, logarithm, Mobius, read-out, all in
 // shared memory). Above, the low 9 elements are handled inside a tile and the
@@ -281,155 +282,185 @@ __device__ __forceinline__ void fsc_log(double *T, int nx, int n, const uint16_t
     }
 }
 
+// Orders of the tile's masks by popcount, one table per number of bits.
+struct FscOrders {
+    uint16_t order[kFscTile];                                // tile entries by (popcount, value)
+    double inv[kFscMaxN + 1];                                // 1/k
+    uint8_t ordh[1 << (kFscMaxN - kFscTileBits - 1)];        // masks of h - 1 bits
+    uint8_t ordh2[1 << (kFscMaxN - kFscTileBits - 2)];       // masks of h - 2 bits
+    uint8_t ord8[kFscTile / 2];                              // masks of 8 bits
+    uint8_t ord7[kFscTile / 4];                              // masks of 7 bits
+    uint8_t binom[kFscTileBits + 1][kFscTileBits + 1];
+};
+
+// position of t among the masks of `bits` bits by (popcount, value): the classes
+// of fewer elements first, then t's rank in its own (combinatorial number system)
+__device__ __forceinline__ int fsc_position(const FscOrders &s, int t, int bits) {
+    const int p = __popc(t);
+    int pos = 0;
+    for (int c = 0; c < p; ++c) pos += s.binom[bits][c];
+    int i = 0;
+    for (int r = t; r; r &= r - 1) pos += s.binom[__ffs(r) - 1][++i];
+    return pos;
+}
+
+__device__ __forceinline__ void fsc_orders(FscOrders &s, int n) {
+    const int tid = threadIdx.x;
+    if (tid <= kFscMaxN) s.inv[tid] = tid ? 1.0 / tid : 0.0;
+    if (tid < (kFscTileBits + 1) * (kFscTileBits + 1))
+        s.binom[tid / (kFscTileBits + 1)][tid % (kFscTileBits + 1)] =
+            static_cast<uint8_t>(binom_small(tid / (kFscTileBits + 1), tid % (kFscTileBits + 1)));
+    __syncthreads();
+    for (int t = tid; t < kFscTile; t += kFscThreads) s.order[fsc_position(s, t, kFscTileBits)] = static_cast<uint16_t>(t);
+    for (int t = tid; t < kFscTile / 2; t += kFscThreads)
+        s.ord8[fsc_position(s, t, kFscTileBits - 1)] = static_cast<uint8_t>(t);
+    for (int t = tid; t < kFscTile / 4; t += kFscThreads)
+        s.ord7[fsc_position(s, t, kFscTileBits - 2)] = static_cast<uint8_t>(t);
+    const int hb = n > kFscTileBits ? n - kFscTileBits - 1 : 0;  // bits of the high part minus one
+    for (int t = tid; t < (1 << hb); t += kFscThreads) s.ordh[fsc_position(s, t, hb)] = static_cast<uint8_t>(t);
+    const int hb2 = n > kFscTileBits + 1 ? n - kFscTileBits - 2 : 0;  // bits of the high part minus two
+    for (int t = tid; t < (1 << hb2); t += kFscThreads) s.ordh2[fsc_position(s, t, hb2)] = static_cast<uint8_t>(t);
+    __syncthreads();
+}
+
+// pass A, one high pattern XH: partial zeta over the low elements
+__device__ __forceinline__ void fsc_pass_a(double *T, const FscOrders &s, const double *ab, double *R, int n, int XH) {
+    const int tid = threadIdx.x, N = 1 << n;
+    const int p = __popc(XH), k0 = p > 1 ? p : 1, k1 = p + kFscTileBits < n ? p + kFscTileBits : n;
+    const int nr = k1 - k0 + 1;
+    const size_t base = static_cast<size_t>(XH) << kFscTileBits;
+    for (int q = tid; q < nr * kFscTile; q += kFscThreads) {
+        const int r = q >> kFscTileBits, x = q & (kFscTile - 1);
+        if (__popc(x) + p == k0 + r)
+            cp_async8(T + q, ab + base + x);
+        else
+            T[q] = 0.0;
+    }
+    cp_async_wait_all();
+    __syncthreads();
+    fsc_transform_low(T, nr, k0 - p, false, s.ord8, s.ord7);
+    for (int q = tid; q < n * kFscTile; q += kFscThreads) {
+        const int k = (q >> kFscTileBits) + 1, x = q & (kFscTile - 1);
+        R[static_cast<size_t>(k - 1) * N + base + x] = k >= k0 && k <= k1 ? T[(k - k0) * kFscTile + x] : 0.0;
+    }
+    __syncthreads();
+}
+
+// pass B, one group g of low patterns: zeta over the high elements, logarithm,
+// Mobius over the high elements
+__device__ __forceinline__ void fsc_pass_b(double *T, const FscOrders &s, double *R, int n, int g) {
+    const int tid = threadIdx.x, N = 1 << n, lg = 2 * kFscTileBits - n;
+    // pairs of entries (lg >= 1: j and j + 1 are adjacent in R as in T)
+    for (int q2 = tid; q2 < n * kFscTile / 2; q2 += kFscThreads) {
+        const int q = 2 * q2, r = q >> kFscTileBits, t = q & (kFscTile - 1);
+        const int XH = t >> lg, j = t & ((1 << lg) - 1);
+        cp_async16(T + q, R + static_cast<size_t>(r) * N + (static_cast<size_t>(XH) << kFscTileBits) + (g << lg) + j);
+    }
+    cp_async_wait_all();
+    __syncthreads();
+    fsc_transform_high(T, lg, n, false, s.ordh, s.ordh2);
+    fsc_log(T, kFscTile, n, s.order, __popc(g));
+    __syncthreads();
+    fsc_transform_high(T, lg, n, true, s.ordh, s.ordh2);
+    for (int q = tid; q < n * kFscTile; q += kFscThreads) {
+        const int r = q >> kFscTileBits, t = q & (kFscTile - 1);
+        const int XH = t >> lg, j = t & ((1 << lg) - 1);
+        R[static_cast<size_t>(r) * N + (static_cast<size_t>(XH) << kFscTileBits) + (g << lg) + j] = T[q];
+    }
+    __syncthreads();
+}
+
+// pass C, one high pattern: Mobius over the low elements and the read-out
+// c[X] = L_|X|(X)
+__device__ __forceinline__ void fsc_pass_c(double *T, const FscOrders &s, const double *R, double *cb, int n, int XH) {
+    const int tid = threadIdx.x, N = 1 << n;
+    const int p = __popc(XH), k0 = p > 1 ? p : 1, k1 = p + kFscTileBits < n ? p + kFscTileBits : n;
+    const int nr = k1 - k0 + 1;
+    const size_t base = static_cast<size_t>(XH) << kFscTileBits;
+    for (int q2 = tid; q2 < nr * kFscTile / 2; q2 += kFscThreads) {
+        const int q = 2 * q2, r = q >> kFscTileBits, x = q & (kFscTile - 1);
+        cp_async16(T + q, R + static_cast<size_t>(k0 + r - 1) * N + base + x);
+    }
+    cp_async_wait_all();
+    __syncthreads();
+    fsc_transform_low(T, nr, k0 - p, true, s.ord8, s.ord7);
+    for (int x = tid; x < kFscTile; x += kFscThreads)
+        cb[base + x] = (XH | x) ? T[(__popc(x) + p - k0) * kFscTile + x] * s.inv[__popc(x) + p] : 0.0;
+    __syncthreads();
+}
+
 // Rows: a + b 2^n -> c + b 2^n for b < batch, or, with `order`, in place on the
 // rows c + c_off[order[*first + i]] for i < *count (a may equal c: every row is
 // read in pass A before pass C writes it).
-__global__ void __launch_bounds__(kFscThreads, 3) fsc_kernel(const double *a, int n, int64_t batch, double *c,
-                                                              double *ws, const int *order, const int64_t *c_off,
-                                                              const unsigned *first, const unsigned *count) {
+struct FscRows {
+    const double *a;
+    double *c;
+    const int *order;
+    const int64_t *c_off;
+    const unsigned *first, *count;
+    int64_t batch;
+    int full;  // rows of one round: a last, partial one is left to fsc_pass_kernel (1: none)
+    __device__ __forceinline__ int64_t items() const { return order ? static_cast<int64_t>(*count) : batch; }
+    __device__ __forceinline__ double *out(int64_t i, int n) const {
+        return order ? c + c_off[order[static_cast<int64_t>(*first) + i]] : c + (i << n);
+    }
+    __device__ __forceinline__ const double *in(int64_t i, int n) const { return order ? out(i, n) : a + (i << n); }
+};
+
+__global__ void __launch_bounds__(kFscThreads, 3) fsc_kernel(const FscRows rows, int n, double *ws) {
     extern __shared__ __align__(16) double T[];
-    __shared__ uint16_t s_order[kFscTile];  // tile entries by (popcount, value)
-    __shared__ double s_inv[kFscMaxN + 1];  // 1/k
-    __shared__ uint8_t s_ordh[1 << (kFscMaxN - kFscTileBits - 1)];  // masks of h - 1 bits by popcount
-    __shared__ uint8_t s_ordh2[1 << (kFscMaxN - kFscTileBits - 2)];  // masks of h - 2 bits by popcount
-    __shared__ uint8_t s_ord8[kFscTile / 2];                        // masks of 8 bits by popcount
-    __shared__ uint8_t s_ord7[kFscTile / 4];                        // masks of 7 bits by popcount
+    __shared__ FscOrders s;
     const int tid = threadIdx.x;
     const int N = 1 << n;
-    if (tid <= kFscMaxN) s_inv[tid] = tid ? 1.0 / tid : 0.0;
-    for (int t = tid; t < kFscTile; t += kFscThreads) {
-        // position of t: the classes of fewer elements first, then the rank of t
-        // among the masks of its popcount (combinatorial number system)
-        const int p = __popc(t);
-        int pos = 0;
-        for (int c = 0; c < p; ++c) pos += binom_small(kFscTileBits, c);
-        int i = 0;
-        for (int r = t; r; r &= r - 1) pos += binom_small(__ffs(r) - 1, ++i);
-        s_order[pos] = static_cast<uint16_t>(t);
-    }
-    for (int t = tid; t < kFscTile / 2; t += kFscThreads) {
-        const int p = __popc(t);
-        int pos = 0;
-        for (int c = 0; c < p; ++c) pos += binom_small(kFscTileBits - 1, c);
-        int i = 0;
-        for (int r = t; r; r &= r - 1) pos += binom_small(__ffs(r) - 1, ++i);
-        s_ord8[pos] = static_cast<uint8_t>(t);
-    }
-    for (int t = tid; t < kFscTile / 4; t += kFscThreads) {
-        const int p = __popc(t);
-        int pos = 0;
-        for (int c = 0; c < p; ++c) pos += binom_small(kFscTileBits - 2, c);
-        int i = 0;
-        for (int r = t; r; r &= r - 1) pos += binom_small(__ffs(r) - 1, ++i);
-        s_ord7[pos] = static_cast<uint8_t>(t);
-    }
-    const int hb = n > kFscTileBits ? n - kFscTileBits - 1 : 0;  // bits of the high part minus one
-    for (int t = tid; t < (1 << hb); t += kFscThreads) {
-        const int p = __popc(t);
-        int pos = 0;
-        for (int c = 0; c < p; ++c) pos += binom_small(hb, c);
-        int i = 0;
-        for (int r = t; r; r &= r - 1) pos += binom_small(__ffs(r) - 1, ++i);
-        s_ordh[pos] = static_cast<uint8_t>(t);
-    }
-    const int hb2 = n > kFscTileBits + 1 ? n - kFscTileBits - 2 : 0;  // bits of the high part minus two
-    for (int t = tid; t < (1 << hb2); t += kFscThreads) {
-        const int p = __popc(t);
-        int pos = 0;
-        for (int c = 0; c < p; ++c) pos += binom_small(hb2, c);
-        int i = 0;
-        for (int r = t; r; r &= r - 1) pos += binom_small(__ffs(r) - 1, ++i);
-        s_ordh2[pos] = static_cast<uint8_t>(t);
-    }
-    __syncthreads();
-    const int64_t items = order ? static_cast<int64_t>(*count) : batch;
-    const int64_t i0 = order ? static_cast<int64_t>(*first) : 0;
-    auto row_in = [&](int64_t i) { return order ? c + c_off[order[i0 + i]] : a + i * N; };
-    auto row_out = [&](int64_t i) { return order ? c + c_off[order[i0 + i]] : c + i * N; };
+    const int64_t items = rows.items() / rows.full * rows.full;
+    if (blockIdx.x >= items) return;
+    fsc_orders(s, n);
     if (n <= kFscTileBits) {
         for (int64_t b = blockIdx.x; b < items; b += gridDim.x) {
-            const double *ab = row_in(b);
+            const double *ab = rows.in(b, n);
             for (int q = tid; q < n * N; q += kFscThreads) {
                 const int r = q >> n, x = q & (N - 1);
                 T[r * kFscTile + x] = __popc(x) == r + 1 ? ab[x] : 0.0;
             }
             __syncthreads();
-            fsc_butterfly_low(T, n, n, 1, false, s_ord8);
+            fsc_butterfly_low(T, n, n, 1, false, s.ord8);
             fsc_log(T, N, n, nullptr, 0);
             __syncthreads();
-            fsc_butterfly_low(T, n, n, 1, true, s_ord8);
-            double *cb = row_out(b);
+            fsc_butterfly_low(T, n, n, 1, true, s.ord8);
+            double *cb = rows.out(b, n);
             for (int x = tid; x < N; x += kFscThreads)
-                cb[x] = x ? T[(__popc(x) - 1) * kFscTile + x] * s_inv[__popc(x)] : 0.0;
+                cb[x] = x ? T[(__popc(x) - 1) * kFscTile + x] * s.inv[__popc(x)] : 0.0;
             __syncthreads();
         }
         return;
     }
-    const int h = n - kFscTileBits, NH = 1 << h, lg = kFscTileBits - h;  // G = 2^lg low patterns per group
-    double *R = ws + static_cast<size_t>(blockIdx.x) * n * N;           // [n][N]
+    const int NH = 1 << (n - kFscTileBits);
+    double *R = ws + static_cast<size_t>(blockIdx.x) * n * N;  // [n][N]
     for (int64_t b = blockIdx.x; b < items; b += gridDim.x) {
-        const double *ab = row_in(b);
-        // pass A: partial zeta over the low elements
-        for (int XH = 0; XH < NH; ++XH) {
-            const int p = __popc(XH), k0 = p > 1 ? p : 1, k1 = p + kFscTileBits < n ? p + kFscTileBits : n;
-            const int nr = k1 - k0 + 1;
-            const size_t base = static_cast<size_t>(XH) << kFscTileBits;
-            for (int q = tid; q < nr * kFscTile; q += kFscThreads) {
-                const int r = q >> kFscTileBits, x = q & (kFscTile - 1);
-                if (__popc(x) + p == k0 + r)
-                    cp_async8(T + q, ab + base + x);
-                else
-                    T[q] = 0.0;
-            }
-            cp_async_wait_all();
-            __syncthreads();
-            fsc_transform_low(T, nr, k0 - p, false, s_ord8, s_ord7);
-            for (int q = tid; q < n * kFscTile; q += kFscThreads) {
-                const int k = (q >> kFscTileBits) + 1, x = q & (kFscTile - 1);
-                R[static_cast<size_t>(k - 1) * N + base + x] =
-                    k >= k0 && k <= k1 ? T[(k - k0) * kFscTile + x] : 0.0;
-            }
-            __syncthreads();
-        }
-        // pass B: zeta over the high elements, logarithm, Mobius over the high elements
-        for (int g = 0; g < NH; ++g) {
-            // pairs of entries (lg >= 1: j and j + 1 are adjacent in R as in T)
-            for (int q2 = tid; q2 < n * kFscTile / 2; q2 += kFscThreads) {
-                const int q = 2 * q2, r = q >> kFscTileBits, t = q & (kFscTile - 1);
-                const int XH = t >> lg, j = t & ((1 << lg) - 1);
-                cp_async16(T + q, R + static_cast<size_t>(r) * N + (static_cast<size_t>(XH) << kFscTileBits) +
-                                      (g << lg) + j);
-            }
-            cp_async_wait_all();
-            __syncthreads();
-            fsc_transform_high(T, lg, n, false, s_ordh, s_ordh2);
-            fsc_log(T, kFscTile, n, s_order, __popc(g));
-            __syncthreads();
-            fsc_transform_high(T, lg, n, true, s_ordh, s_ordh2);
-            for (int q = tid; q < n * kFscTile; q += kFscThreads) {
-                const int r = q >> kFscTileBits, t = q & (kFscTile - 1);
-                const int XH = t >> lg, j = t & ((1 << lg) - 1);
-                R[static_cast<size_t>(r) * N + (static_cast<size_t>(XH) << kFscTileBits) + (g << lg) + j] = T[q];
-            }
-            __syncthreads();
-        }
-        // pass C: Mobius over the low elements and the read-out c[X] = L_|X|(X)
-        double *cb = row_out(b);
-        for (int XH = 0; XH < NH; ++XH) {
-            const int p = __popc(XH), k0 = p > 1 ? p : 1, k1 = p + kFscTileBits < n ? p + kFscTileBits : n;
-            const int nr = k1 - k0 + 1;
-            const size_t base = static_cast<size_t>(XH) << kFscTileBits;
-            for (int q2 = tid; q2 < nr * kFscTile / 2; q2 += kFscThreads) {
-                const int q = 2 * q2, r = q >> kFscTileBits, x = q & (kFscTile - 1);
-                cp_async16(T + q, R + static_cast<size_t>(k0 + r - 1) * N + base + x);
-            }
-            cp_async_wait_all();
-            __syncthreads();
-            fsc_transform_low(T, nr, k0 - p, true, s_ord8, s_ord7);
-            for (int x = tid; x < kFscTile; x += kFscThreads)
-                cb[base + x] = (XH | x) ? T[(__popc(x) + p - k0) * kFscTile + x] * s_inv[__popc(x) + p] : 0.0;
-            __syncthreads();
-        }
+        const double *ab = rows.in(b, n);
+        for (int XH = 0; XH < NH; ++XH) fsc_pass_a(T, s, ab, R, n, XH);
+        for (int g = 0; g < NH; ++g) fsc_pass_b(T, s, R, n, g);
+        double *cb = rows.out(b, n);
+        for (int XH = 0; XH < NH; ++XH) fsc_pass_c(T, s, R, cb, n, XH);
+    }
+}
+
+// One pass of the rows of the last, partial round: a CTA per tile, so that a few
+// rows fill the chip (n > 9; same tiles, same additions as fsc_kernel).
+template <int PASS>
+__global__ void __launch_bounds__(kFscThreads, 3) fsc_pass_kernel(const FscRows rows, int n, double *ws) {
+    extern __shared__ __align__(16) double T[];
+    __shared__ FscOrders s;
+    const int64_t items = rows.items(), i0 = items / rows.full * rows.full;
+    const int h = n - kFscTileBits, tiles = static_cast<int>(items - i0) << h;  // less than a round's
+    if (static_cast<int>(blockIdx.x) >= tiles) return;
+    fsc_orders(s, n);
+    for (int t = blockIdx.x; t < tiles; t += gridDim.x) {
+        const int i = t >> h, x = t - (i << h);
+        double *R = ws + (static_cast<size_t>(i) * n << n);
+        if (PASS == 0) fsc_pass_a(T, s, rows.in(i0 + i, n), R, n, x);
+        if (PASS == 1) fsc_pass_b(T, s, R, n, x);
+        if (PASS == 2) fsc_pass_c(T, s, R, rows.out(i0 + i, n), n, x);
     }
 }
 
@@ -462,23 +493,47 @@ size_t fsc_workspace_bytes(int n, int64_t batch, int *err) {
     return static_cast<size_t>(grid) * n * (static_cast<size_t>(1) << n) * sizeof(double);
 }
 
-int launch_fsc(const double *a, int n, int64_t batch, double *c, void *workspace, cudaStream_t s) {
+// Rounds of one CTA per row (as many rows as CTAs are resident), and the last,
+// partial one by tiles, where that pays: a row's CTA takes the same 6.9 ms at
+// order 16 whether it has the chip to itself or not. us per call, one CTA per
+// row | by tiles: n = 16: 1 row 6882 | 85, 40 6985 | 1405, 300 10783 | 10009, 456 + 56
+// 21377 | 16736; n = 14: 1 1372 | 74, 228 2113 | 1547; n = 12: 40 301 | 111, 228 448 | 535;
+// n = 10: 83 | 100.
+static bool fsc_tiles_pay(int n, int64_t rest) { return n >= 13 || (n == 12 && rest <= 64); }
+
+static int fsc_run(FscRows rows, int64_t most, int n, void *workspace, cudaStream_t s) {
     int err = 0;
-    const int grid = fsc_grid(n, batch, &err);
+    const int grid = fsc_grid(n, most, &err), full = fsc_grid(n, INT64_MAX, &err);
     if (err) return err;
-    fsc_kernel<<<grid, kFscThreads, fsc_smem(n), s>>>(a, n, batch, c, static_cast<double *>(workspace), nullptr,
-                                                      nullptr, nullptr, nullptr);
+    const int64_t rest = rows.order ? (most < full ? most : full) : most % full;
+    const bool tiled = n > kFscTileBits && rest && fsc_tiles_pay(n, rest);
+    rows.full = tiled ? full : 1;
+    double *ws = static_cast<double *>(workspace);
+    if (!tiled || most >= full) fsc_kernel<<<grid, kFscThreads, fsc_smem(n), s>>>(rows, n, ws);
+    if (tiled) {
+        const int64_t tiles = rest << (n - kFscTileBits);
+        const int g = static_cast<int>(tiles < 4 * full ? tiles : 4 * full);
+        const size_t smem = fsc_smem(n);
+        auto allow = [&](auto kern) {
+            return static_cast<int>(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                         static_cast<int>(fsc_smem(kFscMaxN))));
+        };
+        if ((err = allow(fsc_pass_kernel<0>)) || (err = allow(fsc_pass_kernel<1>)) || (err = allow(fsc_pass_kernel<2>)))
+            return err;
+        fsc_pass_kernel<0><<<g, kFscThreads, fsc_smem(10), s>>>(rows, n, ws);
+        fsc_pass_kernel<1><<<g, kFscThreads, smem, s>>>(rows, n, ws);
+        fsc_pass_kernel<2><<<g, kFscThreads, fsc_smem(10), s>>>(rows, n, ws);
+    }
     return static_cast<int>(cudaGetLastError());
+}
+
+int launch_fsc(const double *a, int n, int64_t batch, double *c, void *workspace, cudaStream_t s) {
+    return fsc_run({a, c, nullptr, nullptr, nullptr, nullptr, batch, 0}, batch, n, workspace, s);
 }
 
 int launch_fsc_items(double *c, const int64_t *c_off, const int *order, const unsigned *first,
                      const unsigned *count, int64_t max_items, int n, void *workspace, cudaStream_t s) {
-    int err = 0;
-    const int grid = fsc_grid(n, max_items, &err);
-    if (err) return err;
-    fsc_kernel<<<grid, kFscThreads, fsc_smem(n), s>>>(c, n, max_items, c, static_cast<double *>(workspace), order,
-                                                      c_off, first, count);
-    return static_cast<int>(cudaGetLastError());
+    return fsc_run({c, c, order, c_off, first, count, max_items, 0}, max_items, n, workspace, s);
 }
 
 }  // namespace apm

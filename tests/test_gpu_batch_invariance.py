@@ -118,3 +118,12 @@ def test_blocked_orders_from_weights(apm, n, batch):
     apm._check(apm.lib().apm_cdet_from_weights(apm._ptr(z), n, 4, apm._ptr(z), apm._ptr(ws), nb, apm._stream(z)),
                "apm_cdet_from_weights")
     rows_equal((c,), (z,), few)
+
+
+# the fast subset convolution: rounds of one CTA per row, the last one by tiles
+@pytest.mark.parametrize("n,batch", [(10, 500), (12, 520), (12, 530), (13, 460), (14, 457), (16, 459)])
+def test_fast_subset_convolution(apm, n, batch):
+    w = torch.rand((batch, 1 << n), dtype=torch.float64, device="cuda",
+                   generator=torch.Generator(device="cuda").manual_seed(n))
+    few = torch.as_tensor([0, 3, 455, 456, batch - 1]).cuda()
+    rows_equal((apm.cdet_from_weights_fsc(w),), (apm.cdet_from_weights_fsc(w[few]),), few)
