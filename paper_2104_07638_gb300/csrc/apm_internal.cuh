@@ -47,6 +47,15 @@ __device__ __forceinline__ void cp_async_wait_all() {
     asm volatile("cp.async.wait_group 0;" ::: "memory");
 }
 
+// CTAs of `threads` threads and `smem` bytes of dynamic shared memory that the
+// current device holds of this kernel, which is allowed `allow` bytes (the most
+// any launch of it takes) first; 0 and *err on failure. Remembered per context.
+int resident_ctas(const void *kern, int threads, size_t smem, size_t allow, int *err);
+template <class... A>
+inline int resident_ctas(void (*kern)(A...), int threads, size_t smem, size_t allow, int *err) {
+    return resident_ctas(reinterpret_cast<const void *>(kern), threads, smem, allow, err);
+}
+
 // Threads per CTA of the minor / connected-sum kernels.
 constexpr int kCdetThreads = 256;
 // Capacity of the per-matrix pivot-correction log.

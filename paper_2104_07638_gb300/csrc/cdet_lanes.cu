@@ -394,18 +394,11 @@ static int lanes_launch(const LanesParams &P, cudaStream_t s) {
     using T = Lanes<N, LG>;
     const size_t arrays = P.a.two_mats ? 3 : 2;
     const size_t smem = ((sizeof(typename T::Smem) + 15) & ~size_t(15)) + arrays * (T::STR << N) * sizeof(double);
-    int dev = 0, sms = 0, per_sm = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(cdet_lanes_kernel<N, LG>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 static_cast<int>(((sizeof(typename T::Smem) + 15) & ~size_t(15)) +
-                                                  3 * (T::STR << N) * sizeof(double)));
-    if (e == cudaSuccess)
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, cdet_lanes_kernel<N, LG>, 32, smem);
-    if (e != cudaSuccess) return static_cast<int>(e);
-    if (per_sm < 1) return static_cast<int>(cudaErrorInvalidConfiguration);
-    const int64_t need = (P.a.batch + T::MPW - 1) / T::MPW, most = static_cast<int64_t>(sms) * per_sm;
+    const size_t allow = ((sizeof(typename T::Smem) + 15) & ~size_t(15)) + 3 * (T::STR << N) * sizeof(double);
+    int err = 0;
+    const int64_t most = resident_ctas(cdet_lanes_kernel<N, LG>, 32, smem, allow, &err);
+    if (err) return err;
+    const int64_t need = (P.a.batch + T::MPW - 1) / T::MPW;
     cdet_lanes_kernel<N, LG><<<static_cast<int>(need < most ? need : most), 32, smem, s>>>(P);
     return static_cast<int>(cudaGetLastError());
 }

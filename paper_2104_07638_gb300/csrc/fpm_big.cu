@@ -300,9 +300,10 @@ int launch_fpm_big(const double *A, int n, int64_t batch, double *minors, double
     // levels s1 .. H-1 for each node of level s1; the leaves' minors in det[0]
     const int s1 = p.s1, s2 = H - s1;
     const BigSubLayout L1 = big_sub_layout(n, 0, s1), L2 = big_sub_layout(n, s1, s2);
-    err = static_cast<int>(cudaFuncSetAttribute(big_subtree_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                static_cast<int>(L1.bytes > L2.bytes ? L1.bytes : L2.bytes)));
+    const size_t most = 160 * 1024;  // more than either takes at any order (order 24: 142 KB)
+    resident_ctas(big_subtree_kernel, kBigSubThreads, most, most, &err);
     if (err) return err;
+    if (L1.bytes > most || L2.bytes > most) return static_cast<int>(cudaErrorInvalidValue);
     big_subtree_kernel<<<static_cast<unsigned>(batch), kBigSubThreads, L1.bytes, s>>>(
         A, det[0], nodeM, det[1], n, 0, s1, L1.odd, L1.ip, L1.nd, thrA, Cm, ccount, clog, flags);
     big_subtree_kernel<<<static_cast<unsigned>(batch << s1), kBigSubThreads, L2.bytes, s>>>(

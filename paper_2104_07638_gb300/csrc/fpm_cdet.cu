@@ -1038,31 +1038,11 @@ static int cdet_threads(int n, int64_t batch) {
 }
 
 int cdet_grid(int n, int64_t batch, bool two_mats, bool smem_arrays, int *err) {
-    int dev = 0, sms = 0, per_sm = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const size_t smem = cdet_smem_bytes(n, two_mats, smem_arrays);
-    if (e == cudaSuccess) {
-        if (smem_arrays) {
-            e = cudaFuncSetAttribute(fpm_cdet_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     static_cast<int>(smem));
-            if (e == cudaSuccess)
-                e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fpm_cdet_kernel<true>,
-                                                                  cdet_threads(n, batch), smem);
-        } else {
-            e = cudaFuncSetAttribute(fpm_cdet_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     static_cast<int>(smem));
-            if (e == cudaSuccess)
-                e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fpm_cdet_kernel<false>,
-                                                                  kCdetThreads, smem);
-        }
-    }
-    if (e != cudaSuccess || per_sm < 1) {
-        if (err) *err = e != cudaSuccess ? static_cast<int>(e) : static_cast<int>(cudaErrorInvalidConfiguration);
-        return 0;
-    }
-    if (err) *err = 0;
-    int64_t g = static_cast<int64_t>(sms) * per_sm;
+    int64_t g = smem_arrays ? resident_ctas(fpm_cdet_kernel<true>, cdet_threads(n, batch), smem,
+                                            cdet_smem_bytes(cdet_smem_max_n(true), true, true), err)
+                            : resident_ctas(fpm_cdet_kernel<false>, kCdetThreads, smem, smem, err);
+    if (*err) return 0;
     if (batch < g) g = batch;
     return static_cast<int>(g < 1 ? 1 : g);
 }
@@ -1227,21 +1207,17 @@ static int varlen_smem_n(int n_max) { return n_max < kVarlenSmemMaxN ? n_max : k
 static size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
 
 static int cdet_varlen_grid(int n_max, bool two_mats, int *err) {
-    int dev = 0, sms = 0, per_sm = 0;
+    int dev = 0, sms = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const size_t smem = cdet_smem_bytes(varlen_smem_n(n_max), two_mats, true);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(fpm_cdet_varlen_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 static_cast<int>(cdet_smem_bytes(kVarlenSmemMaxN, true, true)));
-    if (e == cudaSuccess)
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fpm_cdet_varlen_kernel, varlen_threads(n_max),
-                                                          smem);
-    if (e != cudaSuccess || per_sm < 1) {
-        *err = e != cudaSuccess ? static_cast<int>(e) : static_cast<int>(cudaErrorInvalidConfiguration);
+    if (e != cudaSuccess) {
+        *err = static_cast<int>(e);
         return 0;
     }
-    *err = 0;
+    int per_sm = resident_ctas(fpm_cdet_varlen_kernel, varlen_threads(n_max),
+                               cdet_smem_bytes(varlen_smem_n(n_max), two_mats, true),
+                               cdet_smem_bytes(kVarlenSmemMaxN, true, true), err) / sms;
+    if (*err) return 0;
     // the tuned limit counts CTAs of kCdetThreads threads
     const int most = g_varlen_ctas * (kCdetThreads / varlen_threads(n_max));
     if (most > 0 && most < per_sm) per_sm = most;

@@ -406,20 +406,8 @@ static FwRouteKernel fw_route_kernel_for(int T) {
 // The warps the chip holds (CTAs of kFwWarps) of one of the kernels above.
 template <class K>
 static int fw_resident(K kern, int *err) {
-    int dev = 0, sms = 0, per_sm = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const size_t smem = kFwWarps * sizeof(FwWarpSmem);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
-    if (e == cudaSuccess)
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kFwWarps * 32, smem);
-    if (e != cudaSuccess || per_sm < 1) {
-        *err = e != cudaSuccess ? static_cast<int>(e) : static_cast<int>(cudaErrorInvalidConfiguration);
-        return 0;
-    }
-    *err = 0;
-    return sms * per_sm * kFwWarps;
+    return resident_ctas(kern, kFwWarps * 32, smem, smem, err) * kFwWarps;
 }
 
 // Tail size and runs per matrix (log2) for a batch: the longest tail whose

@@ -467,20 +467,8 @@ __global__ void __launch_bounds__(kFscThreads, 3) fsc_pass_kernel(const FscRows 
 static size_t fsc_smem(int n) { return static_cast<size_t>(n) * kFscTile * sizeof(double); }
 
 int fsc_grid(int n, int64_t batch, int *err) {
-    int dev = 0, sms = 0, per_sm = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const size_t smem = fsc_smem(n);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(fsc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 static_cast<int>(fsc_smem(kFscMaxN)));
-    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fsc_kernel, kFscThreads, smem);
-    if (e != cudaSuccess || per_sm < 1) {
-        *err = e != cudaSuccess ? static_cast<int>(e) : static_cast<int>(cudaErrorInvalidConfiguration);
-        return 0;
-    }
-    *err = 0;
-    int64_t g = static_cast<int64_t>(sms) * per_sm;
+    int64_t g = resident_ctas(fsc_kernel, kFscThreads, fsc_smem(n), fsc_smem(kFscMaxN), err);
+    if (*err) return 0;
     if (batch < g) g = batch;
     return static_cast<int>(g < 1 ? 1 : g);
 }
@@ -515,11 +503,10 @@ static int fsc_run(FscRows rows, int64_t most, int n, void *workspace, cudaStrea
         const int g = static_cast<int>(tiles < 4 * full ? tiles : 4 * full);
         const size_t smem = fsc_smem(n);
         auto allow = [&](auto kern) {
-            return static_cast<int>(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                         static_cast<int>(fsc_smem(kFscMaxN))));
+            if (!err) resident_ctas(kern, kFscThreads, smem, fsc_smem(kFscMaxN), &err);
         };
-        if ((err = allow(fsc_pass_kernel<0>)) || (err = allow(fsc_pass_kernel<1>)) || (err = allow(fsc_pass_kernel<2>)))
-            return err;
+        allow(fsc_pass_kernel<0>), allow(fsc_pass_kernel<1>), allow(fsc_pass_kernel<2>);
+        if (err) return err;
         fsc_pass_kernel<0><<<g, kFscThreads, fsc_smem(10), s>>>(rows, n, ws);
         fsc_pass_kernel<1><<<g, kFscThreads, smem, s>>>(rows, n, ws);
         fsc_pass_kernel<2><<<g, kFscThreads, fsc_smem(10), s>>>(rows, n, ws);

@@ -451,13 +451,8 @@ int launch_keldysh_varlen(const double *Mt, const int64_t *m_off, const int *n_a
     if (err) return err;
     const int warps = g_kel_varlen_warps > 0 ? g_kel_varlen_warps : kKelWarps;
     const size_t smem = static_cast<size_t>(warps) * sizeof(KelWarpSmem);
-    int dev = 0, sms = 0, per_sm = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e == cudaSuccess)
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, keldysh_varlen_kernel, warps * 32, smem);
-    if (e != cudaSuccess || per_sm < 1) return e != cudaSuccess ? static_cast<int>(e) : 1;
-    int64_t grid = static_cast<int64_t>(sms) * per_sm;
+    int64_t grid = resident_ctas(keldysh_varlen_kernel, warps * 32, smem, kKelWarps * sizeof(KelWarpSmem), &err);
+    if (err) return err;
     const int64_t slots = static_cast<int64_t>(full) * kKelWarps;  // stacks in the workspace
     if (grid * warps > slots) grid = slots / warps;
     const int64_t need = (batch + warps - 1) / warps;
@@ -471,25 +466,10 @@ int launch_keldysh_varlen(const double *Mt, const int64_t *m_off, const int *n_a
 size_t keldysh_stack_entries(int n) { return kel_stack_entries(n); }
 
 int keldysh_grid(int64_t batch, int *err) {
-    int dev = 0, sms = 0, per_sm = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const size_t smem = kKelWarps * sizeof(KelWarpSmem);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(keldysh_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 static_cast<int>(smem));
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(keldysh_varlen_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 static_cast<int>(smem));
-    if (e == cudaSuccess)
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, keldysh_kernel, kKelWarps * 32, smem);
-    if (e != cudaSuccess || per_sm < 1) {
-        *err = e != cudaSuccess ? static_cast<int>(e) : static_cast<int>(cudaErrorInvalidConfiguration);
-        return 0;
-    }
-    *err = 0;
+    int64_t g = resident_ctas(keldysh_kernel, kKelWarps * 32, smem, smem, err);
+    if (*err) return 0;
     const int64_t need = (batch + kKelWarps - 1) / kKelWarps;
-    int64_t g = static_cast<int64_t>(sms) * per_sm;
     if (need < g) g = need;
     return static_cast<int>(g < 1 ? 1 : g);
 }

@@ -333,22 +333,10 @@ __global__ void __launch_bounds__(kK2Warps * 32, 1) keldysh2_kernel(
 }
 
 int keldysh2_grid(int64_t batch, int *err) {
-    int dev = 0, sms = 0, per_sm = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const size_t smem = kK2Warps * sizeof(K2WarpSmem);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(keldysh2_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 static_cast<int>(smem));
-    if (e == cudaSuccess)
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, keldysh2_kernel, kK2Warps * 32, smem);
-    if (e != cudaSuccess || per_sm < 1) {
-        *err = e != cudaSuccess ? static_cast<int>(e) : static_cast<int>(cudaErrorInvalidConfiguration);
-        return 0;
-    }
-    *err = 0;
+    int64_t g = resident_ctas(keldysh2_kernel, kK2Warps * 32, smem, smem, err);
+    if (*err) return 0;
     const int64_t need = (batch + kK2Warps - 1) / kK2Warps;
-    int64_t g = static_cast<int64_t>(sms) * per_sm;
     if (need < g) g = need;
     return static_cast<int>(g < 1 ? 1 : g);
 }

@@ -679,35 +679,18 @@ __global__ void __launch_bounds__(kNdWarps * 32, kNdMinBlocks) nand_kernel(const
 }
 
 int nand_grid(int64_t batch, int *err) {
-    int dev = 0, sms = 0, per_sm = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const size_t smem = kNdWarps * sizeof(NdWarpSmem);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(nand_kernel<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 static_cast<int>(smem));
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(nand_kernel<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 static_cast<int>(smem));
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(nand_kernel<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 static_cast<int>(smem));
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(nand_kernel<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 static_cast<int>(smem));
-    int per_sm2 = 0;
-    if (e == cudaSuccess)
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, nand_kernel<true, false>, kNdWarps * 32, smem);
-    if (e == cudaSuccess)
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm2, nand_kernel<true, true>, kNdWarps * 32, smem);
-    if (per_sm2 < per_sm) per_sm = per_sm2;
-    if (e != cudaSuccess || per_sm < 1) {
-        *err = e != cudaSuccess ? static_cast<int>(e) : static_cast<int>(cudaErrorInvalidConfiguration);
-        return 0;
-    }
+    int64_t g = 0;
+    auto fits = [&](auto kern) {
+        if (*err) return;
+        const int c = resident_ctas(kern, kNdWarps * 32, smem, smem, err);
+        if (g == 0 || c < g) g = c;
+    };
     *err = 0;
+    fits(nand_kernel<false, false>), fits(nand_kernel<false, true>);
+    fits(nand_kernel<true, false>), fits(nand_kernel<true, true>);
+    if (*err) return 0;
     const int64_t need = (batch + kNdWarps - 1) / kNdWarps;
-    int64_t g = static_cast<int64_t>(sms) * per_sm;
     if (need < g) g = need;
     return static_cast<int>(g < 1 ? 1 : g);
 }

@@ -609,17 +609,9 @@ static int ensure_ppm_schedules() {
 int launch_ppm(const double *A, int n, int64_t batch, double *perms, cudaStream_t s) {
     int err = ensure_ppm_schedules();
     if (err) return err;
-    int dev = 0, sms = 0, per_sm = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const size_t smem = sizeof(PpmSmem);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(ppm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
-    if (e == cudaSuccess)
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, ppm_kernel, kPpmWarps * 32, smem);
-    if (e != cudaSuccess) return static_cast<int>(e);
-    if (per_sm < 1) return static_cast<int>(cudaErrorInvalidConfiguration);
-    int64_t g = static_cast<int64_t>(sms) * per_sm;
+    int64_t g = resident_ctas(ppm_kernel, kPpmWarps * 32, smem, smem, &err);
+    if (err) return err;
     if (batch < g) g = batch;
     const int l = n < kPpmMaxL ? n : kPpmMaxL;
     ppm_kernel<<<static_cast<int>(g), kPpmWarps * 32, smem, s>>>(A, n, batch, perms, h_sched[l]);

@@ -327,21 +327,10 @@ __global__ void __launch_bounds__(kXnWarps * 32, kXnMinBlocks) xnor_kernel(const
 }
 
 int xnor_grid(int64_t batch, int *err) {
-    int dev = 0, sms = 0, per_sm = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const size_t smem = kXnWarps * sizeof(XnWarpSmem);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(xnor_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
-    if (e == cudaSuccess)
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, xnor_kernel, kXnWarps * 32, smem);
-    if (e != cudaSuccess || per_sm < 1) {
-        *err = e != cudaSuccess ? static_cast<int>(e) : static_cast<int>(cudaErrorInvalidConfiguration);
-        return 0;
-    }
-    *err = 0;
+    int64_t g = resident_ctas(xnor_kernel, kXnWarps * 32, smem, smem, err);
+    if (*err) return 0;
     const int64_t need = (batch + kXnWarps - 1) / kXnWarps;
-    int64_t g = static_cast<int64_t>(sms) * per_sm;
     if (need < g) g = need;
     return static_cast<int>(g < 1 ? 1 : g);
 }
