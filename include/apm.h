@@ -350,8 +350,10 @@ apm_status_t apm_keldysh_sum(const double *Mt, int n, int64_t batch, int flags, 
  *   status   [batch] or NULL; APM_ST_ZERO_PIVOT marks a zero or non-finite pivot
  *            in either spin, and then that pair's results are NaN.
  *   workspace / workspace_bytes: scratch for the depth-first part (both spins'
- *            path matrices), needed for n > 7 (apm_workspace_size with
- *            APM_OP_KELDYSH2).
+ *            path matrices) and the sums of split pairs, needed for n > 7
+ *            (apm_workspace_size with APM_OP_KELDYSH2). A small batch's pairs are
+ *            split over several warps as apm_keldysh_sum's matrices are: such
+ *            results differ from whole pairs' by rounding, and are reproducible.
  */
 apm_status_t apm_keldysh2_sum(const double *Mu, const double *Md, int n, int64_t batch, int flags, double *sum,
                               double *partial, uint32_t *status, void *workspace, size_t workspace_bytes,

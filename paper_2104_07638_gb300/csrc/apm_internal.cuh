@@ -181,7 +181,7 @@ void cdet_group_table(int n, int threads, uint8_t *gsel /*[17]*/);
 // Fixed-order Keldysh launch layout: grid, chunks per matrix (log2) and the
 // workspace parts (depth-first stacks, chunk slots, chunk flags, counters).
 struct KeldyshPlan {
-    int grid;
+    int grid, warps;
     int kc;
     size_t stack_bytes, slot_bytes, flag_bytes, ctr_bytes, total;
 };
@@ -190,6 +190,8 @@ int launch_keldysh(const double *Mt, int n, int64_t batch, int sgn, double *sum,
                    uint32_t *status, void *workspace, cudaStream_t s);
 int keldysh_grid(int64_t batch, int *err);
 int keldysh_warps_per_block();
+int keldysh_spread(int64_t items);
+int keldysh_chunks(int64_t batch, int D, int64_t warps);
 size_t keldysh_stack_entries(int n);
 
 int launch_ppm(const double *A, int n, int64_t batch, double *perms, cudaStream_t s);
@@ -201,7 +203,6 @@ int launch_xnor(const double *M, int n, int64_t batch, double *minors, uint32_t 
                 cudaStream_t s);
 
 // Two-spin Keldysh sums (one warp per matrix pair).
-int keldysh2_grid(int64_t batch, int *err);
 size_t keldysh2_workspace_bytes(int n, int64_t batch, int *err);
 int launch_keldysh2(const double *Mu, const double *Md, int n, int64_t batch, int sgn, double *sum,
                     double *partial, uint32_t *status, void *workspace, cudaStream_t s);

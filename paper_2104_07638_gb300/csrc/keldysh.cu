@@ -360,8 +360,8 @@ __global__ void __launch_bounds__(kKelWarps * 32, kKelMinBlocks) keldysh_kernel(
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     KelWarpSmem &w = reinterpret_cast<KelWarpSmem *>(smem_raw)[wid];
-    const int64_t gw = static_cast<int64_t>(blockIdx.x) * kKelWarps + wid;
-    const int64_t nw = static_cast<int64_t>(gridDim.x) * kKelWarps;
+    const int64_t gw = static_cast<int64_t>(blockIdx.x) * (blockDim.x >> 5) + wid;
+    const int64_t nw = static_cast<int64_t>(gridDim.x) * (blockDim.x >> 5);
     double2 *stack = stack_base ? stack_base + gw * stack_per_warp : nullptr;
     const int64_t m0 = 2 * n;
     const int D = n > kKelTail ? n - kKelTail : 0;
@@ -392,6 +392,7 @@ __global__ void __launch_bounds__(kKelWarps * 32, kKelMinBlocks) keldysh_kernel(
         double2 v = make_double2(0.0, 0.0);
         uint32_t fl = 0;
         const double2 *slot_b = slots + (b << kc) * (n + 1);
+#pragma unroll 8
         for (int64_t cc = 0; cc < nchunk; ++cc) {
             if (lane <= n) v = cadd(v, __ldcg(slot_b + cc * (n + 1) + lane));
             fl |= __ldcg(slot_flags + (b << kc) + cc);
@@ -441,6 +442,14 @@ static int g_kel_varlen_warps = 0;
 int keldysh_varlen_warps() { return g_kel_varlen_warps; }
 void keldysh_varlen_warps_set(int w) { g_kel_varlen_warps = w; }
 
+// Warps per CTA for this many work items: no more than put one CTA on every SM
+// (a warp's work is bound by its own SM partition's FP64 unit; 1000 matrices of
+// order 9 in CTAs of 12 warps left 68 of 152 SMs empty: 225 -> 133 us).
+int keldysh_spread(int64_t items) {
+    const int64_t w = (items + 151) / 152;
+    return w < 1 ? 1 : w < kKelWarps ? static_cast<int>(w) : kKelWarps;
+}
+
 int launch_keldysh_varlen(const double *Mt, const int64_t *m_off, const int *n_arr, int64_t batch, int n_max,
                           int sgn, double *sum, double *partial, uint32_t *status, void *stack,
                           const int *order, unsigned *ctr, cudaStream_t s) {
@@ -449,7 +458,8 @@ int launch_keldysh_varlen(const double *Mt, const int64_t *m_off, const int *n_a
     // (keldysh_grid(batch) CTAs of kKelWarps warps, as apm_workspace_size sizes it)
     const int full = keldysh_grid(batch, &err);
     if (err) return err;
-    const int warps = g_kel_varlen_warps > 0 ? g_kel_varlen_warps : kKelWarps;
+    const int spread = keldysh_spread(batch);
+    const int warps = g_kel_varlen_warps > 0 && g_kel_varlen_warps < spread ? g_kel_varlen_warps : spread;
     const size_t smem = static_cast<size_t>(warps) * sizeof(KelWarpSmem);
     int64_t grid = resident_ctas(keldysh_varlen_kernel, warps * 32, smem, kKelWarps * sizeof(KelWarpSmem), &err);
     if (err) return err;
@@ -476,25 +486,21 @@ int keldysh_grid(int64_t batch, int *err) {
 
 int keldysh_warps_per_block() { return kKelWarps; }
 
-// Chunks per matrix for a fixed-order launch: the smallest power of two whose
-// (matrix, chunk) items fill at least 90 % of the warps' last round (chunks of
-// at least 4 depth-first leaves), else the best fill among those allowed.
-static int keldysh_chunk_log2(int n, int64_t batch, int64_t warps) {
-    const int D = n > kKelTail ? n - kKelTail : 0;
-    const int kmax = D > 2 ? D - 2 : 0;
-    int best = 0;
-    double best_fill = 0.0;
-    for (int k = 0; k <= kmax; ++k) {
-        const int64_t items = batch << k;
-        const int64_t rounds = (items + warps - 1) / warps;
-        const double fill = static_cast<double>(items) / static_cast<double>(rounds * warps);
-        if (fill >= 0.9) return k;
-        if (fill > best_fill + 1e-12) {
-            best_fill = fill;
-            best = k;
-        }
+// Chunks per matrix (log2, at most D) for `warps` resident warps. Up to one round
+// of them: as many chunks as that round holds (the FP64 units saturate at about 6
+// warps per SM, and a second round of smaller items costs more than it balances:
+// two-spin sums of order 12, 64 pairs, k = 3..6: 278, 181, 335, 374 us). Beyond:
+// enough items that the last, partial round is a small part, but not more than 4
+// chunks, whose paths the matrix then pays for (2200 pairs, k = 0..3: 6913, 5205,
+// 4434, 4597 us). Items <= warps for batch <= warps, < 9 warps otherwise.
+int keldysh_chunks(int64_t batch, int D, int64_t warps) {
+    int k = 0;
+    if (batch <= warps) {
+        while (k < D && (batch << (k + 1)) <= warps) ++k;
+    } else {
+        while (k < 2 && k < D && 2 * (batch << k) < 9 * warps) ++k;
     }
-    return best;
+    return k;
 }
 
 int keldysh_plan(int n, int64_t batch, KeldyshPlan *p) {
@@ -502,11 +508,13 @@ int keldysh_plan(int n, int64_t batch, KeldyshPlan *p) {
     const int full = keldysh_grid(INT64_MAX / 64, &err);  // all resident CTAs
     if (err) return err;
     const int64_t warps = static_cast<int64_t>(full) * kKelWarps;
-    p->kc = keldysh_chunk_log2(n, batch, warps);
+    // orders 8 and 9 stay whole: they are the uneven batch's sums, bit for bit
+    p->kc = n > kKelTail + 2 ? keldysh_chunks(batch, n - kKelTail, warps) : 0;
     const int64_t items = batch << p->kc;
-    const int64_t need = (items + kKelWarps - 1) / kKelWarps;
+    p->warps = keldysh_spread(items);
+    const int64_t need = (items + p->warps - 1) / p->warps;
     p->grid = static_cast<int>(need < full ? (need < 1 ? 1 : need) : full);
-    p->stack_bytes = static_cast<size_t>(p->grid) * kKelWarps * kel_stack_entries(n) * sizeof(double2);
+    p->stack_bytes = static_cast<size_t>(p->grid) * p->warps * kel_stack_entries(n) * sizeof(double2);
     if (p->kc == 0) {
         p->slot_bytes = p->flag_bytes = p->ctr_bytes = 0;
     } else {
@@ -535,8 +543,8 @@ int launch_keldysh(const double *Mt, int n, int64_t batch, int sgn, double *sum,
         const cudaError_t e = cudaMemsetAsync(ctr, 0, static_cast<size_t>(batch) * sizeof(unsigned), s);
         if (e != cudaSuccess) return static_cast<int>(e);
     }
-    const size_t smem = kKelWarps * sizeof(KelWarpSmem);
-    keldysh_kernel<<<p.grid, kKelWarps * 32, smem, s>>>(reinterpret_cast<const double2 *>(Mt), n, batch, sgn,
+    const size_t smem = p.warps * sizeof(KelWarpSmem);
+    keldysh_kernel<<<p.grid, p.warps * 32, smem, s>>>(reinterpret_cast<const double2 *>(Mt), n, batch, sgn,
                                                         sum, partial, status, stack, kel_stack_entries(n), p.kc,
                                                         slots, slot_flags, ctr);
     return static_cast<int>(cudaGetLastError());

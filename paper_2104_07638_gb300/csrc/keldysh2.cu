@@ -238,16 +238,18 @@ __device__ __forceinline__ void k2_schur(const double2 *s0, const double2 *s1, i
     __syncwarp();
 }
 
-// One matrix pair of order n (whole warp): writes sum[2], partial[(n+1)*2] (if
-// not NULL) and the status word; NaN where a pivot failed or an input is not finite.
-__device__ __forceinline__ void k2_matrix(const double2 *Au, const double2 *Ad, int n, bool sgn, double *sum_out,
-                                          double *partial_out, uint32_t *status_out, double2 *stack,
-                                          K2WarpSmem &w, int lane) {
-    const bool want_part = partial_out != nullptr;
+// Depth-first leaves t0 <= t < t1 of one matrix pair of order n (whole warp; all
+// 2^(n-S), or one chunk). Leaves the sums in w.part[0..n] (part[0] = 1) and sets
+// bad / nonfin. A node's product joins its depth's sum at its first leaf only, so
+// chunks of one pair never count a node twice.
+__device__ __forceinline__ void k2_matrix(const double2 *Au, const double2 *Ad, int n, bool sgn, bool want_part,
+                                          int64_t t0, int64_t t1, double2 *stack, K2WarpSmem &w, int lane, int &bad,
+                                          int &nonfin) {
     const int s = n < kK2Tail ? n : kK2Tail;
     const int D = n - s;
     const int m0 = 2 * n;
-    int bad = 0, nonfin = 0;
+    bad = 0;
+    nonfin = 0;
     for (int e = lane; e < m0 * m0; e += 32) {
         const double2 u = Au[e], d = Ad[e];
         nonfin |= nonfinite_bits(u.x) | nonfinite_bits(u.y) | nonfinite_bits(d.x) | nonfinite_bits(d.y);
@@ -269,8 +271,8 @@ __device__ __forceinline__ void k2_matrix(const double2 *Au, const double2 *Ad, 
         k2_tail_order<kK2Tail>(n, want_part, sgn, w, lane, bad, acc);
     } else {
         const size_t half = k2_stack_entries(n) / 2;  // the down spin's path matrices follow the up spin's
-        for (int64_t t = 0; t < (int64_t(1) << D); ++t) {
-            const int d0 = t == 0 ? 0 : D - __ffsll(t);
+        for (int64_t t = t0; t < t1; ++t) {
+            const int d0 = t == t0 ? 0 : D - __ffsll(t);  // a chunk's first leaf builds its whole path
             size_t off = 0;  // stack offset of depth d0 (depths 1..D-1 are stacked)
             for (int d = 1; d < d0; ++d) off += static_cast<size_t>(2 * (n - d)) * (2 * (n - d));
             for (int d = d0; d < D; ++d) {
@@ -279,14 +281,15 @@ __device__ __forceinline__ void k2_matrix(const double2 *Au, const double2 *Ad, 
                 const double2 *s0 = d == 0 ? Au : stack + off;
                 const double2 *s1 = d == 0 ? Ad : stack + half + off;
                 if (d > 0) off += static_cast<size_t>(m) * m;
-                double2 *t0 = (d + 1 == D) ? w.bufE[0] : stack + off;
-                double2 *t1 = (d + 1 == D) ? w.bufE[1] : stack + half + off;
+                double2 *r0 = (d + 1 == D) ? w.bufE[0] : stack + off;
+                double2 *r1 = (d + 1 == D) ? w.bufE[1] : stack + half + off;
                 double2 p0, p1;
-                k2_schur(s0, s1, m, alpha, t0, t1, d + 1 == D, w, lane, p0, p1, bad);
+                k2_schur(s0, s1, m, alpha, r0, r1, d + 1 == D, w, lane, p0, p1, bad);
                 if (lane == 0) {
                     const double2 pd = cneg_if(cmul(cmul(w.pdet[d], p0), p1), sgn && alpha);
                     w.pdet[d + 1] = pd;
-                    if (want_part) w.part[d + 1] = cadd(w.part[d + 1], pd);
+                    const bool first_leaf = (t & ((int64_t(1) << (D - 1 - d)) - 1)) == 0;
+                    if (want_part && first_leaf) w.part[d + 1] = cadd(w.part[d + 1], pd);
                 }
                 __syncwarp();
             }
@@ -302,6 +305,12 @@ __device__ __forceinline__ void k2_matrix(const double2 *Au, const double2 *Ad, 
     }
     bad = __any_sync(0xffffffffu, bad);
     __syncwarp();
+}
+
+// Results of one pair from w.part: sum[2], partial[(n+1)*2] (if not NULL) and the
+// status word; NaN where a pivot failed or an input is not finite.
+__device__ __forceinline__ void k2_store(int n, int bad, int nonfin, double *sum_out, double *partial_out,
+                                         uint32_t *status_out, const K2WarpSmem &w, int lane) {
     const double nanv = __longlong_as_double(0x7ff8000000000000ll);
     if (lane == 0) {
         const double2 r = (bad || nonfin) ? make_double2(nanv, nanv) : w.part[n];
@@ -309,7 +318,7 @@ __device__ __forceinline__ void k2_matrix(const double2 *Au, const double2 *Ad, 
         sum_out[1] = r.y;
         if (status_out) *status_out = (bad ? APM_ST_ZERO_PIVOT : 0u) | (nonfin ? APM_ST_NONFINITE_INPUT : 0u);
     }
-    if (want_part && lane <= n) {
+    if (partial_out && lane <= n) {
         const double2 r = (bad || nonfin) ? make_double2(nanv, nanv) : w.part[lane];
         partial_out[2 * lane] = r.x;
         partial_out[2 * lane + 1] = r.y;
@@ -317,48 +326,114 @@ __device__ __forceinline__ void k2_matrix(const double2 *Au, const double2 *Ad, 
     __syncwarp();
 }
 
+// Work items are (pair, chunk): 2^kc chunks of consecutive depth-first leaves per
+// pair. With kc > 0 every chunk writes its sums and flags to a slot and counts
+// itself in ctr[b] (zero at launch); the warp that completes the count adds the
+// slots in chunk order, whichever warp that is, and stores the pair's results.
 __global__ void __launch_bounds__(kK2Warps * 32, 1) keldysh2_kernel(
     const double2 *__restrict__ Mu, const double2 *__restrict__ Md, int n, int64_t batch, int sgn_flag,
-    double *sum, double *partial, uint32_t *status, double2 *stack_base, size_t stack_per_warp) {
+    double *sum, double *partial, uint32_t *status, double2 *stack_base, size_t stack_per_warp, int kc,
+    double2 *slots, uint32_t *slot_flags, unsigned *ctr) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     K2WarpSmem &w = reinterpret_cast<K2WarpSmem *>(smem_raw)[wid];
-    const int64_t gw = static_cast<int64_t>(blockIdx.x) * kK2Warps + wid;
-    const int64_t nw = static_cast<int64_t>(gridDim.x) * kK2Warps;
+    const int64_t gw = static_cast<int64_t>(blockIdx.x) * (blockDim.x >> 5) + wid;
+    const int64_t nw = static_cast<int64_t>(gridDim.x) * (blockDim.x >> 5);
     double2 *stack = stack_base ? stack_base + gw * stack_per_warp : nullptr;
     const int64_t m0 = 2 * n;
-    for (int64_t b = gw; b < batch; b += nw)
-        k2_matrix(Mu + b * m0 * m0, Md + b * m0 * m0, n, sgn_flag != 0, sum + 2 * b,
-                  partial ? partial + b * (n + 1) * 2 : nullptr, status ? status + b : nullptr, stack, w, lane);
+    const int D = n > kK2Tail ? n - kK2Tail : 0;
+    const int64_t nchunk = int64_t(1) << kc, leaves = int64_t(1) << (D - kc);
+    for (int64_t it = gw; it < (batch << kc); it += nw) {
+        const int64_t b = it >> kc, c = it & (nchunk - 1);
+        int bad, nonfin;
+        k2_matrix(Mu + b * m0 * m0, Md + b * m0 * m0, n, sgn_flag != 0, partial != nullptr, c * leaves,
+                  (c + 1) * leaves, stack, w, lane, bad, nonfin);
+        if (kc) {
+            double2 *slot = slots + it * (n + 1);
+            if (lane <= n) slot[lane] = w.part[lane];
+            if (lane == 0) slot_flags[it] = (bad ? 1u : 0u) | (nonfin ? 2u : 0u);
+            __threadfence();
+            __syncwarp();
+            unsigned prev = 0;
+            if (lane == 0) prev = atomicAdd(ctr + b, 1u);
+            prev = __shfl_sync(0xffffffffu, prev, 0);
+            if (prev != static_cast<unsigned>(nchunk - 1)) continue;
+            __threadfence();
+            double2 v = make_double2(0.0, 0.0);
+            uint32_t fl = 0;
+#pragma unroll 8
+            for (int64_t cc = b << kc; cc < (b + 1) << kc; ++cc) {
+                if (lane <= n) v = cadd(v, __ldcg(slots + cc * (n + 1) + lane));
+                fl |= __ldcg(slot_flags + cc);
+            }
+            if (lane <= n) w.part[lane] = lane == 0 ? make_double2(1.0, 0.0) : v;
+            __syncwarp();
+            bad = fl & 1u;
+            nonfin = (fl >> 1) & 1u;
+        }
+        k2_store(n, bad, nonfin, sum + 2 * b, partial ? partial + b * (n + 1) * 2 : nullptr,
+                 status ? status + b : nullptr, w, lane);
+    }
 }
 
-int keldysh2_grid(int64_t batch, int *err) {
-    const size_t smem = kK2Warps * sizeof(K2WarpSmem);
-    int64_t g = resident_ctas(keldysh2_kernel, kK2Warps * 32, smem, smem, err);
-    if (*err) return 0;
-    const int64_t need = (batch + kK2Warps - 1) / kK2Warps;
-    if (need < g) g = need;
-    return static_cast<int>(g < 1 ? 1 : g);
+// Grid, warps per CTA, chunks per pair (log2, keldysh_chunks) and the workspace's
+// parts; the warps are spread over the SMs. 300 pairs of order 8, 206 us as whole
+// pairs in CTAs of 12 warps on 25 SMs, take 45 us; 64 of order 12 3451 -> 181 us,
+// 2200 6913 -> 4434.
+struct K2Plan {
+    int grid, warps, kc;
+    size_t stack, slot, flag, ctr, total;
+};
+static int k2_plan(int n, int64_t batch, K2Plan *p) {
+    int err = 0;
+    const int full = resident_ctas(keldysh2_kernel, kK2Warps * 32, kK2Warps * sizeof(K2WarpSmem),
+                                   kK2Warps * sizeof(K2WarpSmem), &err);
+    if (err) return err;
+    const int D = n > kK2Tail ? n - kK2Tail : 0;
+    p->kc = D > 1 ? keldysh_chunks(batch, D, static_cast<int64_t>(full) * kK2Warps) : 0;
+    const int64_t items = batch << p->kc, w = (items + full - 1) / full;
+    p->warps = w < 1 ? 1 : w < kK2Warps ? static_cast<int>(w) : kK2Warps;
+    const int64_t need = (items + p->warps - 1) / p->warps;
+    p->grid = static_cast<int>(need < full ? (need < 1 ? 1 : need) : full);
+    p->stack = static_cast<size_t>(p->grid) * p->warps * k2_stack_entries(n) * sizeof(double2);
+    p->slot = p->kc ? static_cast<size_t>(items) * (n + 1) * sizeof(double2) : 0;
+    p->flag = p->kc ? (static_cast<size_t>(items) * sizeof(uint32_t) + 15) & ~size_t(15) : 0;
+    p->ctr = p->kc ? (static_cast<size_t>(batch) * sizeof(unsigned) + 15) & ~size_t(15) : 0;
+    p->total = p->stack + p->slot + p->flag + p->ctr;
+    return 0;
 }
 
 size_t keldysh2_workspace_bytes(int n, int64_t batch, int *err) {
     *err = 0;
-    const size_t per = k2_stack_entries(n);
-    if (per == 0 || batch == 0) return 0;
-    const int grid = keldysh2_grid(batch, err);
+    if (k2_stack_entries(n) == 0 || batch == 0) return 0;
+    // not less than for any smaller batch: a stack for every resident warp, and
+    // slots for the most items of a split batch (keldysh_chunks)
+    K2Plan p;
+    *err = k2_plan(n, batch, &p);
     if (*err) return 0;
-    return static_cast<size_t>(grid) * kK2Warps * per * sizeof(double2);
+    const int64_t warps = 152 * kK2Warps, items = batch <= warps ? warps : 9 * warps;
+    const size_t split = static_cast<size_t>(warps) * k2_stack_entries(n) * sizeof(double2) +
+                         static_cast<size_t>(items) * ((n + 1) * sizeof(double2) + 2 * sizeof(uint32_t)) + 64;
+    return p.total > split ? p.total : split;
 }
 
 int launch_keldysh2(const double *Mu, const double *Md, int n, int64_t batch, int sgn, double *sum,
                     double *partial, uint32_t *status, void *workspace, cudaStream_t s) {
-    int err = 0;
-    const int grid = keldysh2_grid(batch, &err);
+    K2Plan p;
+    const int err = k2_plan(n, batch, &p);
     if (err) return err;
-    const size_t smem = kK2Warps * sizeof(K2WarpSmem);
-    keldysh2_kernel<<<grid, kK2Warps * 32, smem, s>>>(
+    unsigned char *ws = static_cast<unsigned char *>(workspace);
+    double2 *stack = p.stack ? reinterpret_cast<double2 *>(ws) : nullptr;
+    double2 *slots = p.kc ? reinterpret_cast<double2 *>(ws + p.stack) : nullptr;
+    uint32_t *flags = p.kc ? reinterpret_cast<uint32_t *>(ws + p.stack + p.slot) : nullptr;
+    unsigned *ctr = p.kc ? reinterpret_cast<unsigned *>(ws + p.stack + p.slot + p.flag) : nullptr;
+    if (p.kc) {
+        const cudaError_t e = cudaMemsetAsync(ctr, 0, static_cast<size_t>(batch) * sizeof(unsigned), s);
+        if (e != cudaSuccess) return static_cast<int>(e);
+    }
+    keldysh2_kernel<<<p.grid, p.warps * 32, p.warps * sizeof(K2WarpSmem), s>>>(
         reinterpret_cast<const double2 *>(Mu), reinterpret_cast<const double2 *>(Md), n, batch, sgn, sum, partial,
-        status, static_cast<double2 *>(workspace), k2_stack_entries(n));
+        status, stack, k2_stack_entries(n), p.kc, slots, flags, ctr);
     return static_cast<int>(cudaGetLastError());
 }
 

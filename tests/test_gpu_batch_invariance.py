@@ -127,3 +127,23 @@ def test_fast_subset_convolution(apm, n, batch):
                    generator=torch.Generator(device="cuda").manual_seed(n))
     few = torch.as_tensor([0, 3, 455, 456, batch - 1]).cuda()
     rows_equal((apm.cdet_from_weights_fsc(w),), (apm.cdet_from_weights_fsc(w[few]),), few)
+
+
+# two-spin Keldysh sums: pairs whole or split over warps (a rounding apart), one
+# warp per CTA up to twelve, and scratch sized for a batch serving a smaller one
+@pytest.mark.parametrize("n,batch", [(7, 40), (8, 304), (8, 305), (9, 77), (10, 153), (8, 1825)])
+def test_keldysh2_splits(apm, n, batch):
+    Mu, Md = (torch.as_tensor(x).cuda() for x in I.keldysh2_batch(batch, n, seed=8600 + n))
+    Mu[3, 0, 1] = float("nan")
+    s, p, st = apm.keldysh2_sum(Mu, Md, partial=True, return_status=True)
+    few = [0, 1, 3, batch // 2, batch - 1]
+    sf, pf, stf = apm.keldysh2_sum(Mu[few], Md[few], partial=True, return_status=True)
+    assert torch.equal(st[few], stf) and int(stf[2]) == apm.ST_NONFINITE_INPUT
+    good = [i for i in few if i != 3]
+    scale = oracle.keldysh2_scale(Mu[good].cpu().numpy(), Md[good].cpu().numpy())
+    at = [k for k, i in enumerate(few) if i != 3]
+    assert np.all(np.abs((s[good] - sf[at]).cpu().numpy()) <= TOL * scale)
+    assert np.all(np.abs((p[good] - pf[at]).cpu().numpy()) <= TOL * scale[:, None])
+    assert bool(torch.isnan(s[3].real)) and bool(torch.isnan(pf[2].real).all())
+    sizes = [apm.workspace_size(apm.OP_KELDYSH2, n, b) for b in (1, 76, 152, 305, 608, 1824, 4000)]
+    assert sizes == sorted(sizes)
