@@ -164,7 +164,7 @@ __device__ __forceinline__ void node_pivot(int x, int lev, double &v, double *MA
         piv += piv >= 0.0 ? shift : -shift;
     }
     MA[x | (1 << lev)] = MA[x] * piv;
-    v = 1.0 / piv;
+    v = rcp_nr(piv);
 }
 
 // All 15 principal minors of a 4x4 matrix w (row-major) times `pre`, written to
@@ -265,7 +265,7 @@ __device__ __forceinline__ void bottom43(const double *__restrict__ w, double *M
     const bool corr = fabs(p) <= thr;
     const double C = corr ? (p >= 0.0 ? shift : -shift) : 0.0;
     const double piv = p + C;
-    const double v = 1.0 / piv;
+    const double v = rcp_nr(piv);
     const int mk = m | (1 << L);
     MA[mk] = d * p;
     const double g1 = w[4] * v, g2 = w[8] * v, g3 = w[12] * v;
@@ -377,6 +377,64 @@ __device__ __forceinline__ void fpm_tree(const double *__restrict__ Ag, int n, d
     if (nc > 0 && tid == 0) h.flags |= APM_ST_PIVOT_CORRECTED;
 }
 
+// sum over UH within H, in descending order, of c[j u UL u UH] a[S' less UL and
+// UH], four terms a step, their operands loaded a step ahead: with few warps on
+// an SM the chain of FMAs is what a set costs, not the loads before each (65536
+// rows of order 12 32.6 -> 30.0 ms, one of order 10 22.8 -> 18.7 us, against a
+// loop of one term). first (uniform over the warp): the first term is U = S', whose c[S] is still
+// zero, and is left out.
+__device__ __forceinline__ double cdet_walk(const double *c, const double *a, int j, int Sp, int UL, int H,
+                                            bool first = false) {
+    const int e0 = H & (-H), H1 = H ^ e0, e1 = H1 & (-H1), H2 = H1 ^ e1;
+    double acc = 0.0;
+    if (H1 == 0) {  // one or two terms
+        if (H && !first) acc = fma(c[j | UL | H], a[Sp ^ (UL | H)], acc);
+        return fma(c[j | UL], a[Sp ^ UL], acc);
+    }
+    int X = H2, cu = j | UL | H2, au = Sp ^ (UL | H2);
+    double c3 = c[cu | e1 | e0], a3 = a[au ^ (e1 | e0)], c2 = c[cu | e1], a2 = a[au ^ e1];
+    double c1 = c[cu | e0], a1 = a[au ^ e0], c0 = c[cu], a0 = a[au];
+    if (first) {
+        acc = fma(c0, a0, fma(c1, a1, fma(c2, a2, acc)));
+        if (X == 0) return acc;
+        X = (X - 1) & H2;
+        cu = j | UL | X;
+        au = Sp ^ (UL | X);
+        c3 = c[cu | e1 | e0], a3 = a[au ^ (e1 | e0)], c2 = c[cu | e1], a2 = a[au ^ e1];
+        c1 = c[cu | e0], a1 = a[au ^ e0], c0 = c[cu], a0 = a[au];
+    }
+    while (X) {
+        X = (X - 1) & H2;
+        cu = j | UL | X;
+        au = Sp ^ (UL | X);
+        const double d3 = c[cu | e1 | e0], b3 = a[au ^ (e1 | e0)], d2 = c[cu | e1], b2 = a[au ^ e1];
+        const double d1 = c[cu | e0], b1 = a[au ^ e0], d0 = c[cu], b0 = a[au];
+        acc = fma(c0, a0, fma(c1, a1, fma(c2, a2, fma(c3, a3, acc))));
+        c3 = d3, a3 = b3, c2 = d2, a2 = b2, c1 = d1, a1 = b1, c0 = d0, a0 = b0;
+    }
+    return fma(c0, a0, fma(c1, a1, fma(c2, a2, fma(c3, a3, acc))));
+}
+
+// one group step of a layer: lane's set S, its lanes' shares UL, the rest H
+struct CdetSet {
+    int S, j, Sp, UL, H, gl;
+};
+__device__ __forceinline__ CdetSet cdet_set(int S, int r, int lane) {
+    CdetSet q;
+    q.S = S;
+    q.j = S & (-S);
+    q.Sp = S ^ q.j;
+    q.gl = lane & ((1 << r) - 1);
+    q.UL = 0;
+    q.H = q.Sp;
+    for (int i = 0; i < r; ++i) {
+        const int bt = q.H & (-q.H);
+        q.H ^= bt;
+        if ((q.gl >> i) & 1) q.UL |= bt;
+    }
+    return q;
+}
+
 // Connected sums c[S] = init[S] - sum_{U proper subset of S'} c[{j} u U] a[S' \ U]
 // (init = a for the plain recursion) for all masks of n elements.
 __device__ __forceinline__ void cdet_layers(const double *init, const double *a, double *c, int n,
@@ -392,33 +450,16 @@ __device__ __forceinline__ void cdet_layers(const double *init, const double *a,
         const uint16_t *masks = g_popmasks + g_popoff[k];
         const int r = static_cast<int>((gsel >> (3 * k)) & 7ull);
         const int spw = 32 >> r;  // sets per warp step
-        const int gl = lane & ((1 << r) - 1);
         for (int base = warp * spw; base < cnt; base += nw * spw) {
             const int G = base + (lane >> r);
             const bool act = G < cnt;
-            const int S = masks[act ? G : cnt - 1];
-            const int j = S & (-S);
-            const int Sp = S ^ j;
-            int UL = 0, low = 0, tmp = Sp;
-            for (int i = 0; i < r; ++i) {
-                const int bt = tmp & (-tmp);
-                tmp ^= bt;
-                low |= bt;
-                if ((gl >> i) & 1) UL |= bt;
-            }
-            const int H = Sp ^ low;
-            // c[S] itself (U = Sp) is still 0 here (c[] of this layer is zeroed
-            // before the layer), so the term U = Sp adds exactly 0 and needs no test
-            double acc = 0.0;
-            int UH = H;
-            while (true) {
-                const int U = UL | UH;
-                acc = fma(c[j | U], a[Sp ^ U], acc);
-                if (UH == 0) break;
-                UH = (UH - 1) & H;
-            }
+            const CdetSet q = cdet_set(masks[act ? G : cnt - 1], r, lane);
+            // c[S] itself (U = S') is still 0 here (c[] of this layer is zeroed
+            // before the layer): the term adds exactly 0. Where a lane has the
+            // whole set it is left out, else it needs no test
+            double acc = cdet_walk(c, a, q.j, q.Sp, q.UL, q.H, r == 0);
             for (int o = (1 << r) >> 1; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-            if (act && gl == 0) c[S] = init[S] - acc;
+            if (act && q.gl == 0) c[q.S] = init[q.S] - acc;
         }
         __syncthreads();
     }
@@ -437,31 +478,13 @@ __device__ __forceinline__ void block_conv(const double *cb, const double *ab, d
         const uint16_t *masks = g_popmasks + g_popoff[k];
         const int r = static_cast<int>((gsel >> (3 * k)) & 7ull);
         const int spw = 32 >> r;
-        const int gl = lane & ((1 << r) - 1);
         for (int base = warp * spw; base < cnt; base += nw * spw) {
             const int G = base + (lane >> r);
             const bool act = G < cnt;
-            const int S = masks[act ? G : cnt - 1];
-            const int j = S & (-S);
-            const int Sp = S ^ j;
-            int UL = 0, low = 0, tmp = Sp;
-            for (int i = 0; i < r; ++i) {
-                const int bt = tmp & (-tmp);
-                tmp ^= bt;
-                low |= bt;
-                if ((gl >> i) & 1) UL |= bt;
-            }
-            const int H = Sp ^ low;
-            double sum = 0.0;
-            int UH = H;
-            while (true) {
-                const int U = UL | UH;
-                sum = fma(cb[j | U], ab[Sp ^ U], sum);
-                if (UH == 0) break;
-                UH = (UH - 1) & H;
-            }
+            const CdetSet q = cdet_set(masks[act ? G : cnt - 1], r, lane);
+            double sum = cdet_walk(cb, ab, q.j, q.Sp, q.UL, q.H);
             for (int o = (1 << r) >> 1; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
-            if (act && gl == 0) acc[S] += sum;
+            if (act && q.gl == 0) acc[q.S] += sum;
         }
     }
 }
@@ -653,31 +676,6 @@ __global__ void __launch_bounds__(256) cdet_square_kernel(const double *__restri
     *reinterpret_cast<double2 *>(slots + b * slot + t) = m;
 }
 
-// sum over UH within H, in descending order, of c[j u UL u UH] a[S' less UL and
-// UH], four terms a step, their operands loaded a step ahead: with few warps on
-// an SM the chain of FMAs is what a set costs, not the loads before each.
-__device__ __forceinline__ double cdet_walk(const double *c, const double *a, int j, int Sp, int UL, int H) {
-    const int e0 = H & (-H), H1 = H ^ e0, e1 = H1 & (-H1), H2 = H1 ^ e1;
-    double acc = 0.0;
-    if (H1 == 0) {  // one or two terms
-        if (H) acc = fma(c[j | UL | H], a[Sp ^ (UL | H)], acc);
-        return fma(c[j | UL], a[Sp ^ UL], acc);
-    }
-    int X = H2, cu = j | UL | H2, au = Sp ^ (UL | H2);
-    double c3 = c[cu | e1 | e0], a3 = a[au ^ (e1 | e0)], c2 = c[cu | e1], a2 = a[au ^ e1];
-    double c1 = c[cu | e0], a1 = a[au ^ e0], c0 = c[cu], a0 = a[au];
-    while (X) {
-        X = (X - 1) & H2;
-        cu = j | UL | X;
-        au = Sp ^ (UL | X);
-        const double d3 = c[cu | e1 | e0], b3 = a[au ^ (e1 | e0)], d2 = c[cu | e1], b2 = a[au ^ e1];
-        const double d1 = c[cu | e0], b1 = a[au ^ e0], d0 = c[cu], b0 = a[au];
-        acc = fma(c0, a0, fma(c1, a1, fma(c2, a2, fma(c3, a3, acc))));
-        c3 = d3, a3 = b3, c2 = d2, a2 = b2, c1 = d1, a1 = b1, c0 = d0, a0 = b0;
-    }
-    return fma(c0, a0, fma(c1, a1, fma(c2, a2, fma(c3, a3, acc))));
-}
-
 // first index of popcount class k in g_popmasks, from the constant bank
 __device__ __forceinline__ int cdet_popoff(int k) {
     int o = 0;
@@ -695,26 +693,6 @@ __device__ __forceinline__ void cdet_block_masks(uint16_t *pop) {
         }
         pop[t] = g_popmasks[src];
     }
-}
-
-// one group step of a layer: lane's set S, its lanes' shares UL, the rest H
-struct CdetSet {
-    int S, j, Sp, UL, H, gl;
-};
-__device__ __forceinline__ CdetSet cdet_set(int S, int r, int lane) {
-    CdetSet q;
-    q.S = S;
-    q.j = S & (-S);
-    q.Sp = S ^ q.j;
-    q.gl = lane & ((1 << r) - 1);
-    q.UL = 0;
-    q.H = q.Sp;
-    for (int i = 0; i < r; ++i) {
-        const int bt = q.H & (-q.H);
-        q.H ^= bt;
-        if ((q.gl >> i) & 1) q.UL |= bt;
-    }
-    return q;
 }
 
 // Off-diagonal contributions of the blocks with |S_H| = k. Task = (matrix,
@@ -846,7 +824,7 @@ __global__ void __launch_bounds__(kCdetThreads, 3) cdet_split_diag_kernel(const 
             for (int base = warp * spw; base < cnt; base += nw * spw) {
                 const int G = base + (lane >> r);
                 const CdetSet g = cdet_set(pop[off + (G < cnt ? G : cnt - 1)], r, lane);
-                double acc = cdet_walk(cs, a0, g.j, g.Sp, g.UL, g.H);
+                double acc = cdet_walk(cs, a0, g.j, g.Sp, g.UL, g.H, r == 0);
                 for (int o = (1 << r) >> 1; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
                 if (G < cnt && g.gl == 0) cs[g.S] = as[g.S] - acc;
             }
