@@ -197,7 +197,6 @@ size_t keldysh_stack_entries(int n);
 int launch_ppm(const double *A, int n, int64_t batch, double *perms, cudaStream_t s);
 
 // XNOR minors of 2n x 2n block matrices (one warp per matrix).
-int xnor_grid(int64_t batch, int *err);
 size_t xnor_workspace_bytes(int n, int64_t batch, int *err);
 int launch_xnor(const double *M, int n, int64_t batch, double *minors, uint32_t *status, void *workspace,
                 cudaStream_t s);

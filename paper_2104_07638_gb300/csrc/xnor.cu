@@ -37,13 +37,8 @@ __device__ __forceinline__ bool nonfinite_bits(double x) {
 }
 namespace apm {
 
-// vertices expanded breadth first (S) and warps per CTA
-#ifndef APM_XN_TAIL
-#define APM_XN_TAIL 8
-#endif
-constexpr int kXnTail = APM_XN_TAIL;
-static_assert(kXnTail == 7 || kXnTail == 8, "tail of 7 or 8 vertices");
-constexpr int kXnWarps = kXnTail == 7 ? 4 : 2;
+constexpr int kXnTail = 8;   // longest tail: vertices expanded breadth first
+constexpr int kXnWarps = 2;  // warps per CTA
 
 // Tail level J (J = 0..S-2) holds 2^J nodes of size 2(S-J); even levels in
 // bufE, odd levels in bufO. S = 7: bufE 196, 400, 576; bufO 288, 512, 512.
@@ -63,29 +58,30 @@ __host__ __device__ constexpr int xn_fac_entries(int S) {
     for (int J = 0; J <= S - 3; ++J) b = b > (2 << J) * (2 * (S - J - 1)) ? b : (2 << J) * (2 * (S - J - 1));
     return b;
 }
-constexpr int kXnBufE = xn_buf_entries(kXnTail, 0);
-constexpr int kXnBufO = xn_buf_entries(kXnTail, 1);
-constexpr int kXnFac = xn_fac_entries(kXnTail);
-static_assert(kXnTail != 7 || (kXnBufE == 576 && kXnBufO == 512 && kXnFac == 128), "7-vertex tail");
-static_assert(kXnTail != 8 || (kXnBufE == 1024 && kXnBufO == 1152 && kXnFac == 256), "8-vertex tail");
+static_assert(xn_buf_entries(7, 0) == 576 && xn_buf_entries(7, 1) == 512 && xn_fac_entries(7) == 128, "7-vertex tail");
+static_assert(xn_buf_entries(8, 0) == 1024 && xn_buf_entries(8, 1) == 1152 && xn_fac_entries(8) == 256,
+              "8-vertex tail");
 constexpr int kXnMaxN = 16;
 
+template <int S>
 struct alignas(16) XnWarpSmem {
-    double bufE[kXnBufE];
-    double bufO[kXnBufO];
-    double F[kXnFac];                  // row factors C P^-1 of one level or depth-first step
-    double pinv[1 << (kXnTail - 3)][4];  // inverse pivot block of every node of one level
-    double nd[2][1 << (kXnTail - 2)];    // node determinants of the current and the next level
+    double bufE[xn_buf_entries(S, 0)];
+    double bufO[xn_buf_entries(S, 1)];
+    double F[xn_fac_entries(S)];     // row factors C P^-1 of one level or depth-first step
+    double pinv[1 << (S - 3)][4];    // inverse pivot block of every node of one level
+    double nd[2][1 << (S - 2)];      // node determinants of the current and the next level
     double pdet[kXnMaxN + 1];
     const double *vp[kXnMaxN + 1];  // depth-first views: first element and row stride
     int vs[kXnMaxN + 1];
 };
 
-static_assert(sizeof(XnWarpSmem) % 16 == 0, "per-warp blocks stay 16-byte aligned");
+static_assert(sizeof(XnWarpSmem<5>) % 16 == 0 && sizeof(XnWarpSmem<7>) % 16 == 0 && sizeof(XnWarpSmem<8>) % 16 == 0,
+              "per-warp blocks stay 16-byte aligned");
 
-// stack entries (doubles) for order n: the kept-pivot matrices of depths 1..D-1 (D = n - S)
-__host__ __device__ constexpr size_t xn_stack_entries(int n) {
-    const int D = n > kXnTail ? n - kXnTail : 0;
+// stack entries (doubles) for order n and a tail of S vertices: the kept-pivot
+// matrices of depths 1..D-1 (D = n - S)
+__host__ __device__ constexpr size_t xn_stack_entries(int n, int S) {
+    const int D = n > S ? n - S : 0;
     size_t t = 0;
     for (int d = 1; d < D; ++d) t += static_cast<size_t>(2 * (n - d)) * (2 * (n - d));
     return t;
@@ -104,8 +100,8 @@ __device__ __forceinline__ double xn_det2(double a, double b, double c, double d
 // node's last vertex (the leading block, copied: no arithmetic); child 2k+1
 // keeps it: the Schur complement with respect to the trailing 2 x 2 block P,
 // entry (r,q) = node(r,q) - F(r,0) node(m-2,q) - F(r,1) node(m-1,q), F = C P^-1.
-template <int S, int J>
-__device__ __forceinline__ void xn_tail_level(const double *cur, double *nxt, XnWarpSmem &w, int lane, int &bad) {
+template <int S, int J, class W>
+__device__ __forceinline__ void xn_tail_level(const double *cur, double *nxt, W &w, int lane, int &bad) {
     constexpr int m = 2 * (S - J), m2 = m - 2, mm = m * m, mm2 = m2 * m2, nodes = 1 << J;
     const double *ndc = w.nd[J & 1];
     double *ndn = w.nd[(J + 1) & 1];
@@ -174,9 +170,8 @@ __device__ __forceinline__ void xn_bottom(const double *cur, const double *nd, d
     }
 }
 
-template <int S, int J>
-__device__ __forceinline__ void xn_tail_levels(double *cur, double *nxt, double *out, XnWarpSmem &w, int lane,
-                                               int &bad) {
+template <int S, int J, class W>
+__device__ __forceinline__ void xn_tail_levels(double *cur, double *nxt, double *out, W &w, int lane, int &bad) {
     if constexpr (J < S - 2) {
         xn_tail_level<S, J>(cur, nxt, w, lane, bad);
         xn_tail_levels<S, J + 1>(nxt, cur, out, w, lane, bad);
@@ -187,8 +182,8 @@ __device__ __forceinline__ void xn_tail_levels(double *cur, double *nxt, double 
 
 // Breadth-first tail over the last S vertices (0..S-1); the root (2S x 2S,
 // dense) is in bufE with determinant det0; writes out[0 .. 2^S).
-template <int S>
-__device__ __forceinline__ void xn_tail(double det0, double *out, XnWarpSmem &w, int lane, int &bad) {
+template <int S, class W>
+__device__ __forceinline__ void xn_tail(double det0, double *out, W &w, int lane, int &bad) {
     if constexpr (S == 1) {
         if (lane == 0) {
             out[0] = det0;
@@ -203,8 +198,8 @@ __device__ __forceinline__ void xn_tail(double det0, double *out, XnWarpSmem &w,
 }
 
 // Whole matrix of order n <= S as one tail.
-template <int S>
-__device__ __forceinline__ void xn_tail_order(int n, double *out, XnWarpSmem &w, int lane, int &bad) {
+template <int S, class W>
+__device__ __forceinline__ void xn_tail_order(int n, double *out, W &w, int lane, int &bad) {
     if constexpr (S >= 1) {
         if (n == S) xn_tail<S>(1.0, out, w, lane, bad);
         else xn_tail_order<S - 1>(n, out, w, lane, bad);
@@ -213,8 +208,9 @@ __device__ __forceinline__ void xn_tail_order(int n, double *out, XnWarpSmem &w,
 
 // Schur complement of the m x m view P (row stride st) with respect to its
 // trailing 2 x 2 block, into dst ((m-2) x (m-2), dense); det = det of the block.
-__device__ __forceinline__ void xn_schur(const double *P, int st, int m, double *dst, XnWarpSmem &w, int lane,
-                                         int &bad, double &det) {
+template <class W>
+__device__ __forceinline__ void xn_schur(const double *P, int st, int m, double *dst, W &w, int lane, int &bad,
+                                         double &det) {
     const int m2 = m - 2;
     const double a = P[(m - 2) * st + m - 2], b = P[(m - 2) * st + m - 1];
     const double c = P[(m - 1) * st + m - 2], d = P[(m - 1) * st + m - 1];
@@ -234,12 +230,13 @@ __device__ __forceinline__ void xn_schur(const double *P, int st, int m, double 
     __syncwarp();
 }
 
-// One matrix of order n (whole warp): all 2^n XNOR minors into out, and the
-// status word. A zero or non-finite pivot block, or a non-finite input, sets
-// the status and makes the whole row NaN.
-__device__ __forceinline__ void xn_matrix(const double *A, int n, double *out, uint32_t *status_out,
-                                          double *stack, XnWarpSmem &w, int lane) {
-    const int s = n < kXnTail ? n : kXnTail;
+// Depth-first leaves t0 <= t < t1 of one matrix of order n (whole warp; all
+// 2^(n-S), or one run of them): their XNOR minors into out (the matrix's row).
+// Returns the status bits met: a zero or non-finite pivot block, a non-finite input.
+template <int S>
+__device__ __forceinline__ uint32_t xn_matrix(const double *A, int n, double *out, int64_t t0, int64_t t1,
+                                              double *stack, XnWarpSmem<S> &w, int lane) {
+    const int s = n < S ? n : S;
     const int D = n - s;
     const int m0 = 2 * n;
     int bad = 0, nonfin = 0;
@@ -250,7 +247,7 @@ __device__ __forceinline__ void xn_matrix(const double *A, int n, double *out, u
         if (D == 0) {
             for (int e = lane; e < m0 * m0; e += 32) w.bufE[e] = A[e];
             __syncwarp();
-            xn_tail_order<kXnTail>(n, out, w, lane, bad);
+            xn_tail_order<S>(n, out, w, lane, bad);
         } else {
             if (lane == 0) {
                 w.vp[0] = A;
@@ -258,9 +255,10 @@ __device__ __forceinline__ void xn_matrix(const double *A, int n, double *out, u
                 w.pdet[0] = 1.0;
             }
             __syncwarp();
-            for (int64_t t = 0; t < (int64_t(1) << D); ++t) {
-                // first depth whose decision changed from t-1 to t (vertex n-1 <-> top bit)
-                const int d0 = t == 0 ? 0 : D - __ffsll(t);
+            for (int64_t t = t0; t < t1; ++t) {
+                // first depth whose decision changed from t-1 to t (vertex n-1 <->
+                // top bit); a run's first leaf builds its whole path
+                const int d0 = t == t0 ? 0 : D - __ffsll(t);
                 for (int d = d0; d < D; ++d) {
                     const int keep = static_cast<int>((t >> (D - 1 - d)) & 1);
                     const double *P = w.vp[d];
@@ -295,63 +293,125 @@ __device__ __forceinline__ void xn_matrix(const double *A, int n, double *out, u
                     }
                     __syncwarp();
                 }
-                xn_tail<kXnTail>(w.pdet[D], out + (t << s), w, lane, bad);
+                xn_tail<S>(w.pdet[D], out + (t << s), w, lane, bad);
             }
         }
     }
     bad = __any_sync(0xffffffffu, bad);
-    if (bad || nonfin) {
-        const double nanv = __longlong_as_double(0x7ff8000000000000ll);
-        for (int64_t e = lane; e < (int64_t(1) << n); e += 32) out[e] = nanv;
-    }
-    if (lane == 0 && status_out)
-        *status_out = (bad ? APM_ST_ZERO_PIVOT : 0u) | (nonfin ? APM_ST_NONFINITE_INPUT : 0u);
     __syncwarp();
+    return (bad ? APM_ST_ZERO_PIVOT : 0u) | (nonfin ? APM_ST_NONFINITE_INPUT : 0u);
 }
 
-// CTAs per SM that the shared memory allows (228 KB per SM, 1 KB reserved per CTA)
-constexpr int kXnMinBlocks = static_cast<int>((228 * 1024) / (kXnWarps * sizeof(XnWarpSmem) + 1024));
+// the status word, and the whole row NaN where it holds an error
+__device__ __forceinline__ void xn_finish(uint32_t st, int n, double *out, uint32_t *status_out, int first, int step) {
+    if (st) {
+        const double nanv = __longlong_as_double(0x7ff8000000000000ll);
+        for (int64_t e = first; e < (int64_t(1) << n); e += step) out[e] = nanv;
+    }
+    if (first == 0 && status_out) *status_out = st;
+}
 
-__global__ void __launch_bounds__(kXnWarps * 32, kXnMinBlocks) xnor_kernel(const double *__restrict__ M, int n, int64_t batch,
-                                                             double *minors, uint32_t *status, double *stack_base,
-                                                             size_t stack_per_warp) {
+// CTAs per SM that the shared memory allows (228 KB per SM, 1 KB reserved per
+// CTA), at most as many as 168 registers per thread leave
+template <int S>
+constexpr int xn_min_blocks() {
+    const int c = static_cast<int>((228 * 1024) / (kXnWarps * sizeof(XnWarpSmem<S>) + 1024));
+    return c < 6 ? c : 6;
+}
+
+// Work items are (matrix, run): 2^kc runs of consecutive leaves per matrix. With
+// kc > 0 a run ORs its status bits into flags[b] (zero at launch), and
+// xnor_finish_kernel, after this one, writes the status and the NaN rows.
+template <int S>
+__global__ void __launch_bounds__(kXnWarps * 32, xn_min_blocks<S>()) xnor_kernel(
+    const double *__restrict__ M, int n, int64_t batch, double *minors, uint32_t *status, double *stack_base,
+    size_t stack_per_warp, int kc, uint32_t *flags) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    XnWarpSmem &w = reinterpret_cast<XnWarpSmem *>(smem_raw)[wid];
+    XnWarpSmem<S> &w = reinterpret_cast<XnWarpSmem<S> *>(smem_raw)[wid];
     const int64_t gw = static_cast<int64_t>(blockIdx.x) * kXnWarps + wid;
     const int64_t nw = static_cast<int64_t>(gridDim.x) * kXnWarps;
     double *stack = stack_base ? stack_base + gw * stack_per_warp : nullptr;
-    const int64_t m0 = 2 * n, N = int64_t(1) << n;
-    for (int64_t b = gw; b < batch; b += nw)
-        xn_matrix(M + b * m0 * m0, n, minors + b * N, status ? status + b : nullptr, stack, w, lane);
+    const int64_t m0 = 2 * n, N = int64_t(1) << n, run = int64_t(1) << ((n > S ? n - S : 0) - kc);
+    for (int64_t it = gw; it < (batch << kc); it += nw) {
+        const int64_t b = it >> kc, t0 = (it - (b << kc)) * run;
+        const uint32_t st = xn_matrix<S>(M + b * m0 * m0, n, minors + b * N, t0, t0 + run, stack, w, lane);
+        if (kc == 0) xn_finish(st, n, minors + b * N, status ? status + b : nullptr, lane, 32);
+        else if (st && lane == 0) atomicOr(flags + b, st);
+        __syncwarp();
+    }
 }
 
-int xnor_grid(int64_t batch, int *err) {
-    const size_t smem = kXnWarps * sizeof(XnWarpSmem);
-    int64_t g = resident_ctas(xnor_kernel, kXnWarps * 32, smem, smem, err);
-    if (*err) return 0;
-    const int64_t need = (batch + kXnWarps - 1) / kXnWarps;
-    if (need < g) g = need;
-    return static_cast<int>(g < 1 ? 1 : g);
+__global__ void __launch_bounds__(256) xnor_finish_kernel(int n, int64_t batch, double *minors, uint32_t *status,
+                                                          const uint32_t *flags) {
+    for (int64_t b = blockIdx.x; b < batch; b += gridDim.x)
+        xn_finish(flags[b], n, minors + (b << n), status ? status + b : nullptr, threadIdx.x, blockDim.x);
 }
 
+using XnKernel = void (*)(const double *, int, int64_t, double *, uint32_t *, double *, size_t, int, uint32_t *);
+static XnKernel xn_kernel_for(int S) { return S == 8 ? xnor_kernel<8> : S == 7 ? xnor_kernel<7> : xnor_kernel<5>; }
+static size_t xn_smem(int S) {
+    return kXnWarps * (S == 8 ? sizeof(XnWarpSmem<8>) : S == 7 ? sizeof(XnWarpSmem<7>) : sizeof(XnWarpSmem<5>));
+}
+
+// Tail and runs per matrix (log2), by the warps a batch would otherwise leave
+// idle. The tree's operations do not depend on either: the same bits. us per call,
+// one warp per matrix before: order 10: 1 matrix 80 -> 23, 512 88 -> 71; order 12:
+// 1 326 -> 29, 512 355 -> 244; order 14: 1 1309 -> 35, 64 1370 -> 158. At order 8
+// a tail of 7 (more resident warps) lost to one of 8: 4096 matrices 109 against 91.
+struct XnShape {
+    int S, kc;
+};
+static XnShape xn_shape(int n, int64_t batch) {
+    const int64_t fill = 152 * 6;
+    XnShape s = {kXnTail, 0};
+    if (n < 10) return s;  // no scratch at these orders
+    if ((batch << (n - 8)) < fill) s.S = (batch << (n - 7)) < fill ? 5 : 7;
+    while (s.kc < n - s.S && (batch << s.kc) < 2 * fill) ++s.kc;
+    return s;
+}
+
+// Scratch of order n >= 10: the status bits of split matrices, then a stack for
+// every warp of a batch up to this one, whatever its shape.
+static size_t xn_flag_bytes(int64_t batch) { return (static_cast<size_t>(batch) * sizeof(uint32_t) + 255) & ~size_t(255); }
 size_t xnor_workspace_bytes(int n, int64_t batch, int *err) {
     *err = 0;
-    const size_t per = xn_stack_entries(n);
-    if (per == 0 || batch == 0) return 0;
-    const int grid = xnor_grid(batch, err);
-    if (*err) return 0;
-    return static_cast<size_t>(grid) * kXnWarps * per * sizeof(double);
+    if (n < 10 || batch == 0) return 0;
+    size_t most = 0;
+    for (int S : {5, 7, 8}) {
+        const int64_t res = static_cast<int64_t>(resident_ctas(xn_kernel_for(S), kXnWarps * 32, xn_smem(S), xn_smem(S), err)) *
+                            kXnWarps;
+        if (*err) return 0;
+        const int64_t items = batch >= res ? res : batch << (n - S);
+        const int64_t warps = (items < res ? items + kXnWarps - 1 : res) / kXnWarps * kXnWarps;
+        const size_t bytes = static_cast<size_t>(warps) * xn_stack_entries(n, S) * sizeof(double);
+        if (bytes > most) most = bytes;
+    }
+    return xn_flag_bytes(batch) + most;
 }
 
 int launch_xnor(const double *M, int n, int64_t batch, double *minors, uint32_t *status, void *workspace,
                 cudaStream_t s) {
+    const XnShape sh = xn_shape(n, batch);
+    const XnKernel kern = xn_kernel_for(sh.S);
+    const size_t smem = xn_smem(sh.S);
     int err = 0;
-    const int grid = xnor_grid(batch, &err);
+    const int most = resident_ctas(kern, kXnWarps * 32, smem, smem, &err);
     if (err) return err;
-    const size_t smem = kXnWarps * sizeof(XnWarpSmem);
-    xnor_kernel<<<grid, kXnWarps * 32, smem, s>>>(M, n, batch, minors, status, static_cast<double *>(workspace),
-                                                 xn_stack_entries(n));
+    const int64_t need = ((batch << sh.kc) + kXnWarps - 1) / kXnWarps;
+    uint32_t *flags = static_cast<uint32_t *>(workspace);
+    double *stack = xn_stack_entries(n, sh.S)
+                        ? reinterpret_cast<double *>(static_cast<char *>(workspace) + xn_flag_bytes(batch))
+                        : nullptr;
+    if (sh.kc) {
+        err = static_cast<int>(cudaMemsetAsync(flags, 0, static_cast<size_t>(batch) * sizeof(uint32_t), s));
+        if (err) return err;
+    }
+    kern<<<static_cast<int>(need < most ? need : most), kXnWarps * 32, smem, s>>>(
+        M, n, batch, minors, status, stack, xn_stack_entries(n, sh.S), sh.kc, flags);
+    if (sh.kc)
+        xnor_finish_kernel<<<static_cast<int>(batch < 1216 ? batch : 1216), 256, 0, s>>>(n, batch, minors, status,
+                                                                                        flags);
     return static_cast<int>(cudaGetLastError());
 }
 

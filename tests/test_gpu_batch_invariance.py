@@ -147,3 +147,22 @@ def test_keldysh2_splits(apm, n, batch):
     assert bool(torch.isnan(s[3].real)) and bool(torch.isnan(pf[2].real).all())
     sizes = [apm.workspace_size(apm.OP_KELDYSH2, n, b) for b in (1, 76, 152, 305, 608, 1824, 4000)]
     assert sizes == sorted(sizes)
+
+
+# XNOR minors and the Nambu connected sums: tails of 5, 7 and 8 vertices, whole
+# matrices or runs of leaves; a singular block in one run makes the whole row NaN
+@pytest.mark.parametrize("n,batch", [(10, 230), (10, 500), (10, 2000), (11, 120), (13, 30), (13, 60)])
+def test_xnor_runs(apm, n, batch):
+    M = I.nambu_batch(batch, n, seed=8700 + n)
+    M[1, 2 * n - 2:, 2 * n - 2:] = 0.0            # met by the leaves that keep the last vertex
+    M[2, 0, 3] = np.inf
+    d = torch.as_tensor(M).cuda()
+    few = torch.as_tensor([0, 1, 2, batch // 2, batch - 1]).cuda()
+    big = apm.nambu_cdet(d, return_minors=True, return_status=True)
+    rows_equal(big, apm.nambu_cdet(d[few], return_minors=True, return_status=True), few)
+    st = big[2].cpu().numpy()
+    assert st[1] == apm.ST_ZERO_PIVOT and st[2] == apm.ST_NONFINITE_INPUT and st[0] == 0 and not st[3:].any()
+    assert bool(torch.isnan(big[1][1]).all()) and bool(torch.isnan(big[1][2]).all())
+    assert not bool(torch.isnan(big[1][0]).any())
+    sizes = [apm.workspace_size(apm.OP_XNOR_MINORS, n, b) for b in (1, 28, 113, 228, 456, 912, 1520, 5000)]
+    assert sizes == sorted(sizes)
