@@ -470,9 +470,14 @@ __device__ __noinline__ int nd_fan_drop(const double *fd, double *fn, int fc, in
 // and corrected as described at the top. A zero or non-finite pivot, a
 // non-finite input or more corrections than the records hold set the status
 // and make the whole row NaN.
-template <bool kSum, bool kCorr>
+// kPart (first pass only): the leaves that keep exactly the upper vertices of
+// `keep` alone, 2^|keep| of them, in the order the whole walk takes them; they
+// fill their own part of the row and nothing else does (kSum: the sets that hold
+// these upper vertices). Returns 1 where the matrix is to be redone, and the
+// status bits met at bit 8, and writes no status and no NaN.
+template <bool kSum, bool kCorr, bool kPart = false>
 __device__ __forceinline__ int nd_matrix(const double *A, int n, double *out, uint32_t *status_out, double thr,
-                                         double shf, double *scratch, NdWarpSmem &w, int lane) {
+                                         double shf, double *scratch, NdWarpSmem &w, int lane, int keep = 0) {
     const int s = n < kNdTail ? n : kNdTail;
     const int D = n - s;
     const int m0 = 2 * n;
@@ -501,8 +506,10 @@ __device__ __forceinline__ int nd_matrix(const double *A, int n, double *out, ui
     const double sc = amax > 0.0 ? amax : 1.0;
     cc.thrA = thr * sc;
     cc.Cm = shf * sc;
-    if (kSum)
+    if (kSum && !kPart)
         for (int64_t e = lane; e < row; e += 32) out[e] = 0.0;
+    if (kSum && kPart)
+        for (int e = lane; e < (1 << s); e += 32) out[(static_cast<int64_t>(keep) << s) + e] = 0.0;
     if (lane == 0) {
         w.smask[0] = 0;  // depth 0: the row itself, weight 1
         w.fcnt[0] = 1;
@@ -525,10 +532,22 @@ __device__ __forceinline__ int nd_matrix(const double *A, int n, double *out, ui
             }
             __syncwarp();
             const int64_t T3 = nd_pow3(D), tail3 = nd_pow3(s);
-            for (int64_t t = 0; t < T3; ++t) {
-                // first depth whose digit changed from t-1 to t (vertex n-1 <-> top digit)
+            const int64_t count = kPart ? int64_t(1) << __popc(keep) : T3;
+            for (int64_t q = 0; q < count; ++q) {
+                // leaf t (vertex n-1 <-> top digit) and the first depth whose digit
+                // changed from the last one's: of a part, bit i of q is the type of
+                // the i-th kept vertex from the last depth up
                 int d0 = 0;
-                if (t) {
+                int64_t t = q;
+                if constexpr (kPart) {
+                    t = 0;
+                    int i = 0;
+                    for (int r = keep; r; r &= r - 1, ++i) {
+                        const int bit = __ffs(r) - 1;
+                        t += nd_pow3(bit) * (1 + ((q >> i) & 1));
+                        if (q && i == __ffsll(q) - 1) d0 = D - 1 - bit;
+                    }
+                } else if (t) {
                     int p = 0;
                     for (int64_t u = t; u % 3 == 0; u /= 3) ++p;
                     d0 = D - 1 - p;
@@ -639,6 +658,11 @@ __device__ __forceinline__ int nd_matrix(const double *A, int n, double *out, ui
     bad = __any_sync(0xffffffffu, bad);
     const int ovf = __any_sync(0xffffffffu, cc.ovf);
     const int corr = __any_sync(0xffffffffu, cc.corr);
+    if constexpr (kPart) {
+        __syncwarp();
+        return (corr && !nonfin ? 1 : 0) | (bad ? APM_ST_ZERO_PIVOT << 8 : 0) |
+               (nonfin ? APM_ST_NONFINITE_INPUT << 8 : 0);
+    }
     if (!kCorr && corr && !nonfin) return 1;  // redone by the second pass
     if (bad || nonfin || ovf) {
         const double nanv = __longlong_as_double(0x7ff8000000000000ll);
@@ -661,7 +685,7 @@ __global__ void __launch_bounds__(kNdWarps * 32, kNdMinBlocks) nand_kernel(const
                                                                          int64_t batch, double *out,
                                                                          uint32_t *status, uint32_t *flag,
                                                                          double thr, double shf, double *scratch_base,
-                                                                         size_t scratch_per_warp) {
+                                                                         size_t scratch_per_warp, int parts) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     NdWarpSmem &w = reinterpret_cast<NdWarpSmem *>(smem_raw)[wid];
@@ -671,11 +695,57 @@ __global__ void __launch_bounds__(kNdWarps * 32, kNdMinBlocks) nand_kernel(const
     const int64_t m0 = 2 * n;
     const int64_t row = kSum ? (int64_t(1) << n) : static_cast<int64_t>(nd_pow3(n));
     for (int64_t b = gw; b < batch; b += nw) {
-        if (kCorr && flag[b] == 0u) continue;
+        if (kCorr && (flag[b] & 1u) == 0u) {
+            // (of a first pass in parts) the status bits its parts met
+            const uint32_t st = flag[b] >> 8;
+            if (parts && lane == 0 && status) status[b] = st;
+            if (st)
+                for (int64_t e = lane; e < row; e += 32) out[b * row + e] = __longlong_as_double(0x7ff8000000000000ll);
+            continue;
+        }
         const int redo = nd_matrix<kSum, kCorr>(M + b * m0 * m0, n, out + b * row, status ? status + b : nullptr,
                                                 thr, shf, scratch, w, lane);
         if (!kCorr && lane == 0) flag[b] = static_cast<uint32_t>(redo);
     }
+}
+
+// First pass of few matrices: a warp takes the leaves of one kept set of the
+// upper vertices (the largest sets first), so that a matrix's 3^(n-6) leaves are
+// 2^(n-6) warps' work. flag[b] (zero at launch) collects the parts' answers.
+template <bool kSum>
+__global__ void __launch_bounds__(kNdWarps * 32, kNdMinBlocks) nand_parts_kernel(
+    const double *__restrict__ M, int n, int64_t batch, double *out, uint32_t *flag, double thr, double shf,
+    double *scratch_base, size_t scratch_per_warp) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    NdWarpSmem &w = reinterpret_cast<NdWarpSmem *>(smem_raw)[wid];
+    const int64_t gw = static_cast<int64_t>(blockIdx.x) * kNdWarps + wid;
+    const int64_t nw = static_cast<int64_t>(gridDim.x) * kNdWarps;
+    double *scratch = scratch_base + gw * scratch_per_warp;
+    const int64_t m0 = 2 * n;
+    const int64_t row = kSum ? (int64_t(1) << n) : static_cast<int64_t>(nd_pow3(n));
+    const int sets = 1 << (n - kNdTail);
+    for (int64_t it = gw; it < batch * sets; it += nw) {
+        const int64_t b = it % batch;
+        const int keep = sets - 1 - static_cast<int>(it / batch);
+        const int r = nd_matrix<kSum, false, true>(M + b * m0 * m0, n, out + b * row, nullptr, thr, shf, scratch, w,
+                                                   lane, keep);
+        if (r && lane == 0) atomicOr(flag + b, static_cast<uint32_t>(r));
+        __syncwarp();
+    }
+}
+
+// Whether the first pass runs in parts (the bits are the same either way). They
+// fill a partial round of the 1824 resident warps and balance it, and cost a path
+// each: us per two-type call, whole | parts,
+//   n = 7: 600 matrices 50 | 44, 1000 58 | 62, 2400 110 | 104, 3000 118 | 123
+//   n = 8: 1 112 | 65, 1000 140 | 130, 1500 157 | 172, 2400 287 | 258, 3600 331 | 345
+//   n = 10: 1 849 | 215, 300 863 | 401, 1000 1115 | 973; n = 12: 4096 32440 | 34148
+constexpr int64_t kNdWhole = 4096;  // larger batches are never in parts
+static bool nand_parts(int n, int64_t batch) {
+    const int64_t round = 6 * 2 * 152, r = batch % round;
+    if (n <= kNdTail || batch > kNdWhole || (batch > round && n > 9)) return false;
+    return r > 0 && r < (n == 7 ? 800 : 1150);
 }
 
 int nand_grid(int64_t batch, int *err) {
@@ -689,6 +759,7 @@ int nand_grid(int64_t batch, int *err) {
     *err = 0;
     fits(nand_kernel<false, false>), fits(nand_kernel<false, true>);
     fits(nand_kernel<true, false>), fits(nand_kernel<true, true>);
+    fits(nand_parts_kernel<false>), fits(nand_parts_kernel<true>);
     if (*err) return 0;
     const int64_t need = (batch + kNdWarps - 1) / kNdWarps;
     if (need < g) g = need;
@@ -696,36 +767,53 @@ int nand_grid(int64_t batch, int *err) {
 }
 
 // per resident warp the stack and correction records, then one flag per matrix
+// Scratch: per resident warp the stack and the correction records (as many warps
+// as the parts of the largest batch in parts, or this batch, can occupy), then the
+// flags.
+static int64_t nand_warps(int n, int64_t batch, int *err) {
+    const int64_t parts = n > kNdTail ? batch << (n - kNdTail) : batch;
+    return static_cast<int64_t>(nand_grid(batch > kNdWhole ? INT64_MAX / 64 : parts, err)) * kNdWarps;
+}
 size_t nand_workspace_bytes(int n, int64_t batch, int *err) {
     *err = 0;
     if (batch == 0) return 0;
-    const int grid = nand_grid(batch, err);
+    const int64_t warps = nand_warps(n, batch, err);
     if (*err) return 0;
-    return static_cast<size_t>(grid) * kNdWarps * nd_warp_doubles(n) * sizeof(double) +
+    return static_cast<size_t>(warps) * nd_warp_doubles(n) * sizeof(double) +
            ((static_cast<size_t>(batch) * sizeof(uint32_t) + 15) & ~static_cast<size_t>(15));
+}
+
+template <bool kSum>
+static int nand_run(const double *M, int n, int64_t batch, double *out, double thr, double shf, uint32_t *status,
+                    double *scratch, uint32_t *flag, cudaStream_t s) {
+    int err = 0;
+    const size_t smem = kNdWarps * sizeof(NdWarpSmem), per = nd_warp_doubles(n);
+    const int grid = nand_grid(batch, &err);
+    if (err) return err;
+    const bool parts = nand_parts(n, batch);
+    if (parts) {
+        const int g = nand_grid(batch << (n - kNdTail), &err);
+        if (!err) err = static_cast<int>(cudaMemsetAsync(flag, 0, static_cast<size_t>(batch) * sizeof(uint32_t), s));
+        if (err) return err;
+        nand_parts_kernel<kSum><<<g, kNdWarps * 32, smem, s>>>(M, n, batch, out, flag, thr, shf, scratch, per);
+    } else {
+        nand_kernel<kSum, false><<<grid, kNdWarps * 32, smem, s>>>(M, n, batch, out, status, flag, thr, shf, scratch,
+                                                                   per, 0);
+    }
+    nand_kernel<kSum, true><<<grid, kNdWarps * 32, smem, s>>>(M, n, batch, out, status, flag, thr, shf, scratch, per,
+                                                              parts ? 1 : 0);
+    return static_cast<int>(cudaGetLastError());
 }
 
 int launch_nand(const double *M, int n, int64_t batch, double *out, bool type_sums, double thr, double shf,
                 uint32_t *status, void *workspace, cudaStream_t s) {
     int err = 0;
-    const int grid = nand_grid(batch, &err);
-    if (err) return err;
-    const size_t smem = kNdWarps * sizeof(NdWarpSmem);
     double *scratch = static_cast<double *>(workspace);
-    const size_t per = nd_warp_doubles(n);
-    uint32_t *flag = reinterpret_cast<uint32_t *>(scratch + static_cast<size_t>(grid) * kNdWarps * per);
-    if (type_sums) {
-        nand_kernel<true, false><<<grid, kNdWarps * 32, smem, s>>>(M, n, batch, out, status, flag, thr, shf,
-                                                                   scratch, per);
-        nand_kernel<true, true><<<grid, kNdWarps * 32, smem, s>>>(M, n, batch, out, status, flag, thr, shf,
-                                                                  scratch, per);
-    } else {
-        nand_kernel<false, false><<<grid, kNdWarps * 32, smem, s>>>(M, n, batch, out, status, flag, thr, shf,
-                                                                    scratch, per);
-        nand_kernel<false, true><<<grid, kNdWarps * 32, smem, s>>>(M, n, batch, out, status, flag, thr, shf,
-                                                                   scratch, per);
-    }
-    return static_cast<int>(cudaGetLastError());
+    const int64_t warps = nand_warps(n, batch, &err);
+    if (err) return err;
+    uint32_t *flag = reinterpret_cast<uint32_t *>(scratch + static_cast<size_t>(warps) * nd_warp_doubles(n));
+    return type_sums ? nand_run<true>(M, n, batch, out, thr, shf, status, scratch, flag, s)
+                     : nand_run<false>(M, n, batch, out, thr, shf, status, scratch, flag, s);
 }
 
 }  // namespace apm

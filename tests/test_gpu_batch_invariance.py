@@ -166,3 +166,25 @@ def test_xnor_runs(apm, n, batch):
     assert not bool(torch.isnan(big[1][0]).any())
     sizes = [apm.workspace_size(apm.OP_XNOR_MINORS, n, b) for b in (1, 28, 113, 228, 456, 912, 1520, 5000)]
     assert sizes == sorted(sizes)
+
+
+# two vertex types: the first pass whole (large batches) or by kept sets of the
+# upper vertices, with a small pivot (redone), a singular and a non-finite matrix
+@pytest.mark.parametrize("n,batch", [(7, 900), (7, 2500), (8, 1500), (9, 60), (10, 33)])
+def test_two_type_parts(apm, n, batch):
+    M = I.two_type_batch(batch, n, seed=8800 + n)
+    M[1][np.diag_indices(2 * n)] = 0.0
+    M[2, 1, 2] = np.inf
+    M[4, 2 * n - 1, 2 * n - 1] = 0.0
+    d = torch.as_tensor(M).cuda()
+    few = torch.as_tensor([0, 1, 2, 3, 4, batch // 2, batch - 1]).cuda()
+    for kw in ({}, {"piv_shift": 0.0}):          # no shift leaves a zero pivot flagged
+        big = apm.two_type_cdet(d, return_weights=True, return_status=True, **kw)
+        rows_equal(big, apm.two_type_cdet(d[few], return_weights=True, return_status=True, **kw), few)
+        st = big[2].cpu().numpy()
+        assert st[2] == apm.ST_NONFINITE_INPUT and bool(torch.isnan(big[1][2]).all()) and st[0] == 0
+        assert (st[1] & apm.ST_ZERO_PIVOT) if kw else (st[1] & apm.ST_PIVOT_CORRECTED)
+    if n <= 8:
+        rows_equal(apm.nand_minors(d, return_status=True), apm.nand_minors(d[few], return_status=True), few)
+    sizes = [apm.workspace_size(apm.OP_TWO_TYPE_CDET, n, b) for b in (1, 100, 1000, 4096, 4097, 20000)]
+    assert sizes == sorted(sizes)
