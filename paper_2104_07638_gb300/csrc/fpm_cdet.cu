@@ -87,6 +87,7 @@ struct VarlenParams {
     unsigned *ctr;                 // work counter, zeroed by varlen_order_kernel
     int smem_max_n;
     int n_max;
+    int split_to;                  // unflagged items of orders smem_max_n + 1 .. split_to are done elsewhere
     unsigned long long gsel[17];   // lane-group table per order
 };
 
@@ -662,18 +663,45 @@ __global__ void __launch_bounds__(kCdetThreads, 3) fpm_cdet_kernel(const CdetKer
 // output row, then the diagonal recursion of every block. Each mask's terms are
 // added in the order of cdet_blocked: the results are the same bits.
 
+// The matrices of such a launch: `batch` fixed-order ones (weights a + i astride,
+// sums c + (i << n)), or the items order[*first + i], i < *count, of one order of
+// an uneven batch (sums c + c_off[item]) less the flagged ones, which its
+// persistent kernel takes.
+struct SplitArgs {
+    const double *a;
+    size_t astride;
+    double *c;
+    const int *order;
+    const int64_t *c_off;
+    const unsigned *first, *count;
+    const uint8_t *flag;
+    double *rows;  // scratch rows of 2^kBlkB doubles, `cap` of them
+    int64_t cap, batch;
+    int n;
+    unsigned long long gsel;
+    __device__ __forceinline__ int64_t items() const { return order ? static_cast<int64_t>(*count) : batch; }
+    __device__ __forceinline__ int64_t item(int64_t i) const { return order ? order[static_cast<int64_t>(*first) + i] : i; }
+    __device__ __forceinline__ bool skip(int64_t i) const { return order && flag[item(i)]; }
+    __device__ __forceinline__ double *out(int64_t i) const { return order ? c + c_off[item(i)] : c + (i << n); }
+    // whether the terms of level k get a row per T_H
+    __device__ __forceinline__ bool in_rows(int64_t blocks, int k) const {
+        return rows && blocks * ((1 << k) - 1) <= cap;
+    }
+};
+
 // Weights of the matrices the warp-per-matrix kernel has not flagged, from
-// their minors (rows of 2^n doubles) into the slots' first 2^n doubles.
-__global__ void __launch_bounds__(256) cdet_square_kernel(const double *__restrict__ minors,
-                                                          const uint8_t *__restrict__ flag, double *slots,
-                                                          size_t slot, int n, int64_t batch, int single) {
-    const int64_t pairs = int64_t(1) << (n - 1);
-    const int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x, b = i >> (n - 1);
-    if (b >= batch || flag[b]) return;
-    const int64_t t = 2 * (i & (pairs - 1));
-    double2 m = *reinterpret_cast<const double2 *>(minors + (b << n) + t);
-    if (!single) m = make_double2(m.x * m.x, m.y * m.y);
-    *reinterpret_cast<double2 *>(slots + b * slot + t) = m;
+// their minors (rows laid out as the sums) into the rows of P.a.
+__global__ void __launch_bounds__(256) cdet_square_kernel(const SplitArgs P, const double *__restrict__ minors,
+                                                          const uint8_t *__restrict__ flag, int single) {
+    const int64_t pairs = int64_t(1) << (P.n - 1), all = P.items() << (P.n - 1);
+    for (int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; i < all;
+         i += static_cast<int64_t>(gridDim.x) * blockDim.x) {
+        const int64_t b = i >> (P.n - 1), t = 2 * (i & (pairs - 1));
+        if (flag[P.item(b)]) continue;
+        double2 m = *reinterpret_cast<const double2 *>(minors + (P.out(b) - P.c) + t);
+        if (!single) m = make_double2(m.x * m.x, m.y * m.y);
+        *reinterpret_cast<double2 *>(const_cast<double *>(P.a) + b * P.astride + t) = m;
+    }
 }
 
 // first index of popcount class k in g_popmasks, from the constant bank
@@ -698,27 +726,33 @@ __device__ __forceinline__ void cdet_block_masks(uint16_t *pop) {
 // Off-diagonal contributions of the blocks with |S_H| = k. Task = (matrix,
 // block, part); the warps of a block's parts take the set groups of all layers
 // in turn, and the next T_H's operand blocks arrive while the current ones are
-// used; the sums go to the block's place in the rows of c. With `rows` (few
-// matrices) a task is one T_H alone instead, (matrix, block, T_H, part), and its
+// used; the sums go to the block's place in the rows of c. Of few matrices
+// (in_rows) a task is one T_H alone instead, (matrix, block, T_H, part), and its
 // terms go to a row of their own, which the diagonal launch adds in T_H's order.
-__global__ void __launch_bounds__(kCdetThreads, 3) cdet_split_conv_kernel(const double *__restrict__ a, size_t astride,
-                                                                       double *c, int n, int64_t batch, int k,
-                                                                       int lparts, double *rows,
-                                                                       unsigned long long gsel) {
+// As many parts as give every resident CTA a task.
+__global__ void __launch_bounds__(kCdetThreads, 3) cdet_split_conv_kernel(const SplitArgs P, int k) {
     constexpr int b = kBlkB, NB = 1 << kBlkB;
     __shared__ __align__(16) double cb[2][NB], ab[2][NB], acc[NB];
     __shared__ uint16_t pop[NB];
     const int tid = threadIdx.x, T = blockDim.x, lane = tid & 31;
-    const int h = n - b, nblk = c_binom[h][k], pk = cdet_popoff(k);
+    const int n = P.n, h = n - b, nblk = c_binom[h][k], pk = cdet_popoff(k);
+    const int64_t blocks = P.items() * nblk;
+    const bool in_rows = P.in_rows(blocks, k);
+    const int nth = in_rows ? (1 << k) - 1 : 1;
+    int lparts = 0;
+    while (lparts < (in_rows ? 2 : 3) && (blocks * nth << lparts) < (in_rows ? 152 : 6 * 152)) ++lparts;
     const int parts = 1 << lparts, W = (T >> 5) << lparts;
+    double *const rows = in_rows ? P.rows : nullptr;
+    const unsigned long long gsel = P.gsel;
+    if (blockIdx.x >= (blocks * nth) << lparts) return;
     cdet_block_masks(pop);
-    const int nth = rows ? (1 << k) - 1 : 1;
-    for (int64_t task = blockIdx.x; task < (batch * nblk * nth) << lparts; task += gridDim.x) {
+    for (int64_t task = blockIdx.x; task < (blocks * nth) << lparts; task += gridDim.x) {
         const int part = static_cast<int>(task & (parts - 1));
         const int64_t row = task >> lparts, mb = row / nth, mat = mb / nblk;
+        if (P.skip(mat)) continue;
         const int SH = g_popmasks[pk + static_cast<int>(mb - mat * nblk)], jH = SH & (-SH);
-        const double *am = a + mat * astride;
-        double *cm = c + (mat << n);
+        const double *am = P.a + mat * P.astride;
+        double *cm = P.out(mat);
         const int wg = part * (T >> 5) + (tid >> 5);
         // f(first lane's set) for the sets of this warp, in every layer
         auto sets = [&](auto &&f) {
@@ -774,23 +808,24 @@ __global__ void __launch_bounds__(kCdetThreads, 3) cdet_split_conv_kernel(const 
     }
 }
 
-// The diagonal recursion of the blocks with |S_H| = k, one CTA each; rows: the
-// T_H's terms, one row each, or NULL where the block's place in c holds their sum.
-__global__ void __launch_bounds__(kCdetThreads, 3) cdet_split_diag_kernel(const double *__restrict__ a, size_t astride,
-                                                                       double *c, int n, int64_t batch, int k,
-                                                                       const double *__restrict__ rows,
-                                                                       unsigned long long gsel) {
+// The diagonal recursion of the blocks with |S_H| = k, one CTA each.
+__global__ void __launch_bounds__(kCdetThreads, 3) cdet_split_diag_kernel(const SplitArgs P, int k) {
     constexpr int b = kBlkB, NB = 1 << kBlkB;
     __shared__ __align__(16) double cs[NB], as[NB], a0[NB];
     __shared__ uint16_t pop[NB];
     const int tid = threadIdx.x, T = blockDim.x, lane = tid & 31, warp = tid >> 5, nw = T >> 5;
-    const int nblk = c_binom[n - b][k], pk = cdet_popoff(k);
+    const int nblk = c_binom[P.n - b][k], pk = cdet_popoff(k);
+    const int64_t blocks = P.items() * nblk;
+    const double *const rows = P.in_rows(blocks, k) ? P.rows : nullptr;
+    const unsigned long long gsel = P.gsel;
+    if (blockIdx.x >= blocks) return;
     cdet_block_masks(pop);
-    for (int64_t task = blockIdx.x; task < batch * nblk; task += gridDim.x) {
+    for (int64_t task = blockIdx.x; task < blocks; task += gridDim.x) {
         const int64_t mat = task / nblk;
+        if (P.skip(mat)) continue;
         const int SH = g_popmasks[pk + static_cast<int>(task - mat * nblk)];
-        const double *am = a + mat * astride;
-        double *out = c + (mat << n) + (static_cast<size_t>(SH) << b);
+        const double *am = P.a + mat * P.astride;
+        double *cm = P.out(mat), *out = cm + (static_cast<size_t>(SH) << b);
         for (int t = tid; t < NB; t += T) {
             a0[t] = t ? am[t] : 1.0;
             double sum = 0.0;
@@ -808,7 +843,6 @@ __global__ void __launch_bounds__(kCdetThreads, 3) cdet_split_diag_kernel(const 
                         if (i + e < (1 << k) - 1) sum += v[e];
                 }
             } else if (SH) {
-                const double *cm = c + (mat << n);
                 for (int TH = (SH - 1) & SH; TH; TH = (TH - 1) & SH)
                     if (TH & SH & -SH)
                         sum = fma(cm[static_cast<size_t>(TH) << b], am[static_cast<size_t>(SH ^ TH) << b], sum);
@@ -858,6 +892,7 @@ __global__ void __launch_bounds__(kCdetThreads, 3) fpm_cdet_varlen_kernel(const 
             if (threadIdx.x == 0 && p.status) p.status[b] = APM_ST_BAD_ORDER;
             continue;
         }
+        if (n > V.smem_max_n && n <= V.split_to && !p.wflag[b]) continue;
         const int N = 1 << n;
         const int NC = N > 16 ? N : 16;
         const bool in_smem = n <= V.smem_max_n;
@@ -1070,25 +1105,16 @@ int ensure_tables() {
     return 0;
 }
 
-// The recursion above order 12 with every matrix's blocks on many CTAs: a (rows
-// astride doubles apart) -> c; rows: cdet_split_rows rows of scratch.
-static int launch_cdet_split(const double *a, size_t astride, double *c, int n, int64_t batch, double *rows,
-                             unsigned long long gsel_b, cudaStream_t s) {
-    const int h = n - kBlkB;
-    const int64_t round = 3 * 152;  // resident CTAs of either kernel
+// The recursion above order 12 with every matrix's blocks on many CTAs, for at
+// most `most` matrices.
+static int launch_cdet_split(const SplitArgs &P, int64_t most, cudaStream_t s) {
+    const int h = P.n - kBlkB;
+    const int64_t ctas = 8 * 3 * 152;
     for (int k = 0, nblk = 1; k <= h; nblk = nblk * (h - k) / (k + 1), ++k) {
-        const int64_t tasks = batch * nblk, pairs = tasks * ((1 << k) - 1);
-        double *rk = pairs <= cdet_split_rows(n, batch) ? rows : nullptr;
-        if (k) {
-            int lparts = 0;
-            const int64_t each = rk ? pairs : tasks;
-            while (lparts < (rk ? 2 : 3) && (each << lparts) < (rk ? 152 : 2 * round)) ++lparts;
-            const int64_t g = each << lparts;
-            cdet_split_conv_kernel<<<static_cast<int>(g < 8 * round ? g : 8 * round), kCdetThreads, 0, s>>>(
-                a, astride, c, n, batch, k, lparts, rk, gsel_b);
-        }
-        cdet_split_diag_kernel<<<static_cast<int>(tasks < 8 * round ? tasks : 8 * round), kCdetThreads, 0, s>>>(
-            a, astride, c, n, batch, k, rk, gsel_b);
+        const int64_t blocks = most * nblk, tasks = blocks * 8 * (k < 4 ? 1 << k : 16);  // at least as many as there are
+        if (k)
+            cdet_split_conv_kernel<<<static_cast<int>(tasks < ctas ? tasks : ctas), kCdetThreads, 0, s>>>(P, k);
+        cdet_split_diag_kernel<<<static_cast<int>(blocks < ctas ? blocks : ctas), kCdetThreads, 0, s>>>(P, k);
     }
     return static_cast<int>(cudaGetLastError());
 }
@@ -1141,24 +1167,32 @@ int launch_fpm_cdet(const CdetArgs &a, cudaStream_t s) {
         }
         if (err || !rest) return err;
         const size_t slot = slot_doubles(a.n), row = size_t(1) << a.n, mats = a.two_mats ? 2 : 1;
-        double *rows = a.gscratch + grid * slot, *c = a.c_out + b0 * row;
-        if (a.mode == kModeWeights) return launch_cdet_split(a.a_in + b0 * row, row, c, a.n, rest, rows, P.gsel_b, s);
+        SplitArgs Q = {};
+        Q.c = a.c_out + b0 * row;
+        Q.rows = a.gscratch + grid * slot;
+        Q.cap = cdet_split_rows(a.n, rest);
+        Q.batch = rest;
+        Q.n = a.n;
+        Q.gsel = P.gsel_b;
+        Q.a = a.mode == kModeWeights ? a.a_in + b0 * row : a.gscratch;
+        Q.astride = a.mode == kModeWeights ? row : slot;
+        if (a.mode == kModeWeights) return launch_cdet_split(Q, rest, s);
         P.a.batch = rest;
         P.a.weights_only = 1;
         P.a.A_up += b0 * a.n * a.n;
         if (a.A_dn) P.a.A_dn += b0 * a.n * a.n;
-        P.a.c_out = c;
+        P.a.c_out = Q.c;
         if (a.minors_out) P.a.minors_out += b0 * row * mats;
         if (a.status) P.a.status += b0;
         if (a.wflag) {
             P.a.wflag += b0;
             cdet_square_kernel<<<static_cast<int>(((rest << (a.n - 1)) + 255) / 256), 256, 0, s>>>(
-                a.minors_out ? P.a.minors_out : c, P.a.wflag, a.gscratch, slot, a.n, rest, a.single_det);
+                Q, a.minors_out ? P.a.minors_out : Q.c, P.a.wflag, a.single_det);
         }
         fpm_cdet_kernel<false><<<static_cast<int>(rest), kCdetThreads, smem, s>>>(P);
         err = static_cast<int>(cudaGetLastError());
         if (err) return err;
-        return launch_cdet_split(a.gscratch, slot, c, a.n, rest, rows, P.gsel_b, s);
+        return launch_cdet_split(Q, rest, s);
     }
     if (smem_arrays)
         fpm_cdet_kernel<true><<<grid, cdet_threads(a.n, a.batch), smem, s>>>(P);
@@ -1180,6 +1214,13 @@ constexpr int kVarlenSmemMaxN = 12;
 // and the arrays of its largest order rather than of order 12 (4096 walkers of
 // orders 4..9: 201 -> 156 us).
 static int varlen_threads(int n_max) { return n_max <= 9 ? 64 : n_max <= 11 ? 128 : kCdetThreads; }
+// Largest uneven batch whose items of orders 13..15 go by blocks on many CTAs: a
+// CTA takes 4 ms for one of order 15 by itself, which is the whole call then
+// (300 walkers of orders 4..14 1672 -> 818 us, 100 of 10..16 3872 -> 1764, 1000 of
+// 4..16 9174 -> 5078).
+// Their weights, 2^15 doubles each at most, fit the region of the slots (456 x 3
+// times the largest order's).
+constexpr int64_t kVarlenSplitMax = 1024;
 static int varlen_smem_n(int n_max) { return n_max < kVarlenSmemMaxN ? n_max : kVarlenSmemMaxN; }
 
 static size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
@@ -1210,29 +1251,38 @@ static int warp_route_from(int n_max, bool two_mats) {
 
 // Workspace of an uneven batch: [counter 256 B][order: batch int32]
 // [flags of the warp-kernel minors: batch bytes, with orders >= 13 of one
-// matrix per item][per-CTA slots; the same region holds the warp kernel's
-// stacks before and the ranked arrays after the persistent kernel]
-size_t cdet_varlen_workspace(int n_max, int64_t batch, bool two_mats, int *err) {
-    size_t bytes = 256 + align256(static_cast<size_t>(batch) * sizeof(int));
-    if (n_max > kVarlenSmemMaxN) {
-        const int grid = cdet_varlen_grid(n_max, two_mats, err);
-        if (*err) return 0;
-        size_t slots = static_cast<size_t>(grid) * slot_doubles(n_max) * sizeof(double);
-        if (n_max >= g_fsc_from_n) {  // the same region then holds the ranked arrays
-            const size_t f = fsc_workspace_bytes(n_max, batch, err);
-            if (*err) return 0;
-            if (f > slots) slots = f;
-        }
-        if (warp_route_from(n_max, two_mats)) {
-            const size_t st = fpm_warp_route_stack_bytes(n_max, batch, err);
-            if (*err) return 0;
-            if (st > slots) slots = st;
-            bytes += align256(static_cast<size_t>(batch));
-        }
-        bytes += slots;
-    } else {
-        *err = 0;
+// matrix per item][varlen_region][rows of terms of the items done by blocks]
+// Doubles of the region that holds the CTAs' slots, and before and after them the
+// warp kernel's stacks, the weights of the items done by blocks and the ranked arrays.
+static int varlen_region(int n_max, int64_t batch, bool two_mats, int grid, size_t *doubles) {
+    int err = 0;
+    size_t bytes = static_cast<size_t>(grid) * slot_doubles(n_max) * sizeof(double);
+    if (n_max >= g_fsc_from_n) {
+        const size_t f = fsc_workspace_bytes(n_max, batch, &err);
+        if (err) return err;
+        if (f > bytes) bytes = f;
     }
+    if (warp_route_from(n_max, two_mats)) {
+        const size_t st = fpm_warp_route_stack_bytes(n_max, batch, &err);
+        if (err) return err;
+        if (st > bytes) bytes = st;
+    }
+    *doubles = align256(bytes) / sizeof(double);
+    return 0;
+}
+
+size_t cdet_varlen_workspace(int n_max, int64_t batch, bool two_mats, int *err) {
+    *err = 0;
+    size_t bytes = 256 + align256(static_cast<size_t>(batch) * sizeof(int));
+    if (n_max <= kVarlenSmemMaxN) return bytes;
+    const int grid = cdet_varlen_grid(n_max, two_mats, err);
+    if (*err) return 0;
+    size_t region = 0;
+    *err = varlen_region(n_max, batch, two_mats, grid, &region);
+    if (*err) return 0;
+    bytes += region * sizeof(double);
+    if (warp_route_from(n_max, two_mats))
+        bytes += align256(static_cast<size_t>(batch)) + static_cast<size_t>(kSplitMaxRows << kBlkB) * sizeof(double);
     return bytes;
 }
 
@@ -1271,8 +1321,41 @@ int launch_cdet_varlen(const CdetArgs &a, const int64_t *a_off, const int *n_arr
         err = launch_fpm_warp_route(a.A_up, m, a.batch, a.minors_out ? a.minors_out : a.c_out, a.piv_thr, wflag,
                                     a.status, slots, order, a_off, c_off, ctr + 2 + 2 * m, ctr + 3 + 2 * m, s);
     if (err) return err;
+    // few items: those of orders 13..15 by blocks on many CTAs, one order after
+    // the other, their weights in the slots' region (the persistent kernel, which
+    // takes it over after them, finds only the flagged ones of these orders)
+    int split_to = 0;
+    size_t region = 0;  // of the slots, in doubles; the rows of terms come after it
+    if (wfrom) {
+        err = varlen_region(n_max, a.batch, two, grid, &region);
+        if (err) return err;
+    }
+    const int to = n_max < fsc_from ? n_max : fsc_from - 1;
+    if (wfrom && a.batch <= kVarlenSplitMax && static_cast<size_t>(a.batch) << to <= region) {
+        split_to = to;
+        SplitArgs Q = {};
+        Q.a = slots;
+        Q.c = a.c_out;
+        Q.order = order;
+        Q.c_off = c_off;
+        Q.flag = wflag;
+        Q.rows = slots + region;
+        Q.cap = kSplitMaxRows;
+        Q.batch = a.batch;
+        Q.gsel = cdet_gsel_packed(kBlkB);
+        for (int m = split_to; m > kVarlenSmemMaxN; --m) {
+            Q.n = m;
+            Q.astride = size_t(1) << m;
+            Q.first = ctr + 2 + 2 * m;
+            Q.count = ctr + 3 + 2 * m;
+            cdet_square_kernel<<<8 * 152, 256, 0, s>>>(Q, a.minors_out ? a.minors_out : a.c_out, wflag, a.single_det);
+            err = launch_cdet_split(Q, a.batch, s);
+            if (err) return err;
+        }
+    }
     VarlenParams V;
     V.a = a;
+    V.split_to = split_to;
     V.a.wflag = wflag;
     V.a.warp_from_n = wfrom;
     V.a.gscratch = n_max > kVarlenSmemMaxN ? slots : nullptr;

@@ -188,3 +188,36 @@ def test_two_type_parts(apm, n, batch):
         rows_equal(apm.nand_minors(d, return_status=True), apm.nand_minors(d[few], return_status=True), few)
     sizes = [apm.workspace_size(apm.OP_TWO_TYPE_CDET, n, b) for b in (1, 100, 1000, 4096, 4097, 20000)]
     assert sizes == sorted(sizes)
+
+
+# an uneven batch of few items (orders 13..15 by blocks on many CTAs), of many, and
+# fixed-order calls of the same matrices, with flagged ones among them
+def test_uneven_few_and_many(apm):
+    rng = np.random.default_rng(8900)
+    few = np.concatenate([[15, 13, 16, 14, 15, 13, 14], rng.integers(4, 17, 60)]).astype(np.int32)
+    many = np.concatenate([few, rng.integers(4, 13, 1100)]).astype(np.int32)
+    flat, off = I.hubbard_varlen(many, seed=8901)
+    flat[off[1]:off[1] + 169] = 0.0                     # redone with corrections
+    flat[off[3]] = np.nan                               # non-finite
+    A, ao, nt = (torch.as_tensor(x).cuda() for x in (flat, off, many))
+    cm, mm, sm = apm.cdet_connected_varlen(A, ao, nt, return_minors=True, return_status=True)
+    cf, mf, sf = apm.cdet_connected_varlen(A, ao[:few.size].contiguous(), nt[:few.size].contiguous(),
+                                           return_minors=True, return_status=True)
+    assert np.array_equal(cm[:cf.numel()].cpu().numpy(), cf.cpu().numpy(), equal_nan=True)
+    assert np.array_equal(mm[:mf.numel()].cpu().numpy(), mf.cpu().numpy(), equal_nan=True)
+    assert torch.equal(sm[:few.size], sf)
+    assert int(sf[1]) & apm.ST_PIVOT_CORRECTED and int(sf[3]) & apm.ST_NONFINITE_INPUT
+    c0 = apm.cdet_connected_varlen(A, ao[:few.size].contiguous(), nt[:few.size].contiguous())
+    assert np.array_equal(c0.cpu().numpy(), cf.cpu().numpy(), equal_nan=True)
+    row = np.concatenate([[0], np.cumsum(1 << few.astype(np.int64))])
+    for b in range(7):
+        n = int(few[b])
+        x = torch.as_tensor(flat[off[b]:off[b] + n * n].reshape(1, n, n)).cuda()
+        c1 = apm.cdet_connected(x)[0]
+        assert np.array_equal(cf[row[b]:row[b + 1]].cpu().numpy(), c1.cpu().numpy(), equal_nan=True), b
+    apm.tune_options_set(0, 1, 0)                       # fewer slots than these items' weights take
+    try:
+        c2 = apm.cdet_connected_varlen(A, ao[:few.size].contiguous(), nt[:few.size].contiguous())
+    finally:
+        apm.tune_options_set(0, 0, 0)
+    assert np.array_equal(c2.cpu().numpy(), cf.cpu().numpy(), equal_nan=True)
