@@ -652,6 +652,171 @@ __global__ void __launch_bounds__(kCdetThreads, 3) fpm_cdet_kernel(const CdetKer
 }
 
 // ---------------------------------------------------------------------------
+// Orders 11 and 12, few matrices: a cluster of CTAs per matrix
+// ---------------------------------------------------------------------------
+// One matrix of order 12 is 9400 FP64 warp instructions on one SM, 109 us, with
+// the other SMs idle. Here 2^lc CTAs hold a copy of a[] and c[] each. The tree's
+// first lc levels are expanded by all of them, below those a CTA has the nodes
+// whose masks end in its rank; their minors go to the other CTAs' shared memory.
+// A layer's set groups are dealt out to the warps of all CTAs, each finished c[S]
+// goes to every copy, and a cluster barrier ends the layer. Every value is formed
+// by the operations of fpm_cdet_kernel, in their order: the same bits.
+__device__ __forceinline__ uint32_t cluster_rank() {
+    uint32_t r;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+// all threads of the cluster; orders their shared memory accesses, remote ones too
+__device__ __forceinline__ void cluster_barrier() {
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_put(double *local, uint32_t rank, double v) {
+    uint32_t addr;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(addr) : "r"(smem_u32(local)), "r"(rank));
+    asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(addr), "d"(v) : "memory");
+}
+__device__ __forceinline__ void cluster_or(int *local, uint32_t rank, int v) {
+    uint32_t addr;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(addr) : "r"(smem_u32(local)), "r"(rank));
+    asm volatile("red.shared::cluster.or.b32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
+}
+
+// the corrections logged at levels lo .. hi - 1, deepest first (as in fpm_tree)
+__device__ __forceinline__ void cluster_backprop(double *MA, int n, double shift, const CdetSmemHdr &h, int lo, int hi) {
+    for (int ci = h.ncorr - 1; ci >= 0; --ci) {
+        const int x = h.log_x[ci], lv = h.log_l[ci];
+        if (lv < lo || lv >= hi) continue;
+        const double pv = h.log_p[ci], cs = pv >= 0.0 ? shift : -shift;
+        for (int t = threadIdx.x; t < (1 << (n - lv - 1)); t += blockDim.x) {
+            const int src = x | (t << (lv + 1)), tgt = src | (1 << lv);
+            MA[tgt] = t == 0 ? MA[src] * pv : fma(-cs, MA[src], MA[tgt]);
+        }
+        __syncthreads();
+    }
+}
+
+// fpm_tree over the cluster (n - 4 > lc, and fewer nodes above the 4 x 4 ones
+// than the log holds): every CTA's MA complete and corrected on return.
+__device__ __forceinline__ void cluster_tree(const double *__restrict__ Ag, int n, double *MA, double *MC, double thr,
+                                             double shift, CdetSmemHdr &h, int rank, int lc) {
+    const int tid = threadIdx.x, T = blockDim.x, L = n - 4;
+    double *const bufA = MA + (1 << L);
+    auto buf = [&](int lv) { return ((L - lv) & 1) ? bufA : MC; };
+    double *W0 = buf(0);
+    for (int t = tid; t < n * n; t += T) W0[t] = __ldg(Ag + t);
+    if (tid == 0) MA[0] = 1.0;
+    __syncthreads();
+    for (int l = 0; l < L; ++l) {
+        const int s = n - l, s1 = s - 1, ss = s * s, ss1 = s1 * s1;
+        const bool own = l >= lc;                       // node i is mask (i << lc) | rank, else mask i
+        const int P = own ? 1 << (l - lc) : 1 << l;
+        double *Wl = buf(l), *Wn = buf(l + 1);
+        for (int i = tid; i < P; i += T) {
+            double v = Wl[i * ss];
+            node_pivot(own ? (i << lc) | rank : i, l, v, MA, thr, shift, h);
+            Wl[i * ss] = v;
+        }
+        __syncthreads();
+        for (int e = tid; e < P * s1; e += T) {
+            const int m = e / s1, q = e - m * s1 + 1;
+            Wl[m * ss + q] *= Wl[m * ss];
+        }
+        __syncthreads();
+        // the children: all of them, or at the last shared level only this CTA's
+        const bool one = l + 1 == lc;
+        const int E = (one ? 1 : 2 * P) * ss1;
+        for (int e = tid; e < E; e += T) {
+            const int x = e / ss1, rem = e - x * ss1, p = rem / s1, q = rem - p * s1;
+            const int xi = one ? rank : x;
+            const double *Wp = Wl + (xi & (P - 1)) * ss;
+            double v = Wp[(p + 1) * s + q + 1];
+            if (xi >= P) v = fma(-Wp[(p + 1) * s], Wp[q + 1], v);
+            Wn[x * ss1 + rem] = v;
+        }
+        __syncthreads();
+    }
+    for (int i = tid; i < (1 << (L - lc)); i += T) bottom43(MC + i * 16, MA, (i << lc) | rank, L, thr, shift, h);
+    __syncthreads();
+    cluster_backprop(MA, n, shift, h, lc, L);
+    cluster_barrier();  // nobody's MA or MC holds tree nodes any more
+    for (int i = tid; i < (1 << (n - lc)); i += T) {
+        const int m = (i << lc) | rank;
+        const double v = MA[m];
+        for (int q = 1; q < (1 << lc); ++q) cluster_put(MA + m, rank ^ q, v);
+    }
+    if (tid == 0 && h.ncorr > 0) h.flags |= APM_ST_PIVOT_CORRECTED;
+    __syncthreads();
+    if (tid == 0 && rank && h.flags) cluster_or(&h.flags, 0, h.flags);
+    cluster_barrier();
+    cluster_backprop(MA, n, shift, h, 0, lc);
+}
+
+__global__ void __launch_bounds__(kCdetThreads, 2) fpm_cdet_cluster_kernel(const CdetKernelParams P, int lc) {
+    extern __shared__ __align__(128) unsigned char smem_raw[];
+    CdetSmemHdr &h = *reinterpret_cast<CdetSmemHdr *>(smem_raw);
+    const CdetArgs &p = P.a;
+    const int n = p.n, N = 1 << n, tid = threadIdx.x, T = blockDim.x;
+    const int lane = tid & 31, warp = tid >> 5, nw = T >> 5;
+    const int rank = static_cast<int>(cluster_rank()), size = 1 << lc;
+    const int64_t b = blockIdx.x >> lc;
+    double *MA = reinterpret_cast<double *>(smem_raw + ((sizeof(CdetSmemHdr) + 127) & ~size_t(127)));
+    double *MC = MA + N, *MU = MC + N;
+    const int s0 = rank << (n - lc), s1 = (rank + 1) << (n - lc);  // this CTA's slice of the output rows
+    if (tid == 0) {
+        h.ncorr = 0;
+        h.flags = 0;
+    }
+    __syncthreads();
+    if (p.mode == kModeWeights) {
+        for (int t = tid; t < N; t += T) MA[t] = t ? __ldg(p.a_in + b * N + t) : 1.0;  // a[0] is not read
+        __syncthreads();
+    } else {
+        const int64_t mat = static_cast<int64_t>(n) * n;
+        if (p.two_mats) {
+            matrix_norm(p.A_dn + b * mat, n, h, nullptr);
+            cluster_tree(p.A_dn + b * mat, n, MA, MC, p.piv_thr * h.anorm, p.piv_shift * h.anorm, h, rank, lc);
+            for (int t = tid; t < N; t += T) MU[t] = MA[t];
+            if (tid == 0) h.ncorr = 0;
+            __syncthreads();
+        }
+        matrix_norm(p.A_up + b * mat, n, h, nullptr);
+        cluster_tree(p.A_up + b * mat, n, MA, MC, p.piv_thr * h.anorm, p.piv_shift * h.anorm, h, rank, lc);
+        if (p.minors_out) {
+            double *mo = p.minors_out + b * (p.two_mats ? 2 * N : N);
+            for (int t = s0 + tid; t < s1; t += T) {
+                mo[t] = MA[t];
+                if (p.two_mats) mo[N + t] = MU[t];
+            }
+        }
+        if (tid == 0 && rank == 0 && p.status) p.status[b] = static_cast<uint32_t>(h.flags);
+        __syncthreads();
+        if (!p.single_det)
+            for (int t = tid; t < N; t += T) MA[t] *= p.two_mats ? MU[t] : MA[t];
+        __syncthreads();
+    }
+    for (int t = tid; t < N; t += T) MC[t] = t & (t - 1) ? 0.0 : (t ? MA[t] : 0.0);
+    cluster_barrier();  // every copy of c[] is ready for the others' sums
+    for (int k = 2; k <= n; ++k) {
+        const int cnt = c_binom[n][k];
+        const uint16_t *masks = g_popmasks + g_popoff[k];
+        const int r = static_cast<int>((P.gsel >> (3 * k)) & 7ull), spw = 32 >> r;
+        for (int base = (warp * size + rank) * spw; base < cnt; base += nw * size * spw) {
+            const int G = base + (lane >> r);
+            const CdetSet q = cdet_set(masks[G < cnt ? G : cnt - 1], r, lane);
+            double acc = cdet_walk(MC, MA, q.j, q.Sp, q.UL, q.H, r == 0);
+            for (int o = (1 << r) >> 1; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+            if (G < cnt) {  // all lanes of the group hold the sum
+                const double v = MA[q.S] - acc;
+                for (int to = q.gl; to < size; to += 1 << r) cluster_put(MC + q.S, to, v);
+            }
+        }
+        cluster_barrier();
+    }
+    for (int t = s0 + tid; t < s1; t += T) p.c_out[b * N + t] = MC[t];
+}
+
+// ---------------------------------------------------------------------------
 // Orders 13..15, few matrices: the blocked recursion of cdet_blocked with a
 // matrix's blocks on many CTAs
 // ---------------------------------------------------------------------------
@@ -1128,6 +1293,36 @@ static int launch_cdet_split(const SplitArgs &P, int64_t most, cudaStream_t s) {
 //   n = 15: 1 4195 | 249, 24 4215 | 580, 152 4267 | 2615, 456 6757 | 6756
 static bool cdet_split_pays(int n, int64_t batch) { return batch <= (n == 13 ? 260 : n == 14 ? 350 : 456); }
 
+// CTAs per matrix (log2) of a launch of so many matrices, 0 for one: at most a CTA
+// per SM (two on an SM share its FP64 pipe). us per call, 1, 2, 4 and 8 CTAs:
+//   n = 12: 1 matrix 109, 76, 58, 55; 38 109, 76, 76, 117; 100 109, 109
+//   n = 11: 1 51, 45, 39, 39; 38 51, 45, 45, 77
+//   n = 10: 1 29, 33, 31, 31: a layer's barrier costs what its other lanes save
+static int cdet_cluster_log2(int n, int64_t batch) {
+    if (n < 11 || n > 12 || batch > 76) return 0;
+    return batch > 32 ? 1 : n == 12 && batch <= 10 ? 3 : 2;
+}
+
+static int launch_cdet_cluster(const CdetKernelParams &P, int lc, cudaStream_t s) {
+    const bool two = P.a.two_mats != 0;
+    const size_t smem = cdet_smem_bytes(P.a.n, two, true);
+    int err = 0;
+    resident_ctas(fpm_cdet_cluster_kernel, kCdetThreads, smem, cdet_smem_bytes(cdet_smem_max_n(true), true, true), &err);
+    if (err) return err;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(static_cast<unsigned>(P.a.batch << lc));
+    cfg.blockDim = dim3(kCdetThreads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = 1u << lc;
+    attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return static_cast<int>(cudaLaunchKernelEx(&cfg, fpm_cdet_cluster_kernel, P, lc));
+}
+
 int launch_fpm_cdet(const CdetArgs &a, cudaStream_t s) {
     if (!a.redo_list && !a.pre && !a.anorm_in) {
         const int lg = cdet_lanes_log2(a.n, a.batch, a.mode);
@@ -1193,6 +1388,10 @@ int launch_fpm_cdet(const CdetArgs &a, cudaStream_t s) {
         err = static_cast<int>(cudaGetLastError());
         if (err) return err;
         return launch_cdet_split(Q, rest, s);
+    }
+    if (smem_arrays && a.mode != kModeMinors && !a.redo_list) {
+        const int lc = cdet_cluster_log2(a.n, a.batch);
+        if (lc) return launch_cdet_cluster(P, lc, s);
     }
     if (smem_arrays)
         fpm_cdet_kernel<true><<<grid, cdet_threads(a.n, a.batch), smem, s>>>(P);

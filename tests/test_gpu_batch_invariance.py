@@ -221,3 +221,16 @@ def test_uneven_few_and_many(apm):
     finally:
         apm.tune_options_set(0, 0, 0)
     assert np.array_equal(c2.cpu().numpy(), cf.cpu().numpy(), equal_nan=True)
+
+
+# orders 11 and 12: clusters of 8, 4 and 2 CTAs per matrix, and one CTA each
+@pytest.mark.parametrize("n,batch", [(11, 32), (11, 76), (11, 77), (12, 10), (12, 32), (12, 76), (12, 77)])
+def test_clusters(apm, n, batch):
+    d = torch.as_tensor(mixed(n, batch, 9000 + n)).cuda()
+    e = torch.as_tensor(mixed(n, batch, 9100 + n)).cuda()
+    many = torch.arange(200).cuda() % batch          # the same matrices in a call of one CTA each
+    for f in (lambda x, y: apm.cdet_connected(x, return_minors=True, return_status=True),
+              lambda x, y: apm.cdet_connected(x, y, return_minors=True, return_status=True),
+              lambda x, y: apm.cdet_connected(x, single_det=True, return_status=True, piv_threshold=0.5),
+              lambda x, y: (apm.cdet_from_weights(apm.cdet_connected(x, single_det=True)),)):
+        rows_equal(f(d[many], e[many]), f(d, e), list(range(batch)))
