@@ -108,9 +108,13 @@ typedef struct {
  *   status  [batch] uint32 or NULL.
  *   workspace / workspace_bytes: scratch for n >= 9 (see apm_workspace_size),
  *           256-byte aligned; may be NULL/0 for n <= 8.
- * For n = 9..16 one warp takes a matrix (elements decided from the last one
- * down: above the last 12 depth first, then 5 levels breadth first in shared
- * memory, then each lane finishes one of the 32 nodes left, in registers, down
+ * The size of the batch decides how a matrix is spread over the GPU, here and in
+ * the calls below; unless a call says otherwise it does not change a bit of the
+ * results. For n <= 8 large batches take a few lanes per matrix.
+ * For n = 9..16 one warp takes a matrix, or of few matrices a run of its
+ * depth-first leaves (elements decided from the last one
+ * down: above the last 12, or fewer, depth first, then 5 levels breadth first in
+ * shared memory, then each lane finishes one of the 32 nodes left, in registers, down
  * to 3 x 3 nodes whose 8 minors it writes in closed form); it shifts no pivot, and the matrices that meet a pivot with |p| <= piv_threshold
  * ||A||max are computed again, with the correction, by the one-CTA-per-matrix
  * kernel of apm_cdet_connected, launched after it on those matrices only.
@@ -159,6 +163,9 @@ apm_status_t apm_all_minors(const double *A, int n, int64_t batch, double *minor
  * correction, only for the matrices that tree flagged (a pivot at or below the
  * threshold, a non-finite entry). The workspace then also holds one flag byte
  * per matrix (apm_workspace_size with APM_OP_CDET includes it).
+ * Few matrices (or the last, partial round of more) at n >= 13 have their blocks
+ * of 1024 subsets on many CTAs, level by level, with up to 64 MB of the workspace
+ * for the terms of the blocks; at n = 11, 12 a cluster of CTAs takes a matrix.
  */
 apm_status_t apm_cdet_connected(const double *A_up, const double *A_dn, int n, int64_t batch,
                                 int flags, double *c, double *minors_out,
@@ -245,8 +252,9 @@ apm_status_t apm_cdet_from_weights_fsc(const double *a, int n, int64_t batch, do
  *   status   [batch] or NULL; APM_ST_ZERO_PIVOT marks a singular or non-finite
  *            2 x 2 pivot block met on the way, APM_ST_NONFINITE_INPUT a NaN or
  *            infinity in the input; either makes that matrix's row NaN.
- *   workspace / workspace_bytes: scratch for the depth-first part of the tree,
- *            needed for n > 9 (apm_workspace_size with APM_OP_XNOR_MINORS).
+ *   workspace / workspace_bytes: scratch for the depth-first part of the tree and
+ *            a status word per matrix, needed for n > 9 (apm_workspace_size with
+ *            APM_OP_XNOR_MINORS).
  */
 apm_status_t apm_xnor_minors(const double *M, int n, int64_t batch, double *minors, uint32_t *status,
                              void *workspace, size_t workspace_bytes, apm_stream_t stream);
@@ -439,7 +447,9 @@ apm_status_t apm_perm_minors(const double *A, int n, int64_t batch, double *perm
  * their weights in c and a third launch finishes them in place by the fast
  * subset convolution, as apm_cdet_connected does at n = 16. Without A_dn, the
  * matrices of orders 13..16 take their minors, as apm_cdet_connected does, from
- * one warp-per-matrix launch per order before the persistent kernel.
+ * one warp-per-matrix launch per order before the persistent kernel. Of up to
+ * 1024 matrices those of orders 13..15 that launch has not flagged go by blocks on
+ * many CTAs, as few matrices of a fixed order do (64 MB of the workspace).
  * A matrix whose n[b] is outside 1..n_max is skipped with APM_ST_BAD_ORDER.
  * The call allocates nothing and does not synchronise: it can be captured in a
  * CUDA graph once the first (non-captured) call on the device has run.
@@ -482,9 +492,12 @@ apm_status_t apm_cdet_tune_get(int n, uint64_t *packed);
  *                     apm_cdet_connected and apm_cdet_connected_varlen: 13..16,
  *                     17 for never, 0 for the default 16.
  *   cdet_ctas_per_sm  resident CTAs per SM of the persistent uneven-batch kernel
- *                     of apm_cdet_connected_varlen: 1..3, 0 for as many as fit (3).
+ *                     of apm_cdet_connected_varlen: 1..3, 0 for as many as fit (3);
+ *                     counted in CTAs of 256 threads (batches without orders above
+ *                     9 or 11 run CTAs of 64 or 128, four or two of which count as one).
  *   keldysh_warps     warps per CTA of apm_keldysh_sum_varlen: 4..12, 0 for 12
- *                     (fewer warps per CTA let more CTAs share an SM).
+ *                     (fewer warps per CTA let more CTAs share an SM); fewer where
+ *                     the batch would not give every SM a CTA.
  * Workspace sizes depend on the first two: query apm_workspace_size after
  * setting them (a smaller workspace than the options need is rejected with
  * APM_ERR_WORKSPACE). Results differ between hand-off orders by rounding only.
