@@ -94,7 +94,7 @@ struct Lanes {
         const bool corr = fabs(p) <= t.thr;
         const double C = corr ? (p >= 0.0 ? t.shift : -t.shift) : 0.0;
         const double piv = p + C;
-        const double v = rcp_nr(piv);
+        const double v = 1.0 / piv;
         const int xk = x | (1 << L);
         t.put(xk, d * p, mine);
         const double g1 = w[1][0] * v, g2 = w[2][0] * v, g3 = w[3][0] * v;
@@ -140,7 +140,7 @@ struct Lanes {
             }
             const double dk = d * piv;
             t.put(x | (1 << lev), dk, w);
-            const double iv = rcp_nr(piv);
+            const double iv = 1.0 / piv;
             double S[K - 1][K - 1];
             if constexpr (lev < TOP) {
                 const bool keep = (t.q >> lev) & 1;

@@ -165,7 +165,7 @@ __device__ __forceinline__ void node_pivot(int x, int lev, double &v, double *MA
         piv += piv >= 0.0 ? shift : -shift;
     }
     MA[x | (1 << lev)] = MA[x] * piv;
-    v = rcp_nr(piv);
+    v = 1.0 / piv;
 }
 
 // All 15 principal minors of a 4x4 matrix w (row-major) times `pre`, written to
@@ -266,7 +266,7 @@ __device__ __forceinline__ void bottom43(const double *__restrict__ w, double *M
     const bool corr = fabs(p) <= thr;
     const double C = corr ? (p >= 0.0 ? shift : -shift) : 0.0;
     const double piv = p + C;
-    const double v = rcp_nr(piv);
+    const double v = 1.0 / piv;
     const int mk = m | (1 << L);
     MA[mk] = d * p;
     const double g1 = w[4] * v, g2 = w[8] * v, g3 = w[12] * v;
