@@ -15,15 +15,22 @@
 //     alpha = prod_{i in S_H} u_i(T),   B = prod_{i in S_L} u_i(T),   T = T_H u T_L.
 //
 // One CTA per matrix, 8 warps, three CTAs per SM; the outer loop runs over the
-// high column subsets T_H, two CTA barriers per step:
-//  * tables (each warp alone, for the T_L it owns): U[i][T_L] = u_i(T_H u T_L)
-//    (one add per entry from row sums kept per T_L and per T_H; the high row
-//    sums of the next T_H take one add each, from a stack indexed by
-//    popcount), the 8 starting products base_b(T_L) = prod_{i in T_H u R_b} u_i
-//    over the subsets R_b of the lowest (up to) three high elements outside
-//    T_H, and the 3^l entries B(T_L, S_L) level by level over |S_L \ T_L|, one
-//    multiply each. The owners of T_L are chosen so that the warps get equal
-//    shares.
+// high column subsets T_H, four CTA barriers per step:
+//  * tables: U[i][T_L] = u_i(T_H u T_L), a column per lane (one add per entry
+//    from row sums kept per T_L and per T_H; the high row sums of the next T_H
+//    take one add each, from a stack indexed by popcount); then on half of the
+//    warps the 8 starting products base_b(T_L) = prod_{i in T_H u R_b} u_i over
+//    the subsets R_b of the lowest (up to) three high elements outside T_H, and
+//    on the other half the diagonal entries B(T_L, T_L), in the order of |T_L|
+//    (the lanes of a warp multiply equally often); then the other entries
+//    B(T_L, S_L) level by level over |S_L \ T_L|, one multiply each, every warp
+//    for the T_L it owns (a parent and its entry then belong to one warp: no
+//    barrier per level). The FP64 pipe bounds the kernel and an instruction
+//    costs it the same for one active lane as for 32, so the phases are cut to
+//    fill lanes: with U, the bases and the diagonal also done by the owners of
+//    the T_L (16 of 32 lanes, three barriers less) 4096 matrices of order 14
+//    took 47.4 ms instead of 44.6, 912 of order 12 1531 us instead of 1414 and
+//    one 386 instead of 350.
 //  * products (warp b takes the S_H = T_H u R_b u R' for all R' over the
 //    remaining free high elements, depth first, so that each alpha vector is
 //    its parent's times one u_i; the path stays in registers): for every S_L
@@ -71,10 +78,9 @@ struct PpmSched {
     int rnd;      // [nrounds + 1] CSR offsets of the rounds of slot additions
     int pairs;    // slot additions (dst | src << 16): the runs of a cut set added pairwise, a tree
     int nrounds;
-    int tl;       // [kPpmWarps + 1] CSR offsets of the T_L owned by each warp
-    int tllist;   // [2^l] owned T_L, warp by warp
-    int blvl;     // [kPpmWarps][l + 2] B entries of each warp, level by level
-    int ent;      // [3^l][2] entries: (dst | src << 16), (e | T_L << 8); src 0xffff at level 0
+    int lvl0;     // [2^l] T_L by increasing size | B slot of (T_L, T_L) << 16
+    int blvl;     // [kPpmWarps][l + 1] B entries of each warp, level by level from level 1
+    int ent;      // [3^l - 2^l][2] entries: (dst | src << 16), (e | T_L << 8)
     int len;      // [64] terms of each stream
     int maxlen;   // terms per stream (the first streams; the last one may have fewer)
     int nres;     // result slots used
@@ -231,18 +237,13 @@ static void build_schedules(std::vector<int> &buf) {
             owner[T] = best;
             wload[best] += 1 << (l - popc(T));
         }
-        std::vector<int> tl(kPpmWarps + 1), tllist;
+        std::vector<int> lvl0;  // tls is in the order of increasing size
+        for (int T : tls) lvl0.push_back(T | (pos_of[static_cast<size_t>(T) * NL + pext_host(T, T)] << 16));
+        // B entries, warp by warp, level by level over d = |S \ T| >= 1
+        std::vector<int> blvl(static_cast<size_t>(kPpmWarps) * (l + 1)), ent;
         for (int w = 0; w < kPpmWarps; ++w) {
-            tl[w] = static_cast<int>(tllist.size());
-            for (int T = 0; T < NL; ++T)
-                if (owner[T] == w) tllist.push_back(T);
-        }
-        tl[kPpmWarps] = static_cast<int>(tllist.size());
-        // B entries, warp by warp, level by level over d = |S \ T|
-        std::vector<int> blvl(static_cast<size_t>(kPpmWarps) * (l + 2)), ent;
-        for (int w = 0; w < kPpmWarps; ++w) {
-            for (int d = 0; d <= l; ++d) {
-                blvl[static_cast<size_t>(w) * (l + 2) + d] = static_cast<int>(ent.size() / 2);
+            for (int d = 1; d <= l; ++d) {
+                blvl[static_cast<size_t>(w) * (l + 1) + d - 1] = static_cast<int>(ent.size() / 2);
                 for (int T = 0; T < NL; ++T) {
                     if (owner[T] != w) continue;
                     const int fr = (NL - 1) & ~T;
@@ -250,12 +251,9 @@ static void build_schedules(std::vector<int> &buf) {
                         if (popc(R) == d) {
                             const int S = T | R;
                             const int dst = pos_of[static_cast<size_t>(S) * NL + pext_host(T, S)];
-                            int src = 0xffff, e = 0;
-                            if (d > 0) {
-                                e = 31 - __builtin_clz(static_cast<unsigned>(R));
-                                const int Sp = S ^ (1 << e);
-                                src = pos_of[static_cast<size_t>(Sp) * NL + pext_host(T, Sp)];
-                            }
+                            const int e = 31 - __builtin_clz(static_cast<unsigned>(R));
+                            const int Sp = S ^ (1 << e);
+                            const int src = pos_of[static_cast<size_t>(Sp) * NL + pext_host(T, Sp)];
                             ent.push_back(dst | (src << 16));
                             ent.push_back(e | (T << 8));
                         }
@@ -263,7 +261,7 @@ static void build_schedules(std::vector<int> &buf) {
                     }
                 }
             }
-            blvl[static_cast<size_t>(w) * (l + 2) + l + 1] = static_cast<int>(ent.size() / 2);
+            blvl[static_cast<size_t>(w) * (l + 1) + l] = static_cast<int>(ent.size() / 2);
         }
         // the runs of every cut set are added pairwise (stride 1, 2, 4, ...) into the
         // slot of its first run; round r holds the additions of stride 2^r, at most
@@ -302,8 +300,7 @@ static void build_schedules(std::vector<int> &buf) {
         s.first = put(first);
         s.rnd = put(rnd);
         s.pairs = put(pairs);
-        s.tl = put(tl);
-        s.tllist = put(tllist);
+        s.lvl0 = put(lvl0);
         s.blvl = put(blvl);
         if (buf.size() & 1) buf.push_back(0);  // the entries are read as int2 (8-byte aligned)
         s.ent = put(ent);
@@ -318,8 +315,8 @@ static bool schedules_fit(const std::vector<int> &buf) {
         const PpmSched &s = h_sched[l];
         if (s.maxlen * kPpmVLanes > kPpmBpSlots || s.nres > kPpmResSlots) return false;
         for (int w = 0; w < kPpmWarps; ++w)
-            for (int d = 0; d <= l; ++d) {
-                const int *lv = buf.data() + s.blvl + w * (l + 2);
+            for (int d = 0; d < l; ++d) {
+                const int *lv = buf.data() + s.blvl + w * (l + 1);
                 if (lv[d + 1] - lv[d] > 4 * 32) return false;
             }
         for (int r = 0; r < s.nrounds; ++r)  // one slot addition per lane and round
@@ -406,9 +403,8 @@ __global__ void __launch_bounds__(kPpmWarps * 32, 3) ppm_kernel(const double *__
     const int *first = g_ppm_sched + sc.first;
     const int *rnd = g_ppm_sched + sc.rnd;
     const int *pairs = g_ppm_sched + sc.pairs;
-    const int *tllist = g_ppm_sched + sc.tllist + g_ppm_sched[sc.tl + warp];
-    const int ntl = g_ppm_sched[sc.tl + warp + 1] - g_ppm_sched[sc.tl + warp];
-    const int *blvl = g_ppm_sched + sc.blvl + warp * (l + 2);
+    const int *blvl = g_ppm_sched + sc.blvl + warp * (l + 1);
+    const int *lvl0 = g_ppm_sched + sc.lvl0;
     const int2 *ent = reinterpret_cast<const int2 *>(g_ppm_sched + sc.ent);
     const int lenA = g_ppm_sched[sc.len + 2 * lane];  // the lane's first stream is the longer one
     const int2 *term2 = reinterpret_cast<const int2 *>(term);
@@ -437,25 +433,24 @@ __global__ void __launch_bounds__(kPpmWarps * 32, 3) ppm_kernel(const double *__
             for (int k = 0, r = freeH; k < m; ++k, r &= r - 1) lowmask |= r & (-r);
             const int lm1 = lowmask & (lowmask - 1), lm2 = lm1 & (lm1 - 1);
             const int e0 = __ffs(lowmask) - 1, e1 = __ffs(lm1) - 1, e2 = __ffs(lm2) - 1;  // -1 where absent
-            // ---- tables, each warp for its own T_L ----
-            {
-                // U[i][T_L]: lane = (T_L parity, row i)
-                const int i = lane & 15;
-                if (i < n) {
-                    const double rhi = sm.rhs[__popc(TH)][i];
-                    const bool high = i >= l;
-                    const bool inTH = high && ((TH >> (i - l)) & 1);
-                    for (int k = lane >> 4; k < ntl; k += 2) {
-                        const int TL = tllist[k];
-                        const bool inT = high ? inTH : ((TL >> i) & 1);
-                        const double rr = rhi + sm.RL[i * kPpmLd + TL];
-                        sm.U[i * kPpmLd + TL] = inT ? rr : neg_bits(rr);
-                    }
-                }
+            // ---- tables ----
+            // this lane's B entries of level 1 (l >= 1: there is one)
+            int2 cur[4], nxt[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const int e = blvl[0] + lane + 32 * k;
+                cur[k] = e < blvl[1] ? __ldcg(ent + e) : make_int2(0, 0);
             }
-            __syncwarp();
-            for (int k = lane; k < ntl; k += 32) {
-                const int TL = tllist[k];
+            // U, a column per lane
+            for (int t = tid; t < n << l; t += T) {
+                const int i = t >> l, TL = t & (NL - 1);
+                const bool inT = ((TH << l | TL) >> i) & 1;
+                const double rr = sm.rhs[__popc(TH)][i] + sm.RL[i * kPpmLd + TL];
+                sm.U[i * kPpmLd + TL] = inT ? rr : neg_bits(rr);
+            }
+            __syncthreads();
+            if (tid < NL) {  // half of the warps: the starting products of a T_L
+                const int TL = tid;
                 const double pt = set_prod(sm.U, l, TH, TL);
                 double *base = &sm.alpha[0][TL];  // base[bb * 128] for the lattice element subsets bb
                 base[0] = pt;
@@ -477,36 +472,32 @@ __global__ void __launch_bounds__(kPpmWarps * 32, 3) ppm_kernel(const double *__
                         }
                     }
                 }
+            } else if (tid - 128 >= 0 && tid - 128 < NL) {  // the other half: level 0 of the B table
+                const int w = lvl0[tid - 128], TL = w & 0xffff;
+                sm.Bp[w >> 16] = set_prod(sm.U, 0, TL, TL);
             }
-            {
-                // B entries level by level; this lane's entries of the next
-                // level are fetched while the current one is computed
-                int2 cur[4], nxt[4];
+            __syncthreads();
+            // B entries level by level, each warp for its own T_L; the entries of
+            // the next level are fetched while the current one is computed
+            for (int d = 0; d < l; ++d) {
+                const int beg = blvl[d], end = blvl[d + 1], nend = d + 1 < l ? blvl[d + 2] : end;
 #pragma unroll
                 for (int k = 0; k < 4; ++k) {
-                    const int e = blvl[0] + lane + 32 * k;
-                    cur[k] = e < blvl[1] ? __ldcg(ent + e) : make_int2(0, 0);
+                    const int e = end + lane + 32 * k;
+                    nxt[k] = e < nend ? __ldcg(ent + e) : make_int2(0, 0);
                 }
-                for (int d = 0; d <= l; ++d) {
-                    const int beg = blvl[d], end = blvl[d + 1], nend = d < l ? blvl[d + 2] : end;
 #pragma unroll
-                    for (int k = 0; k < 4; ++k) {
-                        const int e = end + lane + 32 * k;
-                        nxt[k] = e < nend ? __ldcg(ent + e) : make_int2(0, 0);
+                for (int k = 0; k < 4; ++k) {
+                    if (beg + lane + 32 * k < end) {
+                        const int2 w = cur[k];
+                        const int dst = w.x & 0xffff, src = (w.x >> 16) & 0xffff;
+                        const int el = w.y & 0xff, TL = w.y >> 8;
+                        sm.Bp[dst] = sm.Bp[src] * sm.U[el * kPpmLd + TL];
                     }
-#pragma unroll
-                    for (int k = 0; k < 4; ++k) {
-                        if (beg + lane + 32 * k < end) {
-                            const int2 w = cur[k];
-                            const int dst = w.x & 0xffff, src = (w.x >> 16) & 0xffff;
-                            const int el = w.y & 0xff, TL = w.y >> 8;
-                            sm.Bp[dst] = d == 0 ? set_prod(sm.U, 0, TL, TL) : sm.Bp[src] * sm.U[el * kPpmLd + TL];
-                        }
-                    }
-                    __syncwarp();
-#pragma unroll
-                    for (int k = 0; k < 4; ++k) cur[k] = nxt[k];
                 }
+                __syncwarp();
+#pragma unroll
+                for (int k = 0; k < 4; ++k) cur[k] = nxt[k];
             }
             __syncthreads();
             // ---- products: warp w takes S_H = T_H u R_w u R' ----
