@@ -25,12 +25,14 @@
 //    (the lanes of a warp multiply equally often); then the other entries
 //    B(T_L, S_L) level by level over |S_L \ T_L|, one multiply each, every warp
 //    for the T_L it owns (a parent and its entry then belong to one warp: no
-//    barrier per level). The FP64 pipe bounds the kernel and an instruction
+//    barrier per level; the owners are chosen for few, full rounds of 32, see
+//    build_schedules). The FP64 pipe bounds the kernel and an instruction
 //    costs it the same for one active lane as for 32, so the phases are cut to
 //    fill lanes: with U, the bases and the diagonal also done by the owners of
-//    the T_L (16 of 32 lanes, three barriers less) 4096 matrices of order 14
+//    the T_L (16 of 32 lanes, two barriers less) 4096 matrices of order 14
 //    took 47.4 ms instead of 44.6, 912 of order 12 1531 us instead of 1414 and
-//    one 386 instead of 350.
+//    one 386 instead of 350; with the owners by fewest rounds 44.2 ms, 1389
+//    and 343.
 //  * products (warp b takes the S_H = T_H u R_b u R' for all R' over the
 //    remaining free high elements, depth first, so that each alpha vector is
 //    its parent's times one u_i; the path stays in registers): for every S_L
@@ -224,18 +226,58 @@ static void build_schedules(std::vector<int> &buf) {
                     }
                 }
         }
-        // owners of the T_L for the tables: largest share (2^(l-|T_L|) B entries) first
+        // owners of the T_L for the tables: by increasing size, cut into one
+        // contiguous piece per warp. A warp does a level's entries 32 at a time,
+        // so a piece costs the sum over its levels of ceil(entries / 32); taken
+        // is the cut with the smallest largest cost and, among these, the least
+        // cost in total (at l = 7: 11 and 81 warp multiplies; pieces of equal
+        // numbers of entries in total: 13 and 96)
         std::vector<int> tls(NL), owner(NL);
         for (int T = 0; T < NL; ++T) tls[T] = T;
         for (int i = 1; i < NL; ++i)
             for (int j = i; j > 0 && popc(tls[j]) < popc(tls[j - 1]); --j) std::swap(tls[j], tls[j - 1]);
-        int wload[kPpmWarps] = {};
-        for (int T : tls) {
-            int best = 0;
-            for (int w = 1; w < kPpmWarps; ++w)
-                if (wload[w] < wload[best]) best = w;
-            owner[T] = best;
-            wload[best] += 1 << (l - popc(T));
+        {
+            std::vector<int> pre(static_cast<size_t>(NL + 1) * (l + 1), 0);  // entries of the first j T_L by level
+            for (int j = 0; j < NL; ++j) {
+                const int f = l - popc(tls[j]);
+                int c = 1;  // binomial (f, d)
+                for (int d = 0; d <= l; ++d) {
+                    pre[(j + 1) * (l + 1) + d] = pre[j * (l + 1) + d] + c;
+                    c = c * (f - d) / (d + 1);
+                }
+            }
+            const int inf = 1 << 20;
+            const auto cost = [&](int i, int j) {  // of the piece i .. j-1
+                int s2 = 0;
+                for (int d = 1; d <= l; ++d) {
+                    const int c = pre[j * (l + 1) + d] - pre[i * (l + 1) + d];
+                    if (c > 4 * 32) return inf;
+                    s2 += (c + 31) / 32;
+                }
+                return s2;
+            };
+            for (int most = 1;; ++most) {  // ends: one piece per warp of a few T_L each costs little
+                std::vector<int> best(static_cast<size_t>(kPpmWarps + 1) * (NL + 1), inf), cut(best.size(), 0);
+                best[0] = 0;
+                for (int w = 1; w <= kPpmWarps; ++w)
+                    for (int j = 0; j <= NL; ++j)
+                        for (int i = 0; i <= j; ++i) {
+                            const int b0 = best[(w - 1) * (NL + 1) + i];
+                            if (b0 >= inf) continue;
+                            const int c = cost(i, j);
+                            if (c <= most && b0 + c < best[w * (NL + 1) + j]) {
+                                best[w * (NL + 1) + j] = b0 + c;
+                                cut[w * (NL + 1) + j] = i;
+                            }
+                        }
+                if (best[kPpmWarps * (NL + 1) + NL] >= inf) continue;
+                for (int w = kPpmWarps, j = NL; w > 0; --w) {
+                    const int i = cut[w * (NL + 1) + j];
+                    for (int k = i; k < j; ++k) owner[tls[k]] = w - 1;
+                    j = i;
+                }
+                break;
+            }
         }
         std::vector<int> lvl0;  // tls is in the order of increasing size
         for (int T : tls) lvl0.push_back(T | (pos_of[static_cast<size_t>(T) * NL + pext_host(T, T)] << 16));
