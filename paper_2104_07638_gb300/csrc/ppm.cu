@@ -406,9 +406,10 @@ __device__ __forceinline__ void ppm_terms(const int2 *__restrict__ term2, const 
     }
 }
 
-// -x by the sign bit (no FP64 instruction)
-__device__ __forceinline__ double neg_bits(double x) {
-    return __longlong_as_double(__double_as_longlong(x) ^ static_cast<long long>(0x8000000000000000ull));
+// x, or -x where neg, by the sign bit. The mask is chosen, not the result: of
+// the two results the compiler makes two additions, x and the negated one.
+__device__ __forceinline__ double sign_if(double x, bool neg) {
+    return __longlong_as_double(__double_as_longlong(x) ^ (static_cast<long long>(neg) << 63));
 }
 
 // prod over the set bits e of mask of U[(row0 + e) * kPpmLd + col] (1 for an empty
@@ -488,7 +489,7 @@ __global__ void __launch_bounds__(kPpmWarps * 32, 3) ppm_kernel(const double *__
                 const int i = t >> l, TL = t & (NL - 1);
                 const bool inT = ((TH << l | TL) >> i) & 1;
                 const double rr = sm.rhs[__popc(TH)][i] + sm.RL[i * kPpmLd + TL];
-                sm.U[i * kPpmLd + TL] = inT ? rr : neg_bits(rr);
+                sm.U[i * kPpmLd + TL] = sign_if(rr, !inT);
             }
             __syncthreads();
             if (tid < NL) {  // half of the warps: the starting products of a T_L
