@@ -739,14 +739,15 @@ __device__ __forceinline__ void cluster_tree(const double *__restrict__ Ag, int 
     for (int i = tid; i < (1 << (L - lc)); i += T) bottom43(MC + i * 16, MA, (i << lc) | rank, L, thr, shift, h);
     __syncthreads();
     cluster_backprop(MA, n, shift, h, lc, L);
+    // this CTA's status bits are complete before the barrier: after it the other
+    // CTAs' bits arrive in the first one's word
+    if (tid == 0 && h.ncorr > 0) h.flags |= APM_ST_PIVOT_CORRECTED;
     cluster_barrier();  // nobody's MA or MC holds tree nodes any more
     for (int i = tid; i < (1 << (n - lc)); i += T) {
         const int m = (i << lc) | rank;
         const double v = MA[m];
         for (int q = 1; q < (1 << lc); ++q) cluster_put(MA + m, rank ^ q, v);
     }
-    if (tid == 0 && h.ncorr > 0) h.flags |= APM_ST_PIVOT_CORRECTED;
-    __syncthreads();
     if (tid == 0 && rank && h.flags) cluster_or(&h.flags, 0, h.flags);
     cluster_barrier();
     cluster_backprop(MA, n, shift, h, 0, lc);

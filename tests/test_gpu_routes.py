@@ -1,0 +1,50 @@
+"""What the choice of a route must not change: status words, the possibility of
+capture, scratch that serves every smaller batch, results."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2104_07638_gb300 import inputs as I
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def apm():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2104_07638_gb300 import apm as m
+    m.lib()
+    m.tune_set(None)
+    m.tune_options_set(0, 0, 0)
+    return m
+
+
+def zero_pivot_at(n, kept, e, rng):
+    """A matrix whose pivot of element e is zero where exactly the set `kept` of the
+    elements below e is kept, and about 2 elsewhere."""
+    A = 2.0 * np.eye(n) + 0.2 * rng.standard_normal((n, n))
+    k = [i for i in range(e) if kept >> i & 1]
+    A[e, e] = A[e, k] @ np.linalg.solve(A[np.ix_(k, k)], A[k, e]) if k else 0.0
+    return A
+
+
+# a pivot corrected in the subtree of one CTA of the cluster only: its status bit
+# reaches the status word whichever CTA that is, with one matrix and with two
+@pytest.mark.parametrize("n,batch", [(11, 32), (12, 10), (12, 40)])
+def test_cluster_status(apm, n, batch):
+    rng = np.random.default_rng(9200 + n)
+    A = np.stack([zero_pivot_at(n, b % 8, 5 + b % 3, rng) for b in range(batch)])
+    A[8] = I.gaussian_plus_2I(n, 1, seed=3)[0]
+    A[9, n - 1, 0] = np.nan
+    B = np.stack([zero_pivot_at(n, (3 * b + 1) % 8, 6, rng) if b % 2 else I.gaussian_plus_2I(n, 1, seed=b)[0]
+                  for b in range(batch)])
+    d, e = torch.as_tensor(A).cuda(), torch.as_tensor(B).cuda()
+    many = torch.arange(200).cuda() % batch          # the same matrices in a call of one CTA each
+    for x, y in ((d, None), (d, e), (e, d)):
+        ref = apm.cdet_connected(x[many], None if y is None else y[many], return_minors=True, return_status=True)
+        assert int(ref[2][0]) & apm.ST_PIVOT_CORRECTED
+        for _ in range(20):
+            got = apm.cdet_connected(x, y, return_minors=True, return_status=True)
+            for g, r in zip(got, ref):
+                assert np.array_equal(g.cpu().numpy(), r[:batch].cpu().numpy(), equal_nan=True)
