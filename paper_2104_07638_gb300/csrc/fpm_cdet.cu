@@ -1325,12 +1325,15 @@ static int launch_cdet_cluster(const CdetKernelParams &P, int lc, cudaStream_t s
 }
 
 int launch_fpm_cdet(const CdetArgs &a, cudaStream_t s) {
+    // before any route, the lane groups' too, which read none of the tables: a
+    // later call on this device may be one under capture, where they cannot be
+    // uploaded
+    int err = ensure_tables();
+    if (err) return err;
     if (!a.redo_list && !a.pre && !a.anorm_in) {
         const int lg = cdet_lanes_log2(a.n, a.batch, a.mode);
         if (lg >= 0) return launch_cdet_lanes(a, lg, s);
     }
-    int err = ensure_tables();
-    if (err) return err;
     CdetKernelParams P;
     P.a = a;
     P.gsel = cdet_gsel_packed(a.n);

@@ -1,5 +1,9 @@
 """What the choice of a route must not change: status words, the possibility of
 capture, scratch that serves every smaller batch, results."""
+import os
+import subprocess
+import sys
+
 import numpy as np
 import pytest
 import torch
@@ -48,3 +52,35 @@ def test_cluster_status(apm, n, batch):
             got = apm.cdet_connected(x, y, return_minors=True, return_status=True)
             for g, r in zip(got, ref):
                 assert np.array_equal(g.cpu().numpy(), r[:batch].cpu().numpy(), equal_nan=True)
+
+
+CAPTURE = """
+import ctypes, torch
+from paper_2104_07638_gb300 import apm
+g = torch.Generator(device='cuda').manual_seed(1)
+def mats(b, n):
+    return torch.eye(n, device='cuda', dtype=torch.float64) + \
+        0.1 * torch.randn((b, n, n), generator=g, device='cuda', dtype=torch.float64)
+apm.cdet_connected(mats(30000, 6))              # lane groups
+torch.cuda.synchronize()
+s = ctypes.c_void_p()
+assert ctypes.CDLL('libcuda.so.1').cuStreamCreate(ctypes.byref(s), 0) == 0
+for n, b in ((10, 3), (12, 100), (14, 3)):
+    A = mats(b, n)
+    torch.cuda.synchronize()
+    G = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(G, stream=torch.cuda.ExternalStream(s.value)):
+        c = apm.cdet_connected(A)
+    G.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(c, apm.cdet_connected(A))
+print('captured')
+"""
+
+
+def test_capture_after_a_first_call_by_lane_groups(apm):
+    """Any first call uploads the constant tables: the calls after it can be
+    captured, on a stream that waits for the legacy one too."""
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    r = subprocess.run([sys.executable, "-c", CAPTURE], cwd=root, capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0 and "captured" in r.stdout, r.stderr[-2000:]
