@@ -493,8 +493,8 @@ apm_status_t apm_cdet_tune_get(int n, uint64_t *packed);
  *                     17 for never, 0 for the default 16.
  *   cdet_ctas_per_sm  resident CTAs per SM of the persistent uneven-batch kernel
  *                     of apm_cdet_connected_varlen: 1..3, 0 for as many as fit (3);
- *                     counted in CTAs of 256 threads (batches without orders above
- *                     9 or 11 run CTAs of 64 or 128, four or two of which count as one).
+ *                     counted in CTAs of 256 threads (larger batches without orders
+ *                     above 11 run CTAs of 64 or 128, four or two of which count as one).
  *   keldysh_warps     warps per CTA of apm_keldysh_sum_varlen: 4..12, 0 for 12
  *                     (fewer warps per CTA let more CTAs share an SM); fewer where
  *                     the batch would not give every SM a CTA.

@@ -1412,11 +1412,24 @@ int launch_fpm_cdet(const CdetArgs &a, cudaStream_t s) {
 // ---------------------------------------------------------------------------
 
 constexpr int kVarlenSmemMaxN = 12;
-// Threads of a CTA and the order its shared arrays hold, from the largest order
-// present: as for a fixed order, a batch of small orders only takes small CTAs,
-// and the arrays of its largest order rather than of order 12 (4096 walkers of
-// orders 4..9: 201 -> 156 us).
-static int varlen_threads(int n_max) { return n_max <= 9 ? 64 : n_max <= 11 ? 128 : kCdetThreads; }
+// Threads of a CTA, from the largest order present and the batch. Narrow CTAs
+// (four or two times as many on an SM) pay once the batch is several rounds of wide
+// ones: below that the call waits for the items of the largest order, which a wide
+// CTA finishes soonest. Us per call, 64 | 128 | 256 threads (device time):
+//   orders 4..8:  304 items 21 | 20 | 20, 600 22 | 22 | 23, 1500 27 | 27 | 44, 16384 159 | 207 | 361
+//   orders 4..9:  64 31 | 24 | 23, 912 42 | 40 | 35, 1200 42 | 40 | 41, 2736 59 | 54 | 79,
+//                 16384 218 | 268 | 430;  order 9 alone: 912 43 | 41 | 51, 2736 107 | 107 | 139
+//   orders 4..10: 456 56 | 49 | 46, 1500 92 | 79 | 61, 2100 82 | 79 | 83, 4096 119 | 110 | 151
+//   orders 4..11: 456 129 | 108 | 103, 1500 196 | 190 | 104, 3200 197 | 191 | 187, 4096 204 | 195 | 238;
+//                 order 11 alone: 1200 381 | 302 | 266, 3200 750 | 662 | 703
+static int varlen_threads(int n_max, int64_t batch) {
+    if (n_max <= 6) return 64;  // the same at any size below a round, the fastest above
+    if (n_max <= 8) return batch <= 456 ? kCdetThreads : 64;
+    if (n_max == 9) return batch < 1200 ? kCdetThreads : batch < 2700 ? 128 : 64;
+    if (n_max == 10) return batch < 2100 ? kCdetThreads : 128;
+    if (n_max == 11) return batch < 3300 ? kCdetThreads : 128;
+    return kCdetThreads;
+}
 // Largest uneven batch whose items of orders 13..15 go by blocks on many CTAs: a
 // CTA takes 4 ms for one of order 15 by itself, which is the whole call then
 // (300 walkers of orders 4..14 1672 -> 818 us, 100 of 10..16 3872 -> 1764, 1000 of
@@ -1424,11 +1437,14 @@ static int varlen_threads(int n_max) { return n_max <= 9 ? 64 : n_max <= 11 ? 12
 // Their weights, 2^15 doubles each at most, fit the region of the slots (456 x 3
 // times the largest order's).
 constexpr int64_t kVarlenSplitMax = 1024;
+// The order a CTA's shared arrays hold: the largest present rather than 12 leaves
+// room for the narrow CTAs.
 static int varlen_smem_n(int n_max) { return n_max < kVarlenSmemMaxN ? n_max : kVarlenSmemMaxN; }
 
 static size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
 
-static int cdet_varlen_grid(int n_max, bool two_mats, int *err) {
+static int cdet_varlen_grid(int n_max, int64_t batch, bool two_mats, int *err) {
+    const int threads = varlen_threads(n_max, batch);
     int dev = 0, sms = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -1436,12 +1452,12 @@ static int cdet_varlen_grid(int n_max, bool two_mats, int *err) {
         *err = static_cast<int>(e);
         return 0;
     }
-    int per_sm = resident_ctas(fpm_cdet_varlen_kernel, varlen_threads(n_max),
+    int per_sm = resident_ctas(fpm_cdet_varlen_kernel, threads,
                                cdet_smem_bytes(varlen_smem_n(n_max), two_mats, true),
                                cdet_smem_bytes(kVarlenSmemMaxN, true, true), err) / sms;
     if (*err) return 0;
     // the tuned limit counts CTAs of kCdetThreads threads
-    const int most = g_varlen_ctas * (kCdetThreads / varlen_threads(n_max));
+    const int most = g_varlen_ctas * (kCdetThreads / threads);
     if (most > 0 && most < per_sm) per_sm = most;
     return sms * per_sm;
 }
@@ -1478,7 +1494,7 @@ size_t cdet_varlen_workspace(int n_max, int64_t batch, bool two_mats, int *err) 
     *err = 0;
     size_t bytes = 256 + align256(static_cast<size_t>(batch) * sizeof(int));
     if (n_max <= kVarlenSmemMaxN) return bytes;
-    const int grid = cdet_varlen_grid(n_max, two_mats, err);
+    const int grid = cdet_varlen_grid(n_max, batch, two_mats, err);
     if (*err) return 0;
     size_t region = 0;
     *err = varlen_region(n_max, batch, two_mats, grid, &region);
@@ -1500,7 +1516,7 @@ int launch_cdet_varlen(const CdetArgs &a, const int64_t *a_off, const int *n_arr
     int err = ensure_tables();
     if (err) return err;
     const bool two = a.two_mats != 0;
-    const int grid = cdet_varlen_grid(n_max, two, &err);
+    const int grid = cdet_varlen_grid(n_max, a.batch, two, &err);
     if (err) return err;
     unsigned char *ws = static_cast<unsigned char *>(workspace);
     unsigned *ctr = reinterpret_cast<unsigned *>(ws);
@@ -1573,7 +1589,7 @@ int launch_cdet_varlen(const CdetArgs &a, const int64_t *a_off, const int *n_arr
     const bool fsc = a.mode == kModeCdet && n_max >= fsc_from;
     V.a.fsc_from_n = fsc ? fsc_from : 0;
     const int64_t g = a.batch < grid ? a.batch : grid;
-    fpm_cdet_varlen_kernel<<<static_cast<int>(g), varlen_threads(n_max),
+    fpm_cdet_varlen_kernel<<<static_cast<int>(g), varlen_threads(n_max, a.batch),
                              cdet_smem_bytes(varlen_smem_n(n_max), two, true), s>>>(V);
     err = static_cast<int>(cudaGetLastError());
     if (err || !fsc) return err;

@@ -84,3 +84,38 @@ def test_capture_after_a_first_call_by_lane_groups(apm):
     root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
     r = subprocess.run([sys.executable, "-c", CAPTURE], cwd=root, capture_output=True, text=True, timeout=300)
     assert r.returncode == 0 and "captured" in r.stdout, r.stderr[-2000:]
+
+
+# uneven batches without orders above 11, on both sides of every change of the
+# CTA's width, one matrix and two per item, against fixed-order calls
+@pytest.mark.parametrize("hi,batch", [(3, 50), (6, 500), (8, 456), (8, 457), (9, 1199), (9, 1200), (9, 2700),
+                                      (10, 2099), (10, 2100), (11, 3299), (11, 3300)])
+def test_uneven_small_orders(apm, hi, batch):
+    rng = np.random.default_rng(9300 + hi)
+    orders = rng.integers(1, hi + 1, batch).astype(np.int32)
+    orders[:3] = hi
+    off = np.concatenate([[0], np.cumsum(orders.astype(np.int64) ** 2)])[:-1]
+    flat = rng.standard_normal((2, int((orders.astype(np.int64) ** 2).sum())))
+    flat[0, off[1]:off[1] + hi * hi] = 0.0                 # corrected at every pivot
+    flat[0, off[2]] = np.inf
+    A, B = (torch.as_tensor(x).cuda() for x in flat)
+    ao, nt = torch.as_tensor(off).cuda(), torch.as_tensor(orders).cuda()
+    co = apm.varlen_out_offsets(nt)
+    for dn in (None, B):
+        mats = 1 if dn is None else 2
+        c, mo, st = apm.cdet_connected_varlen(A, ao, nt, A_dn=dn, return_minors=True, return_status=True)
+        for m in range(1, hi + 1):
+            at = torch.as_tensor(np.nonzero(orders == m)[0]).cuda()
+            if at.numel() == 0:
+                continue
+            sq = torch.arange(m * m, device="cuda")
+            x = A[ao[at][:, None] + sq].reshape(-1, m, m)
+            y = None if dn is None else B[ao[at][:, None] + sq].reshape(-1, m, m)
+            cr, mr, sr = apm.cdet_connected(x, y, return_minors=True, return_status=True)
+            S = torch.arange(1 << m, device="cuda")
+            got = c[co[at][:, None] + S]
+            assert np.array_equal(got.cpu().numpy(), cr.cpu().numpy(), equal_nan=True), m
+            S = torch.arange(mats << m, device="cuda")
+            got = mo[mats * co[at][:, None] + S].reshape(mr.shape)
+            assert np.array_equal(got.cpu().numpy(), mr.cpu().numpy(), equal_nan=True), m
+            assert torch.equal(st[at], sr), m
