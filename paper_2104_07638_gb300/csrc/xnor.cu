@@ -356,9 +356,12 @@ static size_t xn_smem(int S) {
 
 // Tail and runs per matrix (log2), by the warps a batch would otherwise leave
 // idle. The tree's operations do not depend on either: the same bits. us per call,
-// one warp per matrix before: order 10: 1 matrix 80 -> 23, 512 88 -> 71; order 12:
-// 1 326 -> 29, 512 355 -> 244; order 14: 1 1309 -> 35, 64 1370 -> 158. At order 8
-// a tail of 7 (more resident warps) lost to one of 8: 4096 matrices 109 against 91.
+// one warp per matrix before: order 10: 1 matrix 82 -> 21, 512 88 -> 68; order 12:
+// 1 325 -> 25, 512 356 -> 235; order 14: 1 1309 -> 35, 64 1370 -> 158. From 6 warps
+// per SM on matrices stay whole (at order 10 from 5): halves of more than the 10
+// resident warps per SM leave a second round (whole | halves, 912 of order 10
+// 97 | 115, of order 13 776 | 878; 1216 of order 12 443 | 481). At order 8 a tail of
+// 7 (more resident warps) lost to one of 8: 4096 matrices 109 against 91.
 struct XnShape {
     int S, kc;
 };
@@ -366,6 +369,7 @@ static XnShape xn_shape(int n, int64_t batch) {
     const int64_t fill = 152 * 6;
     XnShape s = {kXnTail, 0};
     if (n < 10) return s;  // no scratch at these orders
+    if (batch >= fill || (n == 10 && batch > 152 * 5)) return s;
     if ((batch << (n - 8)) < fill) s.S = (batch << (n - 7)) < fill ? 5 : 7;
     while (s.kc < n - s.S && (batch << s.kc) < 2 * fill) ++s.kc;
     return s;

@@ -119,3 +119,16 @@ def test_uneven_small_orders(apm, hi, batch):
             got = mo[mats * co[at][:, None] + S].reshape(mr.shape)
             assert np.array_equal(got.cpu().numpy(), mr.cpu().numpy(), equal_nan=True), m
             assert torch.equal(st[at], sr), m
+
+
+# XNOR minors: whole matrices from where halves would take a second round
+@pytest.mark.parametrize("n,batch", [(10, 760), (10, 761), (11, 911), (11, 912), (12, 1216)])
+def test_xnor_whole_from(apm, n, batch):
+    d = torch.as_tensor(I.nambu_batch(64, n, seed=9400 + n)).cuda()
+    few = apm.xnor_minors(d, return_status=True)
+    at = torch.arange(batch).cuda() % 64
+    big = apm.xnor_minors(d[at], return_status=True)
+    for g, r in zip(big, few):
+        assert torch.equal(g, r[at])
+    sizes = [apm.workspace_size(apm.OP_XNOR_MINORS, n, b) for b in (1, 200, 456, 760, 761, 911, 912, 1520, 3000)]
+    assert sizes == sorted(sizes)
