@@ -490,15 +490,27 @@ int keldysh_warps_per_block() { return kKelWarps; }
 // of them: as many chunks as that round holds (the FP64 units saturate at about 6
 // warps per SM, and a second round of smaller items costs more than it balances:
 // two-spin sums of order 12, 64 pairs, k = 3..6: 278, 181, 335, 374 us). Beyond:
-// enough items that the last, partial round is a small part, but not more than 4
-// chunks, whose paths the matrix then pays for (2200 pairs, k = 0..3: 6913, 5205,
-// 4434, 4597 us). Items <= warps for batch <= warps, < 9 warps otherwise.
+// the fewest rounds times what a round takes, the chunk's leaves and, for the path
+// and the sums of a chunk, 0.1 k of a leaf; whole matrices where nothing is gained
+// (us for k = 0..3: two-spin sums of order 10, 2200 pairs 1702, 1288, 1117, 1236,
+// 3300 1701, 1712, 1769, 1839, 3648 1706, 1714, 1772, 1962; single-spin sums of
+// order 12, 1900 matrices 3440, 2590, 2200, 2060). Chunks of fewer than 4 leaves
+// only where a matrix has few. Items <= warps for batch <= warps, <= 16 warps
+// otherwise.
 int keldysh_chunks(int64_t batch, int D, int64_t warps) {
     int k = 0;
     if (batch <= warps) {
         while (k < D && (batch << (k + 1)) <= warps) ++k;
-    } else {
-        while (k < 2 && k < D && 2 * (batch << k) < 9 * warps) ++k;
+        return k;
+    }
+    const int most = D < 3 ? D : D < 5 ? 2 : 3;
+    int64_t best = 0;
+    for (int q = 0; q <= most && (q == 0 || (batch << q) <= 16 * warps); ++q) {
+        const int64_t rounds = ((batch << q) + warps - 1) / warps, cost = rounds * ((int64_t(10) << (D - q)) + q);
+        if (q == 0 || cost < best) {
+            best = cost;
+            k = q;
+        }
     }
     return k;
 }

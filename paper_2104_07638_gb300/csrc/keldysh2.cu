@@ -411,7 +411,7 @@ size_t keldysh2_workspace_bytes(int n, int64_t batch, int *err) {
     K2Plan p;
     *err = k2_plan(n, batch, &p);
     if (*err) return 0;
-    const int64_t warps = 152 * kK2Warps, items = batch <= warps ? warps : 9 * warps;
+    const int64_t warps = 152 * kK2Warps, items = batch <= warps ? warps : 16 * warps;
     const size_t split = static_cast<size_t>(warps) * k2_stack_entries(n) * sizeof(double2) +
                          static_cast<size_t>(items) * ((n + 1) * sizeof(double2) + 2 * sizeof(uint32_t)) + 64;
     return p.total > split ? p.total : split;

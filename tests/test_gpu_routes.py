@@ -8,6 +8,7 @@ import numpy as np
 import pytest
 import torch
 
+import oracle
 from paper_2104_07638_gb300 import inputs as I
 
 pytestmark = pytest.mark.gpu
@@ -132,3 +133,30 @@ def test_xnor_whole_from(apm, n, batch):
         assert torch.equal(g, r[at])
     sizes = [apm.workspace_size(apm.OP_XNOR_MINORS, n, b) for b in (1, 200, 456, 760, 761, 911, 912, 1520, 3000)]
     assert sizes == sorted(sizes)
+
+
+# Keldysh sums of batches above one round of warps: whole where splitting gains no
+# round (then also bit for bit the same matrices of the uneven batch), else split;
+# against a batch of one (other chunks: a rounding apart)
+@pytest.mark.parametrize("n,batch,whole", [(10, 2736, False), (10, 3648, True), (11, 3300, True), (12, 1900, False)])
+def test_keldysh_rounds(apm, n, batch, whole):
+    d = torch.as_tensor(I.keldysh_batch(32, n, seed=9500 + n)).cuda()
+    at = torch.arange(batch).cuda() % 32
+    s, p = apm.keldysh_sum(d[at], partial=True)
+    assert torch.equal(s, s[at]) and torch.equal(p, p[at])
+    o = torch.arange(32).cuda() * (4 * n * n)
+    u = apm.keldysh_sum_varlen(d.reshape(-1), o, torch.full((32,), n, dtype=torch.int32, device="cuda"))
+    if whole:
+        assert torch.equal(s[:32], u)
+    scale = torch.as_tensor(oracle.keldysh_scale(d.cpu().numpy())).cuda()
+    one = apm.keldysh_sum(d[:1])
+    assert bool((abs(s[:32] - u) <= 1e-10 * scale).all()) and bool((abs(s[:1] - one) <= 1e-10 * scale[:1]).all())
+
+
+@pytest.mark.parametrize("n,batch", [(8, 3000), (8, 3648), (9, 5472)])
+def test_keldysh2_rounds(apm, n, batch):
+    u, d = (torch.as_tensor(x).cuda() for x in I.keldysh2_batch(32, n, seed=9600 + n))
+    at = torch.arange(batch).cuda() % 32
+    s, p = apm.keldysh2_sum(u[at], d[at], partial=True)
+    w, q = apm.keldysh2_sum(u[at[:1824]], d[at[:1824]], partial=True)    # one round of whole pairs
+    assert torch.equal(s[:1824], w) and torch.equal(p[:1824], q) and torch.equal(s, s[at])
