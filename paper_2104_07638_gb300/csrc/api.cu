@@ -563,12 +563,9 @@ apm_status_t apm_workspace_size(int op, int n_max, int64_t batch, int two_mats, 
         }
         case APM_OP_KELDYSH: {
             if (n_max < 1 || n_max > APM_MAX_N_KELDYSH) return APM_ERR_UNSUPPORTED_N;
-            if (apm::keldysh_stack_entries(n_max) == 0 || batch == 0) return APM_OK;
-            apm::KeldyshPlan p;
-            const int err = apm::keldysh_plan(n_max, batch, &p);
-            if (err) return cuda_fail(err);
-            *bytes = p.total;
-            return APM_OK;
+            int err = 0;
+            *bytes = apm::keldysh_workspace_bytes(n_max, batch, &err);
+            return err ? cuda_fail(err) : APM_OK;
         }
         case APM_OP_XNOR_MINORS:
         case APM_OP_NAMBU_CDET: {

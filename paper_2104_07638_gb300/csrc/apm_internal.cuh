@@ -192,6 +192,8 @@ int keldysh_grid(int64_t batch, int *err);
 int keldysh_warps_per_block();
 int keldysh_spread(int64_t items);
 int keldysh_chunks(int64_t batch, int D, int64_t warps);
+size_t keldysh_scratch(int n, int64_t batch, int D, int64_t warps, size_t entries);
+size_t keldysh_workspace_bytes(int n, int64_t batch, int *err);
 size_t keldysh_stack_entries(int n);
 
 int launch_ppm(const double *A, int n, int64_t batch, double *perms, cudaStream_t s);

@@ -515,6 +515,30 @@ int keldysh_chunks(int64_t batch, int D, int64_t warps) {
     return k;
 }
 
+// Scratch of a fixed-order launch that serves every batch up to this one (a smaller
+// batch may be split into more chunks): path stacks of `entries` for as many warps
+// as their items occupy, and a slot, a flag and a counter for the most items of a
+// split batch (keldysh_chunks).
+size_t keldysh_scratch(int n, int64_t batch, int D, int64_t warps, size_t entries) {
+    const int64_t most = batch <= warps ? warps : 16 * warps;
+    const int64_t items = batch < most && (batch << D) < most ? batch << D : most;
+    const int64_t used = items + kKelWarps < warps ? items + kKelWarps : warps;
+    return static_cast<size_t>(used) * entries * sizeof(double2) +
+           static_cast<size_t>(items) * ((n + 1) * sizeof(double2) + 2 * sizeof(uint32_t)) + 64;
+}
+
+size_t keldysh_workspace_bytes(int n, int64_t batch, int *err) {
+    *err = 0;
+    if (batch == 0 || kel_stack_entries(n) == 0) return 0;
+    KeldyshPlan p;
+    *err = keldysh_plan(n, batch, &p);
+    if (*err) return 0;
+    if (n <= kKelTail + 2) return p.total;  // never split
+    const int64_t warps = static_cast<int64_t>(keldysh_grid(INT64_MAX / 64, err)) * kKelWarps;
+    if (*err) return 0;
+    return keldysh_scratch(n, batch, n - kKelTail, warps, kel_stack_entries(n));
+}
+
 int keldysh_plan(int n, int64_t batch, KeldyshPlan *p) {
     int err = 0;
     const int full = keldysh_grid(INT64_MAX / 64, &err);  // all resident CTAs

@@ -160,3 +160,20 @@ def test_keldysh2_rounds(apm, n, batch):
     s, p = apm.keldysh2_sum(u[at], d[at], partial=True)
     w, q = apm.keldysh2_sum(u[at[:1824]], d[at[:1824]], partial=True)    # one round of whole pairs
     assert torch.equal(s[:1824], w) and torch.equal(p[:1824], q) and torch.equal(s, s[at])
+
+
+# scratch sized for a batch serves every smaller one, split into more chunks or not
+@pytest.mark.parametrize("n", [9, 10, 11, 12, 14])
+def test_keldysh_scratch_serves_smaller_batches(apm, n):
+    bs = sorted({1, 2, 3, 57, 228, 300, 456, 500, 911, 912, 913, 1000, 1824, 1825, 2052, 3648, 7296, 14592, 14593,
+                 40000} | set(range(1, 4000, 61)))
+    sizes = [apm.workspace_size(apm.OP_KELDYSH, n, b) for b in bs]
+    assert sizes == sorted(sizes)
+    M = torch.as_tensor(I.keldysh_batch(300, n, seed=9700 + n)).cuda()
+    nb = apm.workspace_size(apm.OP_KELDYSH, n, 500)
+    ws = torch.empty(nb, dtype=torch.uint8, device="cuda")
+    for b in (1, 57, 300):
+        s = torch.empty((b, 2), dtype=torch.float64, device="cuda")
+        apm._check(apm.lib().apm_keldysh_sum(apm._ptr(M), n, b, 0, apm._ptr(s), None, None, apm._ptr(ws), nb,
+                                             apm._stream(M)), "apm_keldysh_sum")
+        assert torch.equal(torch.view_as_complex(s), apm.keldysh_sum(M[:b]))
