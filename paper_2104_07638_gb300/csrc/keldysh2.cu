@@ -406,15 +406,11 @@ static int k2_plan(int n, int64_t batch, K2Plan *p) {
 size_t keldysh2_workspace_bytes(int n, int64_t batch, int *err) {
     *err = 0;
     if (k2_stack_entries(n) == 0 || batch == 0) return 0;
-    // not less than for any smaller batch: a stack for every resident warp, and
-    // slots for the most items of a split batch (keldysh_chunks)
-    K2Plan p;
-    *err = k2_plan(n, batch, &p);
+    const int64_t warps = static_cast<int64_t>(resident_ctas(keldysh2_kernel, kK2Warps * 32,
+                                                             kK2Warps * sizeof(K2WarpSmem),
+                                                             kK2Warps * sizeof(K2WarpSmem), err)) * kK2Warps;
     if (*err) return 0;
-    const int64_t warps = 152 * kK2Warps, items = batch <= warps ? warps : 16 * warps;
-    const size_t split = static_cast<size_t>(warps) * k2_stack_entries(n) * sizeof(double2) +
-                         static_cast<size_t>(items) * ((n + 1) * sizeof(double2) + 2 * sizeof(uint32_t)) + 64;
-    return p.total > split ? p.total : split;
+    return keldysh_scratch(n, batch, n - kK2Tail, warps, k2_stack_entries(n));
 }
 
 int launch_keldysh2(const double *Mu, const double *Md, int n, int64_t batch, int sgn, double *sum,

@@ -177,3 +177,23 @@ def test_keldysh_scratch_serves_smaller_batches(apm, n):
         apm._check(apm.lib().apm_keldysh_sum(apm._ptr(M), n, b, 0, apm._ptr(s), None, None, apm._ptr(ws), nb,
                                              apm._stream(M)), "apm_keldysh_sum")
         assert torch.equal(torch.view_as_complex(s), apm.keldysh_sum(M[:b]))
+
+
+# scratch of a few two-spin pairs: stacks for the warps they can occupy, no more,
+# and one that serves every smaller batch
+@pytest.mark.parametrize("n,most", [(8, 0.2e6), (10, 0.8e6), (12, 4.2e6), (14, 27e6), (16, 155e6)])
+def test_keldysh2_scratch(apm, n, most):
+    assert apm.workspace_size(apm.OP_KELDYSH2, n, 1) <= most
+    bs = sorted({1, 2, 7, 28, 57, 300, 1824, 1825, 3648, 14592, 14593, 40000} | set(range(1, 4000, 61)))
+    sizes = [apm.workspace_size(apm.OP_KELDYSH2, n, b) for b in bs]
+    assert sizes == sorted(sizes)
+    if n > 10:
+        return
+    u, d = (torch.as_tensor(x).cuda() for x in I.keldysh2_batch(300, n, seed=9800 + n))
+    nb = apm.workspace_size(apm.OP_KELDYSH2, n, 500)
+    ws = torch.empty(nb, dtype=torch.uint8, device="cuda")
+    for b in (1, 57, 300):
+        s = torch.empty((b, 2), dtype=torch.float64, device="cuda")
+        apm._check(apm.lib().apm_keldysh2_sum(apm._ptr(u), apm._ptr(d), n, b, 0, apm._ptr(s), None, None, apm._ptr(ws),
+                                              nb, apm._stream(u)), "apm_keldysh2_sum")
+        assert torch.equal(torch.view_as_complex(s), apm.keldysh2_sum(u[:b], d[:b]))
