@@ -1490,6 +1490,14 @@ static int varlen_region(int n_max, int64_t batch, bool two_mats, int grid, size
     return 0;
 }
 
+// Rows of terms of the items done by blocks: as many as all items would take, were
+// they of the largest such order (a batch too large for blocks: the most a smaller
+// one takes).
+static int64_t varlen_split_rows(int n_max, int64_t batch) {
+    const int to = n_max < g_fsc_from_n ? n_max : g_fsc_from_n - 1;
+    return batch <= kVarlenSplitMax ? cdet_split_rows(to, batch) : kSplitMaxRows;
+}
+
 size_t cdet_varlen_workspace(int n_max, int64_t batch, bool two_mats, int *err) {
     *err = 0;
     size_t bytes = 256 + align256(static_cast<size_t>(batch) * sizeof(int));
@@ -1501,7 +1509,8 @@ size_t cdet_varlen_workspace(int n_max, int64_t batch, bool two_mats, int *err) 
     if (*err) return 0;
     bytes += region * sizeof(double);
     if (warp_route_from(n_max, two_mats))
-        bytes += align256(static_cast<size_t>(batch)) + static_cast<size_t>(kSplitMaxRows << kBlkB) * sizeof(double);
+        bytes += align256(static_cast<size_t>(batch)) +
+                 static_cast<size_t>(varlen_split_rows(n_max, batch) << kBlkB) * sizeof(double);
     return bytes;
 }
 
@@ -1559,7 +1568,7 @@ int launch_cdet_varlen(const CdetArgs &a, const int64_t *a_off, const int *n_arr
         Q.c_off = c_off;
         Q.flag = wflag;
         Q.rows = slots + region;
-        Q.cap = kSplitMaxRows;
+        Q.cap = varlen_split_rows(n_max, a.batch);
         Q.batch = a.batch;
         Q.gsel = cdet_gsel_packed(kBlkB);
         for (int m = split_to; m > kVarlenSmemMaxN; --m) {

@@ -197,3 +197,17 @@ def test_keldysh2_scratch(apm, n, most):
         apm._check(apm.lib().apm_keldysh2_sum(apm._ptr(u), apm._ptr(d), n, b, 0, apm._ptr(s), None, None, apm._ptr(ws),
                                               nb, apm._stream(u)), "apm_keldysh2_sum")
         assert torch.equal(torch.view_as_complex(s), apm.keldysh2_sum(u[:b], d[:b]))
+
+
+# scratch of an uneven batch: rows of terms for the items there are, not 64 MB for
+# any two, and enough for every smaller batch
+@pytest.mark.parametrize("n_max", [13, 14, 15, 16])
+def test_uneven_scratch(apm, n_max):
+    slots = 456 * (3 << n_max) * 8                       # three CTAs per SM
+    most = {13: 9, 14: 28, 15: 75, 16: 75}[n_max] * 8192     # bytes of rows per item
+    for b in (1, 2, 4):
+        size = apm.workspace_size(apm.OP_CDET_VARLEN, n_max, b)
+        assert slots <= size <= slots + b * most + 1024
+    bs = sorted({1, 2, 8, 100, 109, 110, 292, 293, 910, 911, 1024, 1025, 5000, 70000} | set(range(1, 1200, 37)))
+    sizes = [apm.workspace_size(apm.OP_CDET_VARLEN, n_max, b) for b in bs]
+    assert sizes == sorted(sizes)
