@@ -1194,31 +1194,42 @@ void cdet_tune_set(const unsigned long long *table) {
     for (int n = 0; n <= 16; ++n) g_tuned[n] = table ? table[n] : 0ull;
 }
 
-// Threads of a CTA (one matrix) at order n <= 12. A small order's phases have
+// Threads of a CTA at order n <= 12. A small order's phases have
 // too little to do for 256 threads, and every barrier of its tree and its layers
 // stops the whole CTA: more, smaller CTAs on an SM (its registers hold 768
 // threads of this kernel in any case) fill each other's waits. Wide CTAs are the
-// faster only while one round of them holds the batch. Measured, us per call
-// (256 | 128 | 64 threads; host side of 11 us included):
-//   n = 8:  300 matrices 19 | 19 | 21, 1200 51 | 39 | 26, 65536 2224 | 1173 | 1048
-//   n = 9:  300 24 | 25 | 33, 777 47 | 37 | 41, 1200 68 | 61 | 47, 16384 755 | 555 | 543
-//   n = 10: 456 46 | 49 | 62, 777 86 | 76 | 82, 1200 125 | 119 | 99, 2000 197 | 170 | 179,
-//           16384 1447 | 1258 | 1255
-//   n = 11: 456 103 | 111 | 146, 2000 459 | 443 | 525, 16384 3497 | 3303 | 3436
+// faster only while one round of them holds the batch, or where it fills their last
+// round and not the narrow ones'. Measured, us per call (256 | 128 | 64 threads;
+// device time):
+//   n = 8:  304 matrices 17 | 17 | 18, 1216 46 | 35 | 24, 16384 511 | 284 | 256
+//   n = 9:  304 22 | 22 | 28, 777 46 | 35 | 38, 1216 67 | 57 | 44, 16384 740 | 539 | 526
+//   n = 10: 456 43 | 46 | 52, 777 82 | 74 | 76, 1216 121 | 111 | 94, 1500 152 | 129 | 115,
+//           1672 160 | 140 | 158, 2000 191 | 165 | 170, 16384 1413 | 1240 | 1223
+//   n = 11: 456 99 | 104 | 122, 912 194 | 185 | 191, 1368 286 | 301 | 331, 2000 441 | 424 | 477,
+//           16384 3315 | 3233 | 3299
 //   n = 12: 456 256 | 270 | 353, 16384 8864 | 9299 | 12462
-static int cdet_threads(int n, int64_t batch) {
+// With a second matrix the arrays of a narrow CTA leave room for 7 (n = 10, 64
+// threads) or 4 on an SM (n = 11, 128 threads) instead of 10 and 6:
+//   n = 10: 1216 158 | 142 | 164, 1672 209 | 176 | 188, 16384 1849 | 1542 | 1593
+//   n = 11: 608 200 | 151 | 176, 912 232 | 271 | 321, 1216 343 | 298 | 337, 1368 344 | 391 | 466,
+//           2736 678 | 710 | 802, 3648 899 | 886 | 984
+static int cdet_threads(int n, int64_t batch, bool two_mats) {
     if (n > 11) return kCdetThreads;
     const int64_t round = 3 * 152;  // resident CTAs of 256 threads
     if (n <= 8) return batch <= 2 * round ? 128 : 64;
     if (batch <= round) return kCdetThreads;
     if (n == 9) return batch <= 2 * round ? 128 : 64;
-    if (n == 10) return batch > 2 * round && batch <= 11 * 152 ? 64 : 128;
-    return 128;
+    if (n == 10) return !two_mats && batch > 2 * round && batch <= 10 * 152 ? 64 : 128;
+    if (two_mats) {  // a round of 4 x 152 narrow CTAs takes 5 / 4 of one of wide ones
+        const int64_t wide = (batch + round - 1) / round, narrow = (batch + 4 * 152 - 1) / (4 * 152);
+        return 4 * wide <= 5 * narrow ? kCdetThreads : 128;
+    }
+    return batch > 8 * 152 && batch <= 9 * 152 ? kCdetThreads : 128;
 }
 
 int cdet_grid(int n, int64_t batch, bool two_mats, bool smem_arrays, int *err) {
     const size_t smem = cdet_smem_bytes(n, two_mats, smem_arrays);
-    int64_t g = smem_arrays ? resident_ctas(fpm_cdet_kernel<true>, cdet_threads(n, batch), smem,
+    int64_t g = smem_arrays ? resident_ctas(fpm_cdet_kernel<true>, cdet_threads(n, batch, two_mats), smem,
                                             cdet_smem_bytes(cdet_smem_max_n(true), true, true), err)
                             : resident_ctas(fpm_cdet_kernel<false>, kCdetThreads, smem, smem, err);
     if (*err) return 0;
@@ -1398,7 +1409,7 @@ int launch_fpm_cdet(const CdetArgs &a, cudaStream_t s) {
         if (lc) return launch_cdet_cluster(P, lc, s);
     }
     if (smem_arrays)
-        fpm_cdet_kernel<true><<<grid, cdet_threads(a.n, a.batch), smem, s>>>(P);
+        fpm_cdet_kernel<true><<<grid, cdet_threads(a.n, a.batch, a.two_mats != 0), smem, s>>>(P);
     else
         fpm_cdet_kernel<false><<<grid, kCdetThreads, smem, s>>>(P);
     err = static_cast<int>(cudaGetLastError());

@@ -211,3 +211,18 @@ def test_uneven_scratch(apm, n_max):
     bs = sorted({1, 2, 8, 100, 109, 110, 292, 293, 910, 911, 1024, 1025, 5000, 70000} | set(range(1, 1200, 37)))
     sizes = [apm.workspace_size(apm.OP_CDET_VARLEN, n_max, b) for b in bs]
     assert sizes == sorted(sizes)
+
+
+# the CTA's width at orders 10 and 11, one matrix and two
+@pytest.mark.parametrize("n,batch", [(10, 1520), (10, 1521), (11, 608), (11, 609), (11, 912), (11, 913), (11, 1216),
+                                     (11, 1217), (11, 1368), (11, 1369)])
+def test_cta_widths(apm, n, batch):
+    few = 200                                        # one round of wide CTAs
+    A = torch.as_tensor(I.gaussian_plus_2I(n, few, seed=n)).cuda()
+    B = torch.as_tensor(I.hubbard_batch(few, n, seed=n)).cuda()
+    at = torch.arange(batch).cuda() % few
+    for y in (None, A):
+        ref = apm.cdet_connected(B, y, return_minors=True, return_status=True)
+        got = apm.cdet_connected(B[at], None if y is None else y[at], return_minors=True, return_status=True)
+        for g, r in zip(got, ref):
+            assert torch.equal(g, r[at])
