@@ -407,15 +407,16 @@ static int lanes_most(int n) { return n < 4 ? 2 : n == 4 ? 3 : 4; }
 
 // Lanes per matrix (log2) at order n and this batch, or -1 for the
 // one-CTA-per-matrix kernel (of 64 or 128 threads here). Both sides measured on
-// a GB300, us per call with the host side of about 11 us in it (CTA | this):
-//   minors and sums: n = 5: 1200 matrices 14 | 15, 2000 19 | 17, 65536 410 | 72
-//     n = 6: 1200 15 | 21, 2000 22 | 23, 3000 30 | 25, 65536 498 | 148
-//     n = 7: 4096 51 | 62, 6000 74 | 64, 65536 706 | 355
-//     n = 8: 4096 74 | 97, 16384 267 | 278, 65536 1048 | 918
-//   minors: n = 6: 3500 25 | 18, 65536 375 | 68;  n = 7: 8000 60 | 35, 65536 433 | 140
-//     n = 8: 8000 70 | 83, 12000 98 | 88, 65536 514 | 323
-//   sums from weights: n = 6: 4096 17 | 21, 9000 25 | 23, 65536 146 | 78
-//     n = 7: 16384 74 | 72, 65536 282 | 205;  n = 8: 65536 537 | 595
+// a GB300, device us per call (CTA | this):
+//   minors and sums: n = 4: 457 matrices 8.7 | 8.8;  n = 5: 1500 14.4 | 15.3, 2000 18 | 16, 16384 105 | 24
+//     n = 6: 2000 20.7 | 21.6, 2300 25.6 | 21.8, 16384 126 | 48
+//     n = 7: 4096 49 | 60, 5500 64 | 65, 6000 71 | 65, 16384 175 | 128
+//     n = 8: 16384 255 | 276, 20000 312 | 341, 24000 374 | 359, 65536 1018 | 921
+//   minors: n = 5: 1824 12 | 12, 2300 15 | 11;  n = 6: 2000 15 | 14, 8000 50 | 17;  n = 7: 3648 28 | 27,
+//     4096 30 | 32, 6000 44 | 36;  n = 8: 9000 72 | 81, 11000 88 | 86, 16384 129 | 113
+//   sums from weights: n = 4: 1500 5.6 | 5.9, 2300 8.3 | 6.0;  n = 5: 2100 7.0 | 8.9, 2200 10.0 | 8.9, 3200 10.3 | 9.6
+//     n = 6: 8000 23 | 28, 11000 29 | 31, 13000 34 | 31, 16384 41 | 31
+//     n = 7: 12000 52 | 51, 14000 60 | 77, 18000 75 | 80, 24000 97 | 87, 65536 266 | 205;  n = 8: 65536 489 | 596
 // (256-thread CTAs took 1220, 1581 and 2210 us on 65536 of order 6, 7 and 8.)
 // As few lanes per matrix as fill the chip (6 warps per SM) waste the fewest;
 // below `least` lanes a warp's arrays leave too few warps per SM (n = 8, 65536:
@@ -423,9 +424,9 @@ static int lanes_most(int n) { return n < 4 ? 2 : n == 4 ? 3 : 4; }
 int cdet_lanes_log2(int n, int64_t batch, int mode) {
     if (n > kLanesMaxN) return -1;
     static const int from[3][kLanesMaxN + 1] = {
-        {0, 0, 0, 0, 456, 2500, 2500, 5000, 10000},       // minors
-        {0, 0, 0, 0, 456, 1500, 2200, 5500, 20000},       // minors and sums
-        {0, 0, 0, 0, 456, 4000, 8000, 16000, 1 << 30}};   // sums from weights
+        {0, 0, 0, 0, 457, 2000, 2000, 5000, 10500},        // minors
+        {0, 0, 0, 0, 457, 1800, 2200, 5600, 22000},        // minors and sums
+        {0, 0, 0, 0, 1900, 2200, 11500, 20000, 1 << 30}};  // sums from weights
     if (batch < from[mode][n]) return -1;
     const int least = mode == kModeMinors ? (n > 6 ? n - 6 : 0) : (n > 5 ? n - 5 : n == 5 ? 1 : 0);
     int lg = least;

@@ -226,3 +226,24 @@ def test_cta_widths(apm, n, batch):
         got = apm.cdet_connected(B[at], None if y is None else y[at], return_minors=True, return_status=True)
         for g, r in zip(got, ref):
             assert torch.equal(g, r[at])
+
+
+# both sides of the lines between CTAs and lane groups
+@pytest.mark.parametrize("n,lines", [(4, (457, 1900)), (5, (1800, 2000, 2200)), (6, (2000, 2200, 11500)),
+                                     (7, (5000, 5600, 20000)), (8, (10500, 22000))])
+def test_lane_group_lines(apm, n, lines):
+    A = torch.as_tensor(I.gaussian_plus_2I(n, 64, seed=40 + n)).cuda()
+    A[3] = 0.0
+    A[5, 0, 1] = float("nan")
+    c, m, st = (x.nan_to_num(nan=1.5e300) if x.is_floating_point() else x
+                for x in apm.cdet_connected(A, return_minors=True, return_status=True))
+    w = apm.all_minors(A[6:])
+    cw = apm.cdet_from_weights(w)
+    for b in (x + y for x in lines for y in (-1, 0)):
+        at = torch.arange(b).cuda() % 64
+        got = apm.cdet_connected(A[at], return_minors=True, return_status=True)
+        for g, r in zip(got, (c, m, st)):
+            assert torch.equal(g.nan_to_num(nan=1.5e300) if g.is_floating_point() else g, r[at])
+        assert torch.equal(apm.all_minors(A[at]).nan_to_num(nan=1.5e300), m[at])
+        at = torch.arange(b).cuda() % 58
+        assert torch.equal(apm.cdet_from_weights(w[at]), cw[at])
