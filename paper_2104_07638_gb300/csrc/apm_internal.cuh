@@ -67,8 +67,9 @@ int cdet_smem_max_n(bool two_mats);
 // Bytes of dynamic shared memory of the minor / connected-sum kernel.
 size_t cdet_smem_bytes(int n, bool two_mats, bool smem_arrays);
 
-// Grid size used for a fixed-order launch (also sizes the workspace).
-int cdet_grid(int n, int64_t batch, bool two_mats, bool smem_arrays, int *err);
+// Grid size used for a fixed-order launch (also sizes the workspace); threads per
+// CTA at orders up to 12, 0 for those the order and the batch decide.
+int cdet_grid(int n, int64_t batch, bool two_mats, bool smem_arrays, int *err, int threads = 0);
 
 // Bytes of global scratch of a fixed-order connected-sum launch above order 12:
 // the CTAs' slots, and rows for the terms of few matrices' blocks.

@@ -1227,9 +1227,10 @@ static int cdet_threads(int n, int64_t batch, bool two_mats) {
     return batch > 8 * 152 && batch <= 9 * 152 ? kCdetThreads : 128;
 }
 
-int cdet_grid(int n, int64_t batch, bool two_mats, bool smem_arrays, int *err) {
+int cdet_grid(int n, int64_t batch, bool two_mats, bool smem_arrays, int *err, int threads) {
     const size_t smem = cdet_smem_bytes(n, two_mats, smem_arrays);
-    int64_t g = smem_arrays ? resident_ctas(fpm_cdet_kernel<true>, cdet_threads(n, batch, two_mats), smem,
+    if (threads == 0) threads = cdet_threads(n, batch, two_mats);
+    int64_t g = smem_arrays ? resident_ctas(fpm_cdet_kernel<true>, threads, smem,
                                             cdet_smem_bytes(cdet_smem_max_n(true), true, true), err)
                             : resident_ctas(fpm_cdet_kernel<false>, kCdetThreads, smem, smem, err);
     if (*err) return 0;
@@ -1350,7 +1351,10 @@ int launch_fpm_cdet(const CdetArgs &a, cudaStream_t s) {
     P.gsel = cdet_gsel_packed(a.n);
     P.gsel_b = cdet_gsel_packed(kBlkB);
     const bool smem_arrays = a.n <= cdet_smem_max_n(a.two_mats != 0);
-    const int grid = cdet_grid(a.n, a.batch, a.two_mats != 0, smem_arrays, &err);
+    // (a redo launch, which usually finds nothing to do, in the fewest CTAs: the
+    // 12 per SM of 64 threads cost minors of 4096 matrices of order 9 1.4 of 43 us)
+    const int threads = a.redo_list ? kCdetThreads : cdet_threads(a.n, a.batch, a.two_mats != 0);
+    const int grid = cdet_grid(a.n, a.batch, a.two_mats != 0, smem_arrays, &err, threads);
     if (err) return err;
     const size_t smem = cdet_smem_bytes(a.n, a.two_mats != 0, smem_arrays);
     const bool fsc = a.mode == kModeCdet && a.n >= g_fsc_from_n;
@@ -1409,7 +1413,7 @@ int launch_fpm_cdet(const CdetArgs &a, cudaStream_t s) {
         if (lc) return launch_cdet_cluster(P, lc, s);
     }
     if (smem_arrays)
-        fpm_cdet_kernel<true><<<grid, cdet_threads(a.n, a.batch, a.two_mats != 0), smem, s>>>(P);
+        fpm_cdet_kernel<true><<<grid, threads, smem, s>>>(P);
     else
         fpm_cdet_kernel<false><<<grid, kCdetThreads, smem, s>>>(P);
     err = static_cast<int>(cudaGetLastError());
