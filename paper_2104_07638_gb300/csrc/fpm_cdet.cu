@@ -87,7 +87,8 @@ struct VarlenParams {
     unsigned *ctr;                 // work counter, zeroed by varlen_order_kernel
     int smem_max_n;
     int n_max;
-    int split_to;                  // unflagged items of orders smem_max_n + 1 .. split_to are done elsewhere
+    int split_to;                  // unflagged items of orders smem_max_n + 1 .. split_to are done elsewhere,
+    const unsigned *split_on;      // if this word is not 0
     unsigned long long gsel[17];   // lane-group table per order
 };
 
@@ -840,12 +841,13 @@ struct SplitArgs {
     const int *order;
     const int64_t *c_off;
     const unsigned *first, *count;
+    const unsigned *on;  // 0: the persistent kernel takes all of them (varlen_split_pays)
     const uint8_t *flag;
     double *rows;  // scratch rows of 2^kBlkB doubles, `cap` of them
     int64_t cap, batch;
     int n;
     unsigned long long gsel;
-    __device__ __forceinline__ int64_t items() const { return order ? static_cast<int64_t>(*count) : batch; }
+    __device__ __forceinline__ int64_t items() const { return order ? (*on ? static_cast<int64_t>(*count) : 0) : batch; }
     __device__ __forceinline__ int64_t item(int64_t i) const { return order ? order[static_cast<int64_t>(*first) + i] : i; }
     __device__ __forceinline__ bool skip(int64_t i) const { return order && flag[item(i)]; }
     __device__ __forceinline__ double *out(int64_t i) const { return order ? c + c_off[item(i)] : c + (i << n); }
@@ -1058,7 +1060,7 @@ __global__ void __launch_bounds__(kCdetThreads, 3) fpm_cdet_varlen_kernel(const 
             if (threadIdx.x == 0 && p.status) p.status[b] = APM_ST_BAD_ORDER;
             continue;
         }
-        if (n > V.smem_max_n && n <= V.split_to && !p.wflag[b]) continue;
+        if (n > V.smem_max_n && n <= V.split_to && *V.split_on && !p.wflag[b]) continue;
         const int N = 1 << n;
         const int NC = N > 16 ? N : 16;
         const bool in_smem = n <= V.smem_max_n;
@@ -1076,11 +1078,43 @@ __global__ void __launch_bounds__(kCdetThreads, 3) fpm_cdet_varlen_kernel(const 
     if (threadIdx.x == 0) bulk_wait_all();
 }
 
+// Whether the items of orders 13..to of an uneven batch go by blocks on many CTAs,
+// order after order, or all orders together with one CTA per matrix. Each side's
+// time from hist, the items per order: of the first a launch's fixed part and a part
+// per item; of the second what its work takes on 3 CTAs per SM, but not less than
+// the rounds of any one order, whose last takes less with fewer CTAs on an SM.
+// 4 % in favour of the second. Measured, us per call (blocks | one CTA per matrix):
+//   orders 13, 14: 100 items 656 | 1125, 456 1885 | 2256, 912 3483 | 3064
+//   order 13: 100 308 | 404, 300 651 | 559, 500 1038 | 1288, 912 1761 | 1571
+//   orders 13..15: 456 3993 | 6584, 1024 7924 | 7162;  4..14: 1024 1181 | 2230
+__device__ int varlen_split_pays(const int *hist, int64_t batch, int to) {
+    constexpr int kCtas = 456;  // 3 per SM
+    // orders 13..16 (16 only where the recursion takes it): us at 1, 2, 3 per SM; us, 10 ns
+    constexpr int kWhole[4][3] = {{404, 557, 797}, {1093, 1571, 2288}, {3137, 4585, 6650}, {12450, 14840, 19650}};
+    constexpr int kFixed[4] = {150, 250, 400, 300}, kItem[4] = {175, 485, 1430, 4250};
+    const int low = (256 * hist[12] + 99 * hist[11] + 43 * hist[10] + 25 * hist[9]) / kCtas;
+    const int depth = batch <= 152 ? 0 : batch <= 304 ? 1 : 2;
+    int blocks = low, work = 0, least = 0;
+    for (int m = 13; m <= to; ++m) {
+        const int c = hist[m], i = m - 13;
+        if (c == 0) continue;
+        blocks += kFixed[i] + kItem[i] * c / 100;
+        work += kWhole[i][2] * c;
+        const int full = c / kCtas, rest = c - full * kCtas;
+        const int rounds = full * kWhole[i][2] + (rest ? kWhole[i][(rest - 1) / 152] : 0);
+        least = max(least, max(rounds, kWhole[i][depth]));
+    }
+    return 104 * blocks <= 100 * max(work / kCtas + low, least);
+}
+
 // Longest-first order of an uneven batch: counting sort by decreasing order n
 // (one CTA), and reset of the work counter of the consumer kernel; per order m
-// the first index and the count of its items (ctr[2 + 2m], ctr[3 + 2m]).
+// the first index and the count of its items (ctr[2 + 2m], ctr[3 + 2m]), and the
+// choice of varlen_split_pays for orders 13..split_to (ctr[kCtrSplit]).
+constexpr int kCtrSplit = 36;
 __global__ void __launch_bounds__(1024) varlen_order_kernel(const int *__restrict__ n_arr, int64_t batch,
-                                                            int n_max, int *order, unsigned *ctr, int fsc_from_n) {
+                                                            int n_max, int *order, unsigned *ctr, int fsc_from_n,
+                                                            int split_to) {
     __shared__ int hist[18];
     __shared__ int start[18];
     if (threadIdx.x < 18) hist[threadIdx.x] = 0;
@@ -1103,6 +1137,7 @@ __global__ void __launch_bounds__(1024) varlen_order_kernel(const int *__restric
         int nf = 0;
         for (int n = fsc_from_n; n <= 16; ++n) nf += hist[n];
         ctr[1] = static_cast<unsigned>(nf);
+        ctr[kCtrSplit] = split_to ? static_cast<unsigned>(varlen_split_pays(hist, batch, split_to)) : 0u;
         for (int n = 0; n <= 16; ++n) {
             ctr[2 + 2 * n] = static_cast<unsigned>(start[n]);
             ctr[3 + 2 * n] = static_cast<unsigned>(hist[n]);
@@ -1445,12 +1480,12 @@ static int varlen_threads(int n_max, int64_t batch) {
     if (n_max == 11) return batch < 3300 ? kCdetThreads : 128;
     return kCdetThreads;
 }
-// Largest uneven batch whose items of orders 13..15 go by blocks on many CTAs: a
-// CTA takes 4 ms for one of order 15 by itself, which is the whole call then
+// Largest uneven batch whose items of orders 13..15 may go by blocks on many CTAs: a
+// CTA takes 3 to 4 ms for one of order 15 by itself, which is the whole call then
 // (300 walkers of orders 4..14 1672 -> 818 us, 100 of 10..16 3872 -> 1764, 1000 of
-// 4..16 9174 -> 5078).
-// Their weights, 2^15 doubles each at most, fit the region of the slots (456 x 3
-// times the largest order's).
+// 4..16 9174 -> 5078). Whether they do: varlen_split_pays, on the device, where the
+// orders are. Their weights, 2^15 doubles each at most, fit the region of the slots
+// (456 x 3 times the largest order's).
 constexpr int64_t kVarlenSplitMax = 1024;
 // The order a CTA's shared arrays hold: the largest present rather than 12 leaves
 // room for the narrow CTAs.
@@ -1530,8 +1565,8 @@ size_t cdet_varlen_workspace(int n_max, int64_t batch, bool two_mats, int *err) 
 }
 
 int launch_order(const int *n_arr, int64_t batch, int n_max, int *order, unsigned *ctr, cudaStream_t s,
-                 int fsc_from_n) {
-    varlen_order_kernel<<<1, 1024, 0, s>>>(n_arr, batch, n_max, order, ctr, fsc_from_n);
+                 int fsc_from_n, int split_to) {
+    varlen_order_kernel<<<1, 1024, 0, s>>>(n_arr, batch, n_max, order, ctr, fsc_from_n, split_to);
     return static_cast<int>(cudaGetLastError());
 }
 
@@ -1551,7 +1586,16 @@ int launch_cdet_varlen(const CdetArgs &a, const int64_t *a_off, const int *n_arr
     if (wfrom) off += align256(static_cast<size_t>(a.batch));
     double *slots = reinterpret_cast<double *>(ws + off);
     const int fsc_from = g_fsc_from_n;
-    err = launch_order(n_arr, a.batch, n_max, order, ctr, s, fsc_from);
+    // few items: those of orders 13..15 by blocks on many CTAs, if that pays
+    int split_to = 0;
+    size_t region = 0;  // of the slots, in doubles; the rows of terms come after it
+    if (wfrom) {
+        err = varlen_region(n_max, a.batch, two, grid, &region);
+        if (err) return err;
+        const int to = n_max < fsc_from ? n_max : fsc_from - 1;
+        if (a.batch <= kVarlenSplitMax && static_cast<size_t>(a.batch) << to <= region) split_to = to;
+    }
+    err = launch_order(n_arr, a.batch, n_max, order, ctr, s, fsc_from, split_to);
     if (err) return err;
     // the minors of the items of orders >= wfrom, one launch per order from its
     // first index and count in the sorted list, the flags zeroed before them
@@ -1564,23 +1608,16 @@ int launch_cdet_varlen(const CdetArgs &a, const int64_t *a_off, const int *n_arr
         err = launch_fpm_warp_route(a.A_up, m, a.batch, a.minors_out ? a.minors_out : a.c_out, a.piv_thr, wflag,
                                     a.status, slots, order, a_off, c_off, ctr + 2 + 2 * m, ctr + 3 + 2 * m, s);
     if (err) return err;
-    // few items: those of orders 13..15 by blocks on many CTAs, one order after
-    // the other, their weights in the slots' region (the persistent kernel, which
-    // takes it over after them, finds only the flagged ones of these orders)
-    int split_to = 0;
-    size_t region = 0;  // of the slots, in doubles; the rows of terms come after it
-    if (wfrom) {
-        err = varlen_region(n_max, a.batch, two, grid, &region);
-        if (err) return err;
-    }
-    const int to = n_max < fsc_from ? n_max : fsc_from - 1;
-    if (wfrom && a.batch <= kVarlenSplitMax && static_cast<size_t>(a.batch) << to <= region) {
-        split_to = to;
+    // the split orders one after the other, their weights in the slots' region (the
+    // persistent kernel, which takes it over after them, finds only the flagged ones
+    // of these orders)
+    if (split_to) {
         SplitArgs Q = {};
         Q.a = slots;
         Q.c = a.c_out;
         Q.order = order;
         Q.c_off = c_off;
+        Q.on = ctr + kCtrSplit;
         Q.flag = wflag;
         Q.rows = slots + region;
         Q.cap = varlen_split_rows(n_max, a.batch);
@@ -1599,6 +1636,7 @@ int launch_cdet_varlen(const CdetArgs &a, const int64_t *a_off, const int *n_arr
     VarlenParams V;
     V.a = a;
     V.split_to = split_to;
+    V.split_on = ctr + kCtrSplit;
     V.a.wflag = wflag;
     V.a.warp_from_n = wfrom;
     V.a.gscratch = n_max > kVarlenSmemMaxN ? slots : nullptr;

@@ -247,3 +247,30 @@ def test_lane_group_lines(apm, n, lines):
         assert torch.equal(apm.all_minors(A[at]).nan_to_num(nan=1.5e300), m[at])
         at = torch.arange(b).cuda() % 58
         assert torch.equal(apm.cdet_from_weights(w[at]), cw[at])
+
+
+# uneven batches of orders 13..15 by blocks on many CTAs or, where that would take
+# longer, with one CTA per matrix: fixed-order results either way, flagged matrices
+# among them
+@pytest.mark.parametrize("orders", [[13] * 300, [13] * 100, [13, 14] * 430, [12, 13, 14] * 90, [14] * 460, [15, 13] * 20])
+def test_uneven_blocks_or_not(apm, orders):
+    uniq, o = 16, np.asarray(orders, dtype=np.int32)
+    mats = {m: I.hubbard_batch(uniq, m, seed=9900 + m) for m in set(orders)}
+    for m in mats:
+        mats[m][3] = 0.0                                   # corrected at every pivot
+        mats[m][5, 0, m - 1] = np.nan
+    flat = np.concatenate([mats[m][b % uniq].ravel() for b, m in enumerate(orders)])
+    off = np.concatenate([[0], np.cumsum(o.astype(np.int64) ** 2)])[:-1]
+    A, ao, nt = (torch.as_tensor(x).cuda() for x in (flat, off, o))
+    c, mo, st = apm.cdet_connected_varlen(A, ao, nt, return_minors=True, return_status=True)
+    co = apm.varlen_out_offsets(nt)
+    for m in mats:
+        ref = apm.cdet_connected(torch.as_tensor(mats[m]).cuda(), return_minors=True, return_status=True)
+        at = np.nonzero(o == m)[0]
+        for x, r in ((c, ref[0]), (mo, ref[1])):
+            for lo in range(0, at.size, 64):               # (bits, so that NaN equals itself)
+                k = torch.as_tensor(at[lo:lo + 64]).cuda()
+                got = x[co[k][:, None] + torch.arange(1 << m, device="cuda")]
+                assert torch.equal(got.nan_to_num(nan=1.5e300), r[k % uniq].nan_to_num(nan=1.5e300)), m
+        k = torch.as_tensor(at).cuda()
+        assert torch.equal(st[k], ref[2][k % uniq])
