@@ -243,8 +243,8 @@ __device__ __forceinline__ void fsc_transform_high(double *T, int lg, int n, boo
 // M_1..M_n (M_k = k L_k, L = log Z) of tile entry t in place of Z_1..Z_n,
 // for a mask with at most X elements (Z_m = 0 for m > X; X <= n). The Z_m
 // are read from the tile as they are needed and the M_k kept in registers,
-// then stored together, which keeps the kernel within the registers of three
-// CTAs per SM without a spill.
+// then stored together, which keeps fsc_kernel within the registers of three
+// CTAs per SM without a spill (fsc_pass_kernel<1> spills 64 bytes).
 template <int X>
 __device__ __forceinline__ void fsc_log_entry(double *T, int t, int n) {
     double M[kFscMaxN + 1];
@@ -483,18 +483,22 @@ size_t fsc_workspace_bytes(int n, int64_t batch, int *err) {
 
 // Rounds of one CTA per row (as many rows as CTAs are resident), and the last,
 // partial one by tiles, where that pays: a row's CTA takes the same 6.9 ms at
-// order 16 whether it has the chip to itself or not. us per call, one CTA per
-// row | by tiles: n = 16: 1 row 6882 | 85, 40 6985 | 1405, 300 10783 | 10009, 456 + 56
-// 21377 | 16736; n = 14: 1 1372 | 74, 228 2113 | 1547; n = 12: 40 301 | 111, 228 448 | 535;
-// n = 10: 83 | 100.
-static bool fsc_tiles_pay(int n, int64_t rest) { return n >= 13 || (n == 12 && rest <= 64); }
+// order 16 whether it has the chip to itself or not, and a round that is all but full
+// is the faster whole. us per call, one CTA per row | by tiles:
+//   n = 16: 1 row 6872 | 74, 40 6965 | 1387, 300 10706 | 9935, 440 14946 | 14476, 450 14957 | 14819,
+//           455 14953 | 15004, 456 + 56 21377 | 16736;  n = 15: 1 3002 | 68, 228 4705 | 3386, 455 6681 | 6672
+//   n = 14: 1 1361 | 62, 228 2100 | 1530, 440 2952 | 2888, 455 2952 | 2979
+//   n = 13: 1 618 | 56, 228 952 | 707, 440 1320 | 1307, 450 1320 | 1341;  n = 12: 40 301 | 111, 228 448 | 535
+//   n = 10: 83 | 100.
+static bool fsc_tiles_pay(int n, int64_t rest) { return rest <= (n >= 14 ? 450 : n == 13 ? 440 : n == 12 ? 64 : 0); }
 
 static int fsc_run(FscRows rows, int64_t most, int n, void *workspace, cudaStream_t s) {
     int err = 0;
     const int grid = fsc_grid(n, most, &err), full = fsc_grid(n, INT64_MAX, &err);
     if (err) return err;
+    // (of an item list the last round's rows are counted on the device only)
     const int64_t rest = rows.order ? (most < full ? most : full) : most % full;
-    const bool tiled = n > kFscTileBits && rest && fsc_tiles_pay(n, rest);
+    const bool tiled = n > kFscTileBits && rest && fsc_tiles_pay(n, rows.order ? 1 : rest);
     rows.full = tiled ? full : 1;
     double *ws = static_cast<double *>(workspace);
     if (!tiled || most >= full) fsc_kernel<<<grid, kFscThreads, fsc_smem(n), s>>>(rows, n, ws);

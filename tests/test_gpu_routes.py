@@ -274,3 +274,12 @@ def test_uneven_blocks_or_not(apm, orders):
                 assert torch.equal(got.nan_to_num(nan=1.5e300), r[k % uniq].nan_to_num(nan=1.5e300)), m
         k = torch.as_tensor(at).cuda()
         assert torch.equal(st[k], ref[2][k % uniq])
+
+
+# the fast subset convolution: a last round by tiles up to where a whole one is faster
+@pytest.mark.parametrize("n,batch", [(12, 64), (12, 65), (13, 440), (13, 441), (14, 450), (14, 451), (13, 456 + 441)])
+def test_fsc_last_round(apm, n, batch):
+    w = torch.rand((32, 1 << n), dtype=torch.float64, device="cuda",
+                   generator=torch.Generator(device="cuda").manual_seed(n))
+    at = torch.arange(batch).cuda() % 32
+    assert torch.equal(apm.cdet_from_weights_fsc(w[at]), apm.cdet_from_weights_fsc(w)[at])
