@@ -403,7 +403,10 @@ static int lanes_launch(const LanesParams &P, cudaStream_t s) {
     return static_cast<int>(cudaGetLastError());
 }
 
-static int lanes_most(int n) { return n < 4 ? 2 : n == 4 ? 3 : 4; }
+// Fewest and most lanes per matrix (log2) that cdet_lanes_log2 gives out; nothing
+// beyond them is compiled.
+__host__ __device__ constexpr int lanes_least(int n) { return n > 6 ? n - 6 : 0; }
+__host__ __device__ constexpr int lanes_most(int n) { return n < 4 ? 2 : n == 5 ? 4 : n == 7 ? 2 : 3; }
 
 // Lanes per matrix (log2) at order n and this batch, or -1 for the
 // one-CTA-per-matrix kernel (of 64 or 128 threads here). Both sides measured on
@@ -428,23 +431,15 @@ int cdet_lanes_log2(int n, int64_t batch, int mode) {
         {0, 0, 0, 0, 457, 1800, 2200, 5600, 22000},        // minors and sums
         {0, 0, 0, 0, 1900, 2200, 11500, 20000, 1 << 30}};  // sums from weights
     if (batch < from[mode][n]) return -1;
-    const int least = mode == kModeMinors ? (n > 6 ? n - 6 : 0) : (n > 5 ? n - 5 : n == 5 ? 1 : 0);
+    const int least = mode == kModeMinors ? lanes_least(n) : (n > 5 ? n - 5 : n == 5 ? 1 : 0);
     int lg = least;
     while (lg < lanes_most(n) && (batch << (lg + 1)) <= int64_t(32) * 6 * 152) ++lg;
     return lg;
 }
 
-template <int N>
+template <int N, int LG = lanes_least(N)>
 static int lanes_for(const LanesParams &P, int lg, cudaStream_t s) {
-    if constexpr (N <= 6)
-        if (lg == 0) return lanes_launch<N, 0>(P, s);
-    if constexpr (N <= 7)
-        if (lg == 1) return lanes_launch<N, 1>(P, s);
-    if (lg == 2) return lanes_launch<N, 2>(P, s);
-    if constexpr (N >= 4)
-        if (lg == 3) return lanes_launch<N, 3>(P, s);
-    if constexpr (N >= 5)
-        if (lg == 4) return lanes_launch<N, 4>(P, s);
+    if constexpr (LG <= lanes_most(N)) return lg == LG ? lanes_launch<N, LG>(P, s) : lanes_for<N, LG + 1>(P, lg, s);
     return static_cast<int>(cudaErrorInvalidValue);
 }
 

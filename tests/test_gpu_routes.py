@@ -283,3 +283,23 @@ def test_fsc_last_round(apm, n, batch):
                    generator=torch.Generator(device="cuda").manual_seed(n))
     at = torch.arange(batch).cuda() % 32
     assert torch.equal(apm.cdet_from_weights_fsc(w[at]), apm.cdet_from_weights_fsc(w)[at])
+
+
+# installed lane-group tables reach the lane groups too, where most of a group's
+# partial sums are one lane's: the largest groups, next to none, some layers, against
+# the one-CTA-per-matrix kernel under the same table
+@pytest.mark.parametrize("n,batch", [(4, 3000), (5, 1800), (5, 40000), (6, 3600), (6, 40000), (7, 6000), (7, 30000),
+                                     (8, 22000)])
+def test_lane_groups_under_installed_tables(apm, n, batch):
+    A = torch.as_tensor(I.gaussian_plus_2I(n, 200, seed=60 + n)).cuda()
+    at = torch.arange(batch).cuda() % 200
+    tables = [[min(5, k - 1) if 2 <= k <= n else 0 for k in range(17)], [int(k == n) for k in range(17)],
+              [k % 2 if 2 <= k <= n else 0 for k in range(17)], [min(2, k - 1) if 2 <= k <= n else 0 for k in range(17)]]
+    try:
+        for r in tables:
+            packed = sum(x << (3 * k) for k, x in enumerate(r))
+            apm.tune_set([packed if m == n else 0 for m in range(17)])
+            few, big = apm.cdet_connected(A), apm.cdet_connected(A[at])
+            assert torch.equal(big, few[at]), r
+    finally:
+        apm.tune_set(None)
