@@ -27,7 +27,7 @@ from . import build as _build
 
 class CdetVarlenGraph:
     def __init__(self, A: torch.Tensor, a_off: torch.Tensor, n: torch.Tensor, n_max: int | None = None,
-                 with_minors: bool = True):
+                 with_minors: bool = True, capture: bool = True):
         self.A, self.a_off, self.n = A, a_off, n
         self.n_max = int(n.max().item()) if n_max is None else n_max
         self.c_off = apm.varlen_out_offsets(n)
@@ -40,6 +40,8 @@ class CdetVarlenGraph:
         self.workspace = torch.empty(max(nb, 16), dtype=torch.uint8, device=dev)
         self._call()                       # eager run: tables uploaded, attributes set
         torch.cuda.synchronize(dev)
+        if not capture:
+            return
         self.graph = torch.cuda.CUDAGraph()
         with torch.cuda.graph(self.graph):
             self._call()
@@ -141,7 +143,8 @@ def autotune(orders=range(4, 13), fsc_orders=range(13, 17), reps: int = 3, use_c
     returns it (cached per GPU name under _build/):
 
       lane_groups[n]  (orders in `orders`) the lane-group size of every popcount
-                      layer of Eq. recursion: starting from the cost model, each
+                      layer of Eq. recursion, timed on an uneven batch of that
+                      order alone: starting from the cost model, each
                       layer holding at least 5 % of the order's submask terms
                       tries one size smaller and one larger, kept when faster
                       (orders above 12 run the recursion in blocks of 10 low
@@ -174,13 +177,17 @@ def autotune(orders=range(4, 13), fsc_orders=range(13, 17), reps: int = 3, use_c
     for n in orders:
         base = apm.tune_get(n)
         batch = int(max(1216, min(65536, 4e9 / (3 ** n))))
+        # on the kernel the tables serve: an uneven batch of this order alone, in the
+        # CTAs of one that holds larger orders too (a fixed-order call may take lane
+        # groups or narrower CTAs, whose best sizes slowed it by up to 4 %)
         A = torch.as_tensor(inputs.hubbard_batch(batch, n, seed=50 + n)).cuda()
-        c = torch.empty((batch, 1 << n), dtype=torch.float64, device="cuda")
-        ws = torch.empty(max(apm.workspace_size(apm.OP_CDET, n, batch), 16), dtype=torch.uint8, device="cuda")
+        n_t = torch.full((batch,), n, dtype=torch.int32, device="cuda")
+        call = CdetVarlenGraph(A.reshape(-1), torch.arange(batch, device="cuda") * (n * n), n_t, max(n, 12),
+                               with_minors=False, capture=False)
 
         def run(table):
             apm.tune_set([table if m == n else 0 for m in range(17)])
-            return _event_ms(lambda: apm.cdet_connected(A, out_c=c, workspace=ws), reps)
+            return _event_ms(call._call, reps)
 
         best, t_best = base, run(base)
         t_base = t_best
@@ -199,7 +206,7 @@ def autotune(orders=range(4, 13), fsc_orders=range(13, 17), reps: int = 3, use_c
         timings[f"lane_groups_n{n}"] = {"default_ms": t_base, "tuned_ms": t_best, "batch": batch}
         if verbose:
             print(f"n={n}: cost model {t_base:.3f} ms, tuned {t_best:.3f} ms", flush=True)
-        del A, c, ws
+        del A, n_t, call
     apm.tune_set([lane.get(str(m), 0) for m in range(17)])
     # hand-off from the recursion to the fast subset convolution
     faster = {}

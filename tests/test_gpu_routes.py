@@ -303,3 +303,30 @@ def test_lane_groups_under_installed_tables(apm, n, batch):
             assert torch.equal(big, few[at]), r
     finally:
         apm.tune_set(None)
+
+
+def test_lane_groups_are_timed_on_the_uneven_kernel(apm, monkeypatch):
+    """The tables serve the uneven batch: they are not chosen by fixed-order calls,
+    which take other kernels at these orders, and the batch is not slower by them."""
+    from paper_2104_07638_gb300 import batch
+
+    def fixed(*a, **k):
+        raise AssertionError("a fixed-order call was timed")
+    monkeypatch.setattr(apm, "cdet_connected", fixed)
+    monkeypatch.setattr(batch, "_cache_path", lambda: str(batch._build.BUILD) + "/tune_test.json")
+    try:
+        tuned = batch.autotune(orders=(7, 8), fsc_orders=(), reps=5, use_cache=False, tune_launch=False)
+        for n in (7, 8):
+            t = tuned["timings"][f"lane_groups_n{n}"]
+            assert t["tuned_ms"] <= t["default_ms"]
+        o = np.full(16384, 8, dtype=np.int32)
+        flat, off = I.hubbard_varlen(o, seed=9950)
+        g = batch.CdetVarlenGraph(*(torch.as_tensor(x).cuda() for x in (flat, off, o)), n_max=12, with_minors=False,
+                                  capture=False)
+        with_table = min(batch._event_ms(g._call, 10) for _ in range(3))
+        apm.tune_set(None)
+        without = min(batch._event_ms(g._call, 10) for _ in range(3))
+        assert with_table <= 1.05 * without
+    finally:
+        apm.tune_set(None)
+        apm.tune_options_set(0, 0, 0)
