@@ -12,10 +12,11 @@ popcount layer of the recursion per order, the order from which the connected
 sums take the fast subset convolution, the resident CTAs per SM of the
 persistent uneven batch and the warps per CTA of the uneven Keldysh batch, and
 installs the result (``apm_cdet_tune_set``, ``apm_tune_options_set``); results
-are cached per GPU name in ``_build/``.
+are cached in ``_build/``, by GPU name and sources.
 """
 from __future__ import annotations
 
+import hashlib
 import json
 import os
 
@@ -108,8 +109,13 @@ def _with_layer(packed: int, k: int, r: int) -> int:
 
 
 def _cache_path() -> str:
+    # by the sources too: mappings chosen on other kernels are not the best on these
     name = torch.cuda.get_device_name().replace(" ", "_")
-    return os.path.join(_build.BUILD, f"tune_{name}.json")
+    sha = hashlib.sha256()
+    for path in sorted(_build._deps() + [os.path.abspath(__file__)]):
+        with open(path, "rb") as f:
+            sha.update(f.read())
+    return os.path.join(_build.BUILD, f"tune_{name}_{sha.hexdigest()[:16]}.json")
 
 
 def _event_ms(fn, reps: int) -> float:
@@ -140,7 +146,7 @@ def autotune(orders=range(4, 13), fsc_orders=range(13, 17), reps: int = 3, use_c
              tune_launch: bool = True, verbose: bool = False) -> dict:
     """Searches, on this GPU, the per-order mappings of the connected-sum path
     and the launch shapes of the uneven batches, installs the result and
-    returns it (cached per GPU name under _build/):
+    returns it (cached under _build/ by GPU name and sources):
 
       lane_groups[n]  (orders in `orders`) the lane-group size of every popcount
                       layer of Eq. recursion, timed on an uneven batch of that
