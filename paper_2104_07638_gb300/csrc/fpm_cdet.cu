@@ -858,8 +858,9 @@ struct SplitArgs {
 };
 
 // Weights of the matrices the warp-per-matrix kernel has not flagged, from
-// their minors (rows laid out as the sums) into the rows of P.a.
-__global__ void __launch_bounds__(256) cdet_square_kernel(const SplitArgs P, const double *__restrict__ minors,
+// their minors (rows laid out as the sums) into the rows of P.a, passed as `to`.
+__global__ void __launch_bounds__(256) cdet_square_kernel(const SplitArgs P, double *to,
+                                                          const double *__restrict__ minors,
                                                           const uint8_t *__restrict__ flag, int single) {
     const int64_t pairs = int64_t(1) << (P.n - 1), all = P.items() << (P.n - 1);
     for (int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; i < all;
@@ -868,7 +869,7 @@ __global__ void __launch_bounds__(256) cdet_square_kernel(const SplitArgs P, con
         if (flag[P.item(b)]) continue;
         double2 m = *reinterpret_cast<const double2 *>(minors + (P.out(b) - P.c) + t);
         if (!single) m = make_double2(m.x * m.x, m.y * m.y);
-        *reinterpret_cast<double2 *>(const_cast<double *>(P.a) + b * P.astride + t) = m;
+        *reinterpret_cast<double2 *>(to + b * P.astride + t) = m;
     }
 }
 
@@ -1436,7 +1437,7 @@ int launch_fpm_cdet(const CdetArgs &a, cudaStream_t s) {
         if (a.wflag) {
             P.a.wflag += b0;
             cdet_square_kernel<<<static_cast<int>(((rest << (a.n - 1)) + 255) / 256), 256, 0, s>>>(
-                Q, a.minors_out ? P.a.minors_out : Q.c, P.a.wflag, a.single_det);
+                Q, a.gscratch, a.minors_out ? P.a.minors_out : Q.c, P.a.wflag, a.single_det);
         }
         fpm_cdet_kernel<false><<<static_cast<int>(rest), kCdetThreads, smem, s>>>(P);
         err = static_cast<int>(cudaGetLastError());
@@ -1628,7 +1629,8 @@ int launch_cdet_varlen(const CdetArgs &a, const int64_t *a_off, const int *n_arr
             Q.astride = size_t(1) << m;
             Q.first = ctr + 2 + 2 * m;
             Q.count = ctr + 3 + 2 * m;
-            cdet_square_kernel<<<8 * 152, 256, 0, s>>>(Q, a.minors_out ? a.minors_out : a.c_out, wflag, a.single_det);
+            cdet_square_kernel<<<8 * 152, 256, 0, s>>>(Q, slots, a.minors_out ? a.minors_out : a.c_out, wflag,
+                                                       a.single_det);
             err = launch_cdet_split(Q, a.batch, s);
             if (err) return err;
         }

@@ -475,8 +475,8 @@ int launch_fpm_warp(const double *A, int n, int64_t batch, double *minors, doubl
     const FwShape sh = fw_shape(n, batch);
     const FwKernel kern = fw_kernel_for(sh.T);
     if (sh.T != kFwTail) {
-        // a shorter tail needs no fewer resident warps: the stacks are sized for
-        // the longest tail's, and its grid stays within them
+        // the stacks are as many as the longest tail's kernel has warps resident (and
+        // of the shortest tail's size): a shorter tail's grid stays within them
         int err2 = 0;
         const int r = fw_resident(kern, &err2);
         if (err2) return err2;

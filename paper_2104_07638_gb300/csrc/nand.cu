@@ -766,7 +766,6 @@ int nand_grid(int64_t batch, int *err) {
     return static_cast<int>(g < 1 ? 1 : g);
 }
 
-// per resident warp the stack and correction records, then one flag per matrix
 // Scratch: per resident warp the stack and the correction records (as many warps
 // as the parts of the largest batch in parts, or this batch, can occupy), then the
 // flags.
