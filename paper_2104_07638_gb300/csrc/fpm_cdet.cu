@@ -1243,7 +1243,7 @@ void cdet_tune_set(const unsigned long long *table) {
 //           1672 160 | 140 | 158, 2000 191 | 165 | 170, 16384 1413 | 1240 | 1223
 //   n = 11: 456 99 | 104 | 122, 912 194 | 185 | 191, 1368 286 | 301 | 331, 2000 441 | 424 | 477,
 //           16384 3315 | 3233 | 3299
-//   n = 12: 456 256 | 270 | 353, 16384 8864 | 9299 | 12462
+//   n = 12: 456 252 | 259 | 290, 16384 8643 | 8808 | 9680
 // With a second matrix the arrays of a narrow CTA leave room for 7 (n = 10, 64
 // threads) or 4 on an SM (n = 11, 128 threads) instead of 10 and 6:
 //   n = 10: 1216 158 | 142 | 164, 1672 209 | 176 | 188, 16384 1849 | 1542 | 1593
@@ -1335,12 +1335,21 @@ static int launch_cdet_split(const SplitArgs &P, int64_t most, cudaStream_t s) {
 
 // Whether a launch (or the last, partial round of one) of this many matrices
 // above order 12 goes level by level over many CTAs rather than with one CTA
-// per matrix, whose time hardly depends on how many of a round's 456 there are.
+// per matrix, whose time depends on the most of them that share an SM only: level
+// by level up to most of two on every SM, and again up to most of three.
 // Measured, us per call (one CTA per matrix | level by level):
-//   n = 13: 1 matrix 500 | 152, 24 501 | 184, 152 512 | 373, 300 607 | 640
-//   n = 14: 1 1428 | 198, 24 1435 | 288, 152 1456 | 929, 300 1727 | 1629, 456 2336 | 2410
-//   n = 15: 1 4195 | 249, 24 4215 | 580, 152 4267 | 2615, 456 6757 | 6756
-static bool cdet_split_pays(int n, int64_t batch) { return batch <= (n == 13 ? 260 : n == 14 ? 350 : 456); }
+//   n = 13: 1 matrix 377 | 130, 24 375 | 168, 152 386 | 360, 230 552 | 541, 260 553 | 582, 304 555 | 651,
+//           305 776 | 688, 360 790 | 786, 370 791 | 796, 400 790 | 823
+//   n = 14: 1 1069 | 167, 24 1074 | 270, 152 1096 | 915, 270 1577 | 1563, 290 1578 | 1632, 305 2239 | 1788,
+//           405 2259 | 2205, 420 2279 | 2385
+//   n = 15: 1 3129 | 231, 24 3145 | 554, 152 3199 | 2613, 280 4649 | 4564, 304 4651 | 4818, 305 6578 | 4957,
+//           400 6642 | 6279, 430 6649 | 6740
+//   n = 16 (from weights): 1 12451 | 299, 300 14857 | 13042, 455 19657 | 19456
+static bool cdet_split_pays(int n, int64_t batch) {
+    if (n >= 16) return true;
+    if (batch <= 2 * 152) return batch <= (n == 13 ? 235 : n == 14 ? 275 : 287);
+    return batch <= (n == 13 ? 365 : n == 14 ? 405 : 422);
+}
 
 // CTAs per matrix (log2) of a launch of so many matrices, 0 for one: at most a CTA
 // per SM (two on an SM share its FP64 pipe). us per call, 1, 2, 4 and 8 CTAs:

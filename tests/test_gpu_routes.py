@@ -330,3 +330,19 @@ def test_lane_groups_are_timed_on_the_uneven_kernel(apm, monkeypatch):
     finally:
         apm.tune_set(None)
         apm.tune_options_set(0, 0, 0)
+
+
+# orders above 12 level by level or with one CTA per matrix, on both sides of each line
+@pytest.mark.parametrize("n,batch", [(13, 235), (13, 236), (13, 304), (13, 305), (13, 365), (13, 366), (14, 275),
+                                     (14, 276), (14, 406), (15, 288), (15, 305), (13, 456 + 300)])
+def test_split_lines(apm, n, batch):
+    A = I.hubbard_batch(16, n, seed=70 + n)
+    A[3] = 0.0
+    A[5, 0, n - 1] = np.inf
+    d = torch.as_tensor(A).cuda()
+    at = torch.arange(batch).cuda() % 16
+    ref = apm.cdet_connected(d, return_status=True)
+    got = apm.cdet_connected(d[at], return_status=True)
+    assert torch.equal(got[1], ref[1][at])
+    for lo in range(0, batch, 64):
+        assert torch.equal(got[0][lo:lo + 64].nan_to_num(nan=1.5e300), ref[0][at[lo:lo + 64]].nan_to_num(nan=1.5e300))
