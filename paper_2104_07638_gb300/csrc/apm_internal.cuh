@@ -233,10 +233,10 @@ int launch_cdet_varlen(const CdetArgs &a, const int64_t *a_off, const int *n_arr
                        int n_max, void *workspace, cudaStream_t s);
 // Counting sort by decreasing order into `order`; ctr[0] = 0 (work counter),
 // ctr[1] = the items of orders >= fsc_from_n, and for each order m the first
-// index and the count of its items at ctr[2 + 2m], ctr[3 + 2m]; with split_to, the
-// choice of a route for orders 13..split_to behind them.
+// index and the count of its items at ctr[2 + 2m], ctr[3 + 2m]; behind them
+// the choice of a route for orders 13..split_to and of a CTA's width.
 int launch_order(const int *n_arr, int64_t batch, int n_max, int *order, unsigned *ctr, cudaStream_t s,
-                 int fsc_from_n = kFscFromN, int split_to = 0);
+                 int fsc_from_n = kFscFromN, int split_to = 0, int by_width = 0);
 int launch_keldysh_varlen(const double *Mt, const int64_t *m_off, const int *n_arr, int64_t batch, int n_max,
                           int sgn, double *sum, double *partial, uint32_t *status, void *stack,
                           const int *order, unsigned *ctr, cudaStream_t s);

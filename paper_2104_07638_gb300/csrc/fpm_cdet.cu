@@ -87,8 +87,8 @@ struct VarlenParams {
     unsigned *ctr;                 // work counter, zeroed by varlen_order_kernel
     int smem_max_n;
     int n_max;
-    int split_to;                  // unflagged items of orders smem_max_n + 1 .. split_to are done elsewhere,
-    const unsigned *split_on;      // if this word is not 0
+    int split_to;                  // items of orders smem_max_n + 1 .. split_to with flag 0 are done elsewhere
+    const unsigned *width;         // the threads of the CTAs that run, where both widths are launched
     unsigned long long gsel[17];   // lane-group table per order
 };
 
@@ -858,10 +858,17 @@ struct SplitArgs {
 };
 
 // Weights of the matrices the warp-per-matrix kernel has not flagged, from
-// their minors (rows laid out as the sums) into the rows of P.a, passed as `to`.
+// their minors (rows laid out as the sums) into the rows of P.a, passed as `to`. Where
+// an uneven batch's items do not go by blocks (P.on), their flags get bit 1 instead:
+// the persistent kernel leaves out those with flag 0.
 __global__ void __launch_bounds__(256) cdet_square_kernel(const SplitArgs P, double *to,
-                                                          const double *__restrict__ minors,
-                                                          const uint8_t *__restrict__ flag, int single) {
+                                                          const double *__restrict__ minors, uint8_t *flag,
+                                                          int single) {
+    if (P.order && !*P.on) {
+        for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < static_cast<int>(*P.count); i += gridDim.x * blockDim.x)
+            flag[P.item(i)] |= 2;
+        return;
+    }
     const int64_t pairs = int64_t(1) << (P.n - 1), all = P.items() << (P.n - 1);
     for (int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; i < all;
          i += static_cast<int64_t>(gridDim.x) * blockDim.x) {
@@ -1040,12 +1047,17 @@ __global__ void __launch_bounds__(kCdetThreads, 3) cdet_split_diag_kernel(const 
 
 // Uneven batch: items taken longest-first from `order` through a global
 // counter; arrays on chip for n <= smem_max_n, else in the CTA's scratch slot.
+// kWidths: launched with both widths of CTAs, of which V.width names the one that
+// runs (an instantiation of its own: the test alone, before the first items are
+// taken, let them gather on fewer SMs, 1700 of orders 4..9 51 -> 61 us).
+template <bool kWidths>
 __global__ void __launch_bounds__(kCdetThreads, 3) fpm_cdet_varlen_kernel(const VarlenParams V) {
     extern __shared__ __align__(128) unsigned char smem_raw[];
     CdetSmemHdr &h = *reinterpret_cast<CdetSmemHdr *>(smem_raw);
     __shared__ unsigned long long gsel_s[17];
     __shared__ int item_s;
     const CdetArgs &p = V.a;
+    if (kWidths && *V.width != blockDim.x) return;
     if (threadIdx.x < 17) gsel_s[threadIdx.x] = V.gsel[threadIdx.x];
     double *const sbase = reinterpret_cast<double *>(smem_raw + ((sizeof(CdetSmemHdr) + 127) & ~size_t(127)));
     double *const gbase = p.gscratch ? p.gscratch + static_cast<size_t>(blockIdx.x) * slot_doubles(V.n_max) : nullptr;
@@ -1061,7 +1073,7 @@ __global__ void __launch_bounds__(kCdetThreads, 3) fpm_cdet_varlen_kernel(const 
             if (threadIdx.x == 0 && p.status) p.status[b] = APM_ST_BAD_ORDER;
             continue;
         }
-        if (n > V.smem_max_n && n <= V.split_to && *V.split_on && !p.wflag[b]) continue;
+        if (n > V.smem_max_n && n <= V.split_to && !p.wflag[b]) continue;
         const int N = 1 << n;
         const int NC = N > 16 ? N : 16;
         const bool in_smem = n <= V.smem_max_n;
@@ -1074,7 +1086,7 @@ __global__ void __launch_bounds__(kCdetThreads, 3) fpm_cdet_varlen_kernel(const 
                   p.minors_out ? p.minors_out + (p.two_mats ? 2 * co : co) : nullptr,
                   p.c_out ? p.c_out + co : nullptr, p.status ? p.status + b : nullptr, MA, MC, MU, in_smem,
                   gsel_s[n], gsel_s[kBlkB], sbase, h, nullptr, 1.0,
-                  p.wflag && p.warp_from_n && n >= p.warp_from_n && !p.wflag[b]);
+                  p.wflag && p.warp_from_n && n >= p.warp_from_n && !(p.wflag[b] & 1));
     }
     if (threadIdx.x == 0) bulk_wait_all();
 }
@@ -1083,12 +1095,13 @@ __global__ void __launch_bounds__(kCdetThreads, 3) fpm_cdet_varlen_kernel(const 
 // order after order, or all orders together with one CTA per matrix. Each side's
 // time from hist, the items per order: of the first a launch's fixed part and a part
 // per item; of the second what its work takes on 3 CTAs per SM, but not less than
-// the rounds of any one order, whose last takes less with fewer CTAs on an SM.
+// the rounds of any one order, whose last takes less with fewer CTAs on an SM (after
+// a full one few items do not spread over all SMs).
 // 4 % in favour of the second. Measured, us per call (blocks | one CTA per matrix):
 //   orders 13, 14: 100 items 656 | 1125, 456 1885 | 2256, 912 3483 | 3064
 //   order 13: 100 308 | 404, 300 651 | 559, 500 1038 | 1288, 912 1761 | 1571
 //   orders 13..15: 456 3993 | 6584, 1024 7924 | 7162;  4..14: 1024 1181 | 2230
-__device__ int varlen_split_pays(const int *hist, int64_t batch, int to) {
+__device__ __noinline__ int varlen_split_pays(const int *hist, int64_t batch, int to) {
     constexpr int kCtas = 456;  // 3 per SM
     // orders 13..16 (16 only where the recursion takes it): us at 1, 2, 3 per SM; us, 10 ns
     constexpr int kWhole[4][3] = {{404, 557, 797}, {1093, 1571, 2288}, {3137, 4585, 6650}, {12450, 14840, 19650}};
@@ -1102,20 +1115,40 @@ __device__ int varlen_split_pays(const int *hist, int64_t batch, int to) {
         blocks += kFixed[i] + kItem[i] * c / 100;
         work += kWhole[i][2] * c;
         const int full = c / kCtas, rest = c - full * kCtas;
-        const int rounds = full * kWhole[i][2] + (rest ? kWhole[i][(rest - 1) / 152] : 0);
+        const int last = rest == 0 ? 0 : full && rest <= 152 ? (kWhole[i][0] + kWhole[i][1]) / 2 : kWhole[i][(rest - 1) / 152];
+        const int rounds = full * kWhole[i][2] + last;
         least = max(least, max(rounds, kWhole[i][depth]));
     }
     return 104 * blocks <= 100 * max(work / kCtas + low, least);
 }
 
+// Threads of the CTAs of an uneven batch of orders up to n_max = 9, 10 or 11, of a
+// size where it depends on hist, the items per order: wide (256) while one round of
+// wide CTAs holds the items of the largest order (at order 9, narrow CTAs of 64
+// threads, those of order 8 count by half), else narrow; wide again for two to three
+// rounds of order 11 alone, which narrow CTAs (912 at a time) take in two of their
+// own. us per call, narrow | wide:
+//   orders 4..9: 600 items 36 | 28, 1024 41 | 37;  8, 9: 700 38 | 45;   order 9: 600 37 | 50, 1200 50 | 73
+//   orders 4..10: 912 76 | 48, 1700 79 | 70;       9, 10: 1024 78 | 90; order 10: 600 58 | 88, 1200 126 | 130
+//   orders 4..11: 912 175 | 103, 3200 191 | 187;   10, 11: 1200 191 | 200, 2000 299 | 317
+//   order 11: 600 133 | 171, 1200 302 | 266, 2300 486 | 519
+__device__ unsigned varlen_width(const int *hist, int64_t batch, int n_max) {
+    const int c = hist[n_max];
+    if (n_max == 9) return c + hist[8] / 2 <= 360 ? kCdetThreads : 64u;
+    const bool wide = c <= 456 || (n_max == 11 && c > 912 && c <= 1368 && 10 * c > 9 * batch);
+    return wide ? kCdetThreads : 128u;
+}
+
 // Longest-first order of an uneven batch: counting sort by decreasing order n
 // (one CTA), and reset of the work counter of the consumer kernel; per order m
 // the first index and the count of its items (ctr[2 + 2m], ctr[3 + 2m]), and the
-// choice of varlen_split_pays for orders 13..split_to (ctr[kCtrSplit]).
-constexpr int kCtrSplit = 36;
+// choices of varlen_split_pays for orders 13..split_to (ctr[kCtrSplit]) and, with
+// by_width, of varlen_width (ctr[kCtrWidth]).
+constexpr int kCtrSplit = 36, kCtrWidth = 37;
+template <bool kChoose>
 __global__ void __launch_bounds__(1024) varlen_order_kernel(const int *__restrict__ n_arr, int64_t batch,
                                                             int n_max, int *order, unsigned *ctr, int fsc_from_n,
-                                                            int split_to) {
+                                                            int split_to, int by_width) {
     __shared__ int hist[18];
     __shared__ int start[18];
     if (threadIdx.x < 18) hist[threadIdx.x] = 0;
@@ -1138,7 +1171,10 @@ __global__ void __launch_bounds__(1024) varlen_order_kernel(const int *__restric
         int nf = 0;
         for (int n = fsc_from_n; n <= 16; ++n) nf += hist[n];
         ctr[1] = static_cast<unsigned>(nf);
-        ctr[kCtrSplit] = split_to ? static_cast<unsigned>(varlen_split_pays(hist, batch, split_to)) : 0u;
+        if constexpr (kChoose) {
+            if (by_width) ctr[kCtrWidth] = varlen_width(hist, batch, n_max);
+            if (split_to) ctr[kCtrSplit] = static_cast<unsigned>(varlen_split_pays(hist, batch, split_to));
+        }
         for (int n = 0; n <= 16; ++n) {
             ctr[2 + 2 * n] = static_cast<unsigned>(start[n]);
             ctr[3 + 2 * n] = static_cast<unsigned>(hist[n]);
@@ -1475,20 +1511,20 @@ constexpr int kVarlenSmemMaxN = 12;
 // Threads of a CTA, from the largest order present and the batch. Narrow CTAs
 // (four or two times as many on an SM) pay once the batch is several rounds of wide
 // ones: below that the call waits for the items of the largest order, which a wide
-// CTA finishes soonest. Us per call, 64 | 128 | 256 threads (device time):
+// CTA finishes soonest. Where that depends on how many there are of it (0), both are
+// launched and the kernel that sorts the items chooses (varlen_width; the other's
+// CTAs return at once). us per call, 64 | 128 | 256 threads (device time):
 //   orders 4..8:  304 items 21 | 20 | 20, 600 22 | 22 | 23, 1500 27 | 27 | 44, 16384 159 | 207 | 361
-//   orders 4..9:  64 31 | 24 | 23, 912 42 | 40 | 35, 1200 42 | 40 | 41, 2736 59 | 54 | 79,
-//                 16384 218 | 268 | 430;  order 9 alone: 912 43 | 41 | 51, 2736 107 | 107 | 139
-//   orders 4..10: 456 56 | 49 | 46, 1500 92 | 79 | 61, 2100 82 | 79 | 83, 4096 119 | 110 | 151
-//   orders 4..11: 456 129 | 108 | 103, 1500 196 | 190 | 104, 3200 197 | 191 | 187, 4096 204 | 195 | 238;
-//                 order 11 alone: 1200 381 | 302 | 266, 3200 750 | 662 | 703
+//   orders 4..9:  64 31 | 24 | 23, 456 33 | 29 | 28, 1200 42 | 40 | 41, 16384 218 | 268 | 430
+//   orders 4..10: 456 56 | 49 | 46, 2100 82 | 79 | 83, 4096 119 | 110 | 151
+//   orders 4..11: 456 129 | 108 | 103, 3648 197 | 191 | 214;  order 11: 4096 935 | 839 | 856
+static int varlen_narrow(int n_max) { return n_max <= 9 ? 64 : 128; }
 static int varlen_threads(int n_max, int64_t batch) {
+    if (n_max > 11) return kCdetThreads;
     if (n_max <= 6) return 64;  // the same at any size below a round, the fastest above
-    if (n_max <= 8) return batch <= 456 ? kCdetThreads : 64;
-    if (n_max == 9) return batch < 1200 ? kCdetThreads : batch < 2700 ? 128 : 64;
-    if (n_max == 10) return batch < 2100 ? kCdetThreads : 128;
-    if (n_max == 11) return batch < 3300 ? kCdetThreads : 128;
-    return kCdetThreads;
+    if (batch <= 456) return kCdetThreads;
+    if (n_max <= 8) return 64;
+    return batch <= (n_max == 9 ? 1100 : n_max == 10 ? 2000 : 3100) ? 0 : varlen_narrow(n_max);
 }
 // Largest uneven batch whose items of orders 13..15 may go by blocks on many CTAs: a
 // CTA takes 3 to 4 ms for one of order 15 by itself, which is the whole call then
@@ -1503,8 +1539,7 @@ static int varlen_smem_n(int n_max) { return n_max < kVarlenSmemMaxN ? n_max : k
 
 static size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
 
-static int cdet_varlen_grid(int n_max, int64_t batch, bool two_mats, int *err) {
-    const int threads = varlen_threads(n_max, batch);
+static int cdet_varlen_grid(int n_max, int threads, bool two_mats, bool widths, int *err) {
     int dev = 0, sms = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -1512,9 +1547,10 @@ static int cdet_varlen_grid(int n_max, int64_t batch, bool two_mats, int *err) {
         *err = static_cast<int>(e);
         return 0;
     }
-    int per_sm = resident_ctas(fpm_cdet_varlen_kernel, threads,
-                               cdet_smem_bytes(varlen_smem_n(n_max), two_mats, true),
-                               cdet_smem_bytes(kVarlenSmemMaxN, true, true), err) / sms;
+    const size_t smem = cdet_smem_bytes(varlen_smem_n(n_max), two_mats, true);
+    const size_t allow = cdet_smem_bytes(kVarlenSmemMaxN, true, true);
+    int per_sm = (widths ? resident_ctas(fpm_cdet_varlen_kernel<true>, threads, smem, allow, err)
+                         : resident_ctas(fpm_cdet_varlen_kernel<false>, threads, smem, allow, err)) / sms;
     if (*err) return 0;
     // the tuned limit counts CTAs of kCdetThreads threads
     const int most = g_varlen_ctas * (kCdetThreads / threads);
@@ -1562,7 +1598,7 @@ size_t cdet_varlen_workspace(int n_max, int64_t batch, bool two_mats, int *err) 
     *err = 0;
     size_t bytes = 256 + align256(static_cast<size_t>(batch) * sizeof(int));
     if (n_max <= kVarlenSmemMaxN) return bytes;
-    const int grid = cdet_varlen_grid(n_max, batch, two_mats, err);
+    const int grid = cdet_varlen_grid(n_max, kCdetThreads, two_mats, false, err);  // of orders above 12
     if (*err) return 0;
     size_t region = 0;
     *err = varlen_region(n_max, batch, two_mats, grid, &region);
@@ -1575,8 +1611,9 @@ size_t cdet_varlen_workspace(int n_max, int64_t batch, bool two_mats, int *err) 
 }
 
 int launch_order(const int *n_arr, int64_t batch, int n_max, int *order, unsigned *ctr, cudaStream_t s,
-                 int fsc_from_n, int split_to) {
-    varlen_order_kernel<<<1, 1024, 0, s>>>(n_arr, batch, n_max, order, ctr, fsc_from_n, split_to);
+                 int fsc_from_n, int split_to, int by_width) {
+    const auto kern = split_to || by_width ? varlen_order_kernel<true> : varlen_order_kernel<false>;
+    kern<<<1, 1024, 0, s>>>(n_arr, batch, n_max, order, ctr, fsc_from_n, split_to, by_width);
     return static_cast<int>(cudaGetLastError());
 }
 
@@ -1585,7 +1622,10 @@ int launch_cdet_varlen(const CdetArgs &a, const int64_t *a_off, const int *n_arr
     int err = ensure_tables();
     if (err) return err;
     const bool two = a.two_mats != 0;
-    const int grid = cdet_varlen_grid(n_max, a.batch, two, &err);
+    const int threads = varlen_threads(n_max, a.batch);  // 0: both widths, varlen_width chooses
+    const int grid = cdet_varlen_grid(n_max, threads ? threads : kCdetThreads, two, threads == 0, &err);
+    if (err) return err;
+    const int narrow = threads ? 0 : cdet_varlen_grid(n_max, varlen_narrow(n_max), two, true, &err);
     if (err) return err;
     unsigned char *ws = static_cast<unsigned char *>(workspace);
     unsigned *ctr = reinterpret_cast<unsigned *>(ws);
@@ -1605,7 +1645,7 @@ int launch_cdet_varlen(const CdetArgs &a, const int64_t *a_off, const int *n_arr
         const int to = n_max < fsc_from ? n_max : fsc_from - 1;
         if (a.batch <= kVarlenSplitMax && static_cast<size_t>(a.batch) << to <= region) split_to = to;
     }
-    err = launch_order(n_arr, a.batch, n_max, order, ctr, s, fsc_from, split_to);
+    err = launch_order(n_arr, a.batch, n_max, order, ctr, s, fsc_from, split_to, narrow > 0);
     if (err) return err;
     // the minors of the items of orders >= wfrom, one launch per order from its
     // first index and count in the sorted list, the flags zeroed before them
@@ -1647,7 +1687,7 @@ int launch_cdet_varlen(const CdetArgs &a, const int64_t *a_off, const int *n_arr
     VarlenParams V;
     V.a = a;
     V.split_to = split_to;
-    V.split_on = ctr + kCtrSplit;
+    V.width = narrow ? ctr + kCtrWidth : nullptr;
     V.a.wflag = wflag;
     V.a.warp_from_n = wfrom;
     V.a.gscratch = n_max > kVarlenSmemMaxN ? slots : nullptr;
@@ -1661,9 +1701,14 @@ int launch_cdet_varlen(const CdetArgs &a, const int64_t *a_off, const int *n_arr
     for (int n = 0; n <= 16; ++n) V.gsel[n] = cdet_gsel_packed(n);
     const bool fsc = a.mode == kModeCdet && n_max >= fsc_from;
     V.a.fsc_from_n = fsc ? fsc_from : 0;
-    const int64_t g = a.batch < grid ? a.batch : grid;
-    fpm_cdet_varlen_kernel<<<static_cast<int>(g), varlen_threads(n_max, a.batch),
-                             cdet_smem_bytes(varlen_smem_n(n_max), two, true), s>>>(V);
+    const size_t smem = cdet_smem_bytes(varlen_smem_n(n_max), two, true);
+    const auto ctas = [&](int most) { return static_cast<int>(a.batch < most ? a.batch : most); };
+    if (narrow) {
+        fpm_cdet_varlen_kernel<true><<<ctas(grid), kCdetThreads, smem, s>>>(V);
+        fpm_cdet_varlen_kernel<true><<<ctas(narrow), varlen_narrow(n_max), smem, s>>>(V);
+    } else {
+        fpm_cdet_varlen_kernel<false><<<ctas(grid), threads, smem, s>>>(V);
+    }
     err = static_cast<int>(cudaGetLastError());
     if (err || !fsc) return err;
     // the items of the orders >= fsc_from (the longest-first prefix), one launch

@@ -88,12 +88,15 @@ def test_capture_after_a_first_call_by_lane_groups(apm):
 
 
 # uneven batches without orders above 11, on both sides of every change of the
-# CTA's width, one matrix and two per item, against fixed-order calls
-@pytest.mark.parametrize("hi,batch", [(3, 50), (6, 500), (8, 456), (8, 457), (9, 1199), (9, 1200), (9, 2700),
-                                      (10, 2099), (10, 2100), (11, 3299), (11, 3300)])
-def test_uneven_small_orders(apm, hi, batch):
+# CTA's width, one matrix and two per item, against fixed-order calls; few and many
+# of the largest order where that decides
+@pytest.mark.parametrize("lo,hi,batch", [(1, 3, 50), (1, 6, 500), (1, 8, 456), (1, 8, 457), (1, 9, 456), (1, 9, 457),
+                                         (9, 9, 361), (9, 9, 500), (1, 9, 1100), (1, 9, 1101), (9, 10, 1000),
+                                         (1, 10, 2000), (1, 10, 2001), (11, 11, 457), (11, 11, 1000), (10, 11, 1500),
+                                         (1, 11, 3100), (1, 11, 3101)])
+def test_uneven_small_orders(apm, lo, hi, batch):
     rng = np.random.default_rng(9300 + hi)
-    orders = rng.integers(1, hi + 1, batch).astype(np.int32)
+    orders = rng.integers(lo, hi + 1, batch).astype(np.int32)
     orders[:3] = hi
     off = np.concatenate([[0], np.cumsum(orders.astype(np.int64) ** 2)])[:-1]
     flat = rng.standard_normal((2, int((orders.astype(np.int64) ** 2).sum())))
