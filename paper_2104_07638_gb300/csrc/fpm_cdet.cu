@@ -1372,7 +1372,9 @@ static int launch_cdet_split(const SplitArgs &P, int64_t most, cudaStream_t s) {
 // Whether a launch (or the last, partial round of one) of this many matrices
 // above order 12 goes level by level over many CTAs rather than with one CTA
 // per matrix, whose time depends on the most of them that share an SM only: level
-// by level up to most of two on every SM, and again up to most of three.
+// by level up to most of two on every SM, and again up to most of three. After full
+// rounds the last one's matrices go to the CTAs that finish first, more of them on
+// an SM: level by level up to most of three.
 // Measured, us per call (one CTA per matrix | level by level):
 //   n = 13: 1 matrix 377 | 130, 24 375 | 168, 152 386 | 360, 230 552 | 541, 260 553 | 582, 304 555 | 651,
 //           305 776 | 688, 360 790 | 786, 370 791 | 796, 400 790 | 823
@@ -1381,10 +1383,12 @@ static int launch_cdet_split(const SplitArgs &P, int64_t most, cudaStream_t s) {
 //   n = 15: 1 3129 | 231, 24 3145 | 554, 152 3199 | 2613, 280 4649 | 4564, 304 4651 | 4818, 305 6578 | 4957,
 //           400 6642 | 6279, 430 6649 | 6740
 //   n = 16 (from weights): 1 12451 | 299, 300 14857 | 13042, 455 19657 | 19456
-static bool cdet_split_pays(int n, int64_t batch) {
+//   456 more: n = 13: 152 1285 | 1126, 235 1316 | 1333, 270 1538 | 1386, 340 1539 | 1497, 400 1563 | 1610
+//     n = 14: 152 3746 | 3164, 296 4480 | 3900, 400 4489 | 4447, 430 4493 | 4635;  n = 15: 400 13249 | 12926, 430 13273 | 13398
+static bool cdet_split_pays(int n, int64_t batch, bool after_rounds) {
     if (n >= 16) return true;
-    if (batch <= 2 * 152) return batch <= (n == 13 ? 235 : n == 14 ? 275 : 287);
-    return batch <= (n == 13 ? 365 : n == 14 ? 405 : 422);
+    if (batch <= 2 * 152 && !after_rounds) return batch <= (n == 13 ? 235 : n == 14 ? 275 : 287);
+    return batch <= (n == 13 ? 360 : n == 14 ? 405 : 422);
 }
 
 // CTAs per matrix (log2) of a launch of so many matrices, 0 for one: at most a CTA
@@ -1454,7 +1458,7 @@ int launch_fpm_cdet(const CdetArgs &a, cudaStream_t s) {
         // full rounds of one CTA per matrix, then the rest
         const int full = cdet_grid(a.n, INT64_MAX, a.two_mats != 0, false, &err);
         if (err) return err;
-        const int64_t part = a.batch % full, rest = cdet_split_pays(a.n, part) ? part : 0, b0 = a.batch - rest;
+        const int64_t part = a.batch % full, rest = cdet_split_pays(a.n, part, a.batch > part) ? part : 0, b0 = a.batch - rest;
         if (b0) {
             P.a.batch = b0;
             fpm_cdet_kernel<false><<<grid, kCdetThreads, smem, s>>>(P);

@@ -336,8 +336,8 @@ def test_lane_groups_are_timed_on_the_uneven_kernel(apm, monkeypatch):
 
 
 # orders above 12 level by level or with one CTA per matrix, on both sides of each line
-@pytest.mark.parametrize("n,batch", [(13, 235), (13, 236), (13, 304), (13, 305), (13, 365), (13, 366), (14, 275),
-                                     (14, 276), (14, 406), (15, 288), (15, 305), (13, 456 + 300)])
+@pytest.mark.parametrize("n,batch", [(13, 235), (13, 236), (13, 304), (13, 305), (13, 360), (13, 361), (14, 275),
+                                     (14, 276), (14, 406), (15, 288), (15, 305), (13, 456 + 300), (13, 456 + 400)])
 def test_split_lines(apm, n, batch):
     A = I.hubbard_batch(16, n, seed=70 + n)
     A[3] = 0.0
