@@ -336,9 +336,11 @@ apm_status_t apm_two_type_cdet(const double *M, int n, int64_t batch, double *ab
  *   workspace / workspace_bytes: scratch for the depth-first part of the tree,
  *            needed for n > 8 (apm_workspace_size with APM_OP_KELDYSH says how
  *            much): the per-warp path matrices and, when the batch is too
- *            small to occupy every warp, one slot of n+1 sums per chunk of a
- *            matrix (the matrix's leaves are then split over several warps and
+ *            small to occupy every warp or leaves most of them idle in its last
+ *            round, one slot of n+1 sums per chunk of a matrix (the leaves of a
+ *            matrix of order 10 or more are then split over several warps and
  *            the chunks added in a fixed order, so results stay reproducible).
+ *            Scratch for a batch serves every smaller one.
  */
 apm_status_t apm_keldysh_sum(const double *Mt, int n, int64_t batch, int flags, double *sum,
                              double *partial, uint32_t *status, void *workspace,
@@ -359,9 +361,10 @@ apm_status_t apm_keldysh_sum(const double *Mt, int n, int64_t batch, int flags, 
  *            in either spin, and then that pair's results are NaN.
  *   workspace / workspace_bytes: scratch for the depth-first part (both spins'
  *            path matrices) and the sums of split pairs, needed for n > 7
- *            (apm_workspace_size with APM_OP_KELDYSH2). A small batch's pairs are
- *            split over several warps as apm_keldysh_sum's matrices are: such
- *            results differ from whole pairs' by rounding, and are reproducible.
+ *            (apm_workspace_size with APM_OP_KELDYSH2). Pairs of order 8 or more
+ *            are split over several warps as apm_keldysh_sum's matrices are: such
+ *            results differ from whole pairs' by rounding, and are reproducible
+ *            (the same call gives the same bits; another batch size may not).
  */
 apm_status_t apm_keldysh2_sum(const double *Mu, const double *Md, int n, int64_t batch, int flags, double *sum,
                               double *partial, uint32_t *status, void *workspace, size_t workspace_bytes,
@@ -449,7 +452,10 @@ apm_status_t apm_perm_minors(const double *A, int n, int64_t batch, double *perm
  * matrices of orders 13..16 take their minors, as apm_cdet_connected does, from
  * one warp-per-matrix launch per order before the persistent kernel. Of up to
  * 1024 matrices those of orders 13..15 that launch has not flagged go by blocks on
- * many CTAs, as few matrices of a fixed order do (64 MB of the workspace).
+ * many CTAs, as few matrices of a fixed order do (up to 64 MB of the workspace),
+ * where that is faster: the sort decides from the orders present. For n_max = 9..11
+ * and 457 to 3100 matrices (1100 and 2000 at n_max = 9 and 10) two launches of CTAs
+ * of different widths follow the sort, which names the one that runs.
  * A matrix whose n[b] is outside 1..n_max is skipped with APM_ST_BAD_ORDER.
  * The call allocates nothing and does not synchronise: it can be captured in a
  * CUDA graph once the first (non-captured) call on the device has run.
